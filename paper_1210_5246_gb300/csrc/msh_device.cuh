@@ -46,6 +46,14 @@ template <> __device__ __forceinline__ float frsqrt<float>(float x) { return rsq
 template <typename T> __device__ __forceinline__ T sqrt_ratio(T p, T r) { return sqrt(p / r); }
 template <> __device__ __forceinline__ float sqrt_ratio<float>(float p, float r) { return p * rsqrtf(p * r); }
 
+// Sum and product that are never contracted into a fused multiply-add.  Where an expression
+// leaves the compiler a choice of what to fuse, the Roe-type scheme states it, so that every
+// kernel it is inlined into rounds alike.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // ------------------------------------------------------- paired FP32 arithmetic
 // Componentwise operations on 10-vectors, d_k = a_k s + c_k (v_fma), d_k = a_k s (v_mul),
 // d_k = a_k + b_k (v_add) and d_k = a_k - b_k (v_sub).  In FP32 components (k, k+1) go through the packed f32x2 instructions of sm_100
@@ -395,13 +403,13 @@ __device__ __forceinline__ void reconstruct_upwind(const T (&wm)[NV], const T (&
   }
   const T u = E.u;
   const T s[NV] = {-E.cf, -E.cs, -E.cs, T(0), T(0), T(0), T(0), E.cs, E.cs, E.cf};
-  const T xM = fmax(u + E.cf, T(0)), y0 = fmin(u - E.cf, T(0)), nu2 = T(0.5) * nu;
+  const T xM = fmax(add_rn(u, E.cf), T(0)), y0 = fmin(add_rn(u, -E.cf), T(0)), nu2 = T(0.5) * nu;
   T ch[NV], cl2[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) {
-    const T lam = u + s[k];
-    ch[k] = (T(0.25) - nu2 * (lam > T(0) ? lam : xM)) * m[k];
-    cl2[k] = (T(-0.25) - nu2 * (lam < T(0) ? lam : y0)) * m[k];
+    const T lam = add_rn(u, s[k]);
+    ch[k] = mul_rn(fma(-nu2, lam > T(0) ? lam : xM, T(0.25)), m[k]);
+    cl2[k] = mul_rn(fma(-nu2, lam < T(0) ? lam : y0, T(-0.25)), m[k]);
   }
   T dh[NV], dl[NV];
   E.back(ch, dh);
@@ -410,8 +418,8 @@ __device__ __forceinline__ void reconstruct_upwind(const T (&wm)[NV], const T (&
   for (int k = 0; k < NV; k++) {
     T base = w0[k];
     if constexpr (CTU) base += xget(k);
-    hi[k] = base + dh[k];
-    lo[k] = base + dl[k];
+    hi[k] = add_rn(base, dh[k]);
+    lo[k] = add_rn(base, dl[k]);
   }
   face_state_check(w0, lo, hi);
 }
@@ -538,7 +546,7 @@ __device__ __forceinline__ void roe_flux(const T (&wl)[NV], const T (&wr)[NV], T
   T wm[NV], dw[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) {
-    wm[k] = T(0.5) * (wl[k] + wr[k]);
+    wm[k] = mul_rn(T(0.5), wl[k] + wr[k]);
     dw[k] = wr[k] - wl[k];
   }
   Eig<T> E;
@@ -548,28 +556,27 @@ __device__ __forceinline__ void roe_flux(const T (&wl)[NV], const T (&wr)[NV], T
   const T u = E.u, delta = T(0.1) * E.cf;
   auto fast = [&](T l) {
     const T al = fabs(l);
-    return al < delta ? (l * l + delta * delta) * (T(0.5) * frcp(delta)) : al;
+    return al < delta ? mul_rn(fma(l, l, mul_rn(delta, delta)), mul_rn(T(0.5), frcp(delta))) : al;
   };
-  const T am = fabs(u - E.cs), ap = fabs(u + E.cs), a0 = fabs(u);
-  c[0] *= fast(u - E.cf);
-  c[9] *= fast(u + E.cf);
-  c[1] *= am; c[2] *= am;
-  c[7] *= ap; c[8] *= ap;
-  c[3] *= a0; c[4] *= a0; c[5] *= a0; c[6] *= a0;
+  const T am = fabs(add_rn(u, -E.cs)), ap = fabs(add_rn(u, E.cs)), a0 = fabs(u);
+  const T w[NV] = {fast(add_rn(u, -E.cf)), am, am, a0, a0, a0, a0, ap, ap, fast(add_rn(u, E.cf))};
+#pragma unroll
+  for (int k = 0; k < NV; k++) c[k] = mul_rn(c[k], w[k]);
   T d[NV];
   E.back(c, d);  // primitive dissipation R |Lambda| L dw
   const T r = wm[0], ux = wm[1], uy = wm[2], uz = wm[3];
   T dU[NV];      // through the Jacobian of the conserved map at wm
   dU[0] = d[0];
-  dU[1] = r * d[1] + ux * d[0];
-  dU[2] = r * d[2] + uy * d[0];
-  dU[3] = r * d[3] + uz * d[0];
-  dU[4] = d[4] + d[0] * ux * ux + r * (T(2) * d[1] * ux);
-  dU[5] = d[5] + d[0] * ux * uy + r * (d[1] * uy + ux * d[2]);
-  dU[6] = d[6] + d[0] * ux * uz + r * (d[1] * uz + ux * d[3]);
-  dU[7] = d[7] + d[0] * uy * uy + r * (T(2) * d[2] * uy);
-  dU[8] = d[8] + d[0] * uy * uz + r * (d[2] * uz + uy * d[3]);
-  dU[9] = d[9] + d[0] * uz * uz + r * (T(2) * d[3] * uz);
+  const T vx = mul_rn(d[0], ux), vy = mul_rn(d[0], uy), vz = mul_rn(d[0], uz);
+  dU[1] = fma(r, d[1], vx);
+  dU[2] = fma(r, d[2], vy);
+  dU[3] = fma(r, d[3], vz);
+  dU[4] = fma(r, mul_rn(T(2) * d[1], ux), fma(vx, ux, d[4]));
+  dU[5] = fma(r, fma(d[1], uy, mul_rn(ux, d[2])), fma(vx, uy, d[5]));
+  dU[6] = fma(r, fma(d[1], uz, mul_rn(ux, d[3])), fma(vx, uz, d[6]));
+  dU[7] = fma(r, mul_rn(T(2) * d[2], uy), fma(vy, uy, d[7]));
+  dU[8] = fma(r, fma(d[2], uz, mul_rn(uy, d[3])), fma(vy, uz, d[8]));
+  dU[9] = fma(r, mul_rn(T(2) * d[3], uz), fma(vz, uz, d[9]));
   T Ul[NV], Fl[NV], Ur[NV], Fr[NV];
   phys(wl, Ul, Fl);
   phys(wr, Ur, Fr);

@@ -54,6 +54,11 @@ msh_status fail(msh_status s, const char *fmt, ...) {
   } while (0)
 
 constexpr int kGraphSteps = 16;
+constexpr int kStagedSteps = 64;  // steps of one staged launch at most
+// the staged step's buffers (2 + 2 ndim states) stay below this; larger grids stream
+constexpr size_t kStagedMaxBytes = size_t(2) << 30;
+// FP32 grids of up to this many cells (1D, 2D, 3D) take the staged step
+constexpr size_t kStagedMaxCells32[3] = {size_t(1) << 24, 400000, 600000};
 
 }  // namespace
 
@@ -152,6 +157,89 @@ static cudaError_t launch_characteristic(msh_grid *g, const StepArgs<T> &a, bool
   return launch_step<T>(a, g->ndim, g->rows, retry, g->stream, nblocks_out);
 }
 
+// ------------------------------------------------------------- staged step
+// Layout of a grid's staging allocation (msh_staged.cuh): primitive states of both step
+// parities, face states, ghost face states, counts per block, grid barrier.
+struct StagedLayout {
+  size_t max_pencils, state, ghost, bytes;
+  StagedLayout(const msh_grid *g) {
+    max_pencils = 1;
+    for (int d = 0; d < g->ndim; d++) max_pencils = std::max(max_pencils, g->N / (size_t)g->n[d]);
+    state = 10 * g->N * g->esize;
+    ghost = 2 * (size_t)g->ndim * 10 * max_pencils * g->esize;
+    bytes = (2 + 2 * (size_t)g->ndim) * state + ghost + kStagedMaxBlocks * sizeof(int) + sizeof(GridBar);
+  }
+};
+
+bool staged_wanted(const msh_grid *g) {
+  if (g->ctu || g->tiling_set || g->stg_off) return false;
+  if (StagedLayout(g).bytes > kStagedMaxBytes) return false;
+  if (g->prec == MSH_FP64) return true;
+  return g->N <= kStagedMaxCells32[g->ndim - 1];
+}
+
+// Whether the staged step takes this grid's steps; allocates its buffers at the first use.
+// Where they do not fit, the streaming kernels go on.
+bool use_staged(msh_grid *g) {
+  if (!staged_wanted(g)) return false;
+  if (g->stg_mem) return true;
+  const StagedLayout l(g);
+  if (cudaMalloc(&g->stg_mem, l.bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    g->stg_mem = nullptr;
+    g->stg_off = true;
+    return false;
+  }
+  const size_t tail = kStagedMaxBlocks * sizeof(int) + sizeof(GridBar);
+  if (cudaMemsetAsync(static_cast<char *>(g->stg_mem) + l.bytes - tail, 0, tail, g->stream) != cudaSuccess) {
+    (void)cudaGetLastError();
+    cudaFree(g->stg_mem);
+    g->stg_mem = nullptr;
+    g->stg_off = true;
+    return false;
+  }
+  return true;
+}
+
+template <typename T> StagedArgs<T> make_staged(msh_grid *g, const StepArgs<T> &s, int max_iter) {
+  const StagedLayout l(g);
+  char *p = static_cast<char *>(g->stg_mem);
+  StagedArgs<T> a;
+  a.s = s;
+  a.W[0] = reinterpret_cast<T *>(p);
+  a.W[1] = reinterpret_cast<T *>(p + l.state);
+  a.lo = reinterpret_cast<T *>(p + 2 * l.state);
+  a.hi = reinterpret_cast<T *>(p + (2 + (size_t)g->ndim) * l.state);
+  a.ghost = reinterpret_cast<T *>(p + (2 + 2 * (size_t)g->ndim) * l.state);
+  char *tail = p + (2 + 2 * (size_t)g->ndim) * l.state + l.ghost;
+  a.newly = reinterpret_cast<int *>(tail);
+  a.bar = reinterpret_cast<GridBar *>(tail + kStagedMaxBlocks * sizeof(int));
+  a.max_pencils = l.max_pencils;
+  a.max_iter = max_iter;
+  return a;
+}
+
+template <typename T> cudaError_t dispatch_staged(msh_grid *g, const StagedArgs<T> &a, int *nblk) {
+  switch (g->scheme) {
+    case MSH_SCHEME_KT: return launch_staged<T, 1>(a, g->ndim, g->stream, nblk);
+    case MSH_SCHEME_MUSCL_HANCOCK_ROE: return launch_staged<T, 3>(a, g->ndim, g->stream, nblk);
+    case MSH_SCHEME_MUSCL_HANCOCK_HLLC: return launch_staged<T, 4>(a, g->ndim, g->stream, nblk);
+    default: return launch_staged<T, 0>(a, g->ndim, g->stream, nblk);
+  }
+}
+
+// One staged launch: up to max_iter whole steps, or (phase >= 0) that pass of a phased step.
+cudaError_t run_staged(msh_grid *g, int max_iter, int phase, int *nblk) {
+  if (g->prec == MSH_FP32) {
+    StagedArgs<float> a = make_staged<float>(g, make_args<float>(g), max_iter);
+    a.phase = phase;
+    return dispatch_staged<float>(g, a, nblk);
+  }
+  StagedArgs<double> a = make_staged<double>(g, make_args<double>(g), max_iter);
+  a.phase = phase;
+  return dispatch_staged<double>(g, a, nblk);
+}
+
 msh_status launch_one_step(msh_grid *g, int ev_slot) {
   g->phase_level = -1;  // a whole step closes a phased one that was left open
   int nb = 0;
@@ -162,6 +250,13 @@ msh_status launch_one_step(msh_grid *g, int ev_slot) {
     if (e != cudaSuccess) return fail(MSH_E_CUDA, "self-gravity: %s", cudaGetErrorString(e));
   }
   if (g->profiling && ev_slot >= 0) CUDA_TRY(cudaEventRecord(g->ev[3 * ev_slot], g->stream));
+  if (!(g->test_fault == 1 && g->ndim == 3) && use_staged(g)) {  // the whole step in one launch
+    e = run_staged(g, 1, -1, nullptr);
+    if (e != cudaSuccess) return fail(MSH_E_CUDA, "staged step launch: %s", cudaGetErrorString(e));
+    for (int i = 1; i <= 2 && g->profiling && ev_slot >= 0; i++)
+      CUDA_TRY(cudaEventRecord(g->ev[3 * ev_slot + i], g->stream));
+    return MSH_OK;
+  }
   if (g->scheme == MSH_SCHEME_KT) {
     // the two Runge-Kutta stages of the central scheme, then the finalize (no fallback)
     nb = blocks_for(g, g->rows, g->zchunk);
@@ -203,6 +298,23 @@ msh_status launch_one_step(msh_grid *g, int ev_slot) {
   return MSH_OK;
 }
 
+// n steps in a row (the device control stops them): as few launches as the path allows.
+msh_status launch_steps(msh_grid *g, int64_t n) {
+  if (g->sg_G > 0.0 || (g->test_fault == 1 && g->ndim == 3) || !use_staged(g)) {
+    for (int64_t i = 0; i < n; i++) {
+      msh_status st = launch_one_step(g, -1);
+      if (st) return st;
+    }
+    return MSH_OK;
+  }
+  g->phase_level = -1;
+  for (int64_t i = 0; i < n; i += kStagedSteps) {
+    const cudaError_t e = run_staged(g, (int)std::min<int64_t>(n - i, kStagedSteps), -1, nullptr);
+    if (e != cudaSuccess) return fail(MSH_E_CUDA, "staged step launch: %s", cudaGetErrorString(e));
+  }
+  return MSH_OK;
+}
+
 msh_status build_graph(msh_grid *g) {
   if (g->graph) return MSH_OK;
   const int32_t test_fault = g->test_fault;  // test hooks never enter a graph
@@ -214,6 +326,7 @@ msh_status build_graph(msh_grid *g) {
   } restore{g, test_fault};
   msh_status st = ensure_partials(g, blocks_for(g, g->rows, g->zchunk));
   if (st) return st;
+  (void)use_staged(g);  // its buffers are allocated before the capture
   cudaGraph_t graph;
   CUDA_TRY(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
   for (int i = 0; i < kGraphSteps; i++) {
@@ -449,6 +562,7 @@ msh_status msh_destroy(msh_grid *g) {
   if (g->ctrl_aux) cudaFree(g->ctrl_aux);
   if (g->tag_count) cudaFree(g->tag_count);
   if (g->U1) cudaFree(g->U1);
+  if (g->stg_mem) cudaFree(g->stg_mem);
   free_self_gravity(g);
   free_tape(g);
   free_ensemble(g);
@@ -562,10 +676,8 @@ msh_status msh_run_ensemble(msh_grid *g, int64_t count, const void *const *in, v
     if (e == cudaSuccess) e = launch_finalize(g->ctrl, g->part, kScanBlocks, 1, g->stream);
     if (e == cudaSuccess) e = launch_ensemble_start(g->ctrl, s0, nsteps, g->ens_status + k, g->stream);
     if (e != cudaSuccess) return fail(MSH_E_CUDA, "ensemble start: %s", cudaGetErrorString(e));
-    for (int64_t i = 0; i < nsteps; i++) {
-      st = launch_one_step(g, -1);
-      if (st) return st;
-    }
+    st = launch_steps(g, nsteps);
+    if (st) return st;
     e = launch_ensemble_end(g->ctrl, g->ens_status + k, g->stream);
     if (e != cudaSuccess) return fail(MSH_E_CUDA, "ensemble end: %s", cudaGetErrorString(e));
     CUDA_TRY(cudaMemcpyAsync(slot, g->U[(s0 + nsteps) & 1], bytes, cudaMemcpyDeviceToDevice, g->stream));
@@ -777,13 +889,16 @@ msh_status msh_run(msh_grid *g, double t_end, int64_t max_steps, int64_t *steps,
   if (max_steps < 0 || std::isnan(t_end)) return fail(MSH_E_INVALID_ARG, "bad t_end or max_steps");
   msh_status st = refresh_dt(g);
   if (st) return st;
-  st = g->profiling ? ensure_partials(g, blocks_for(g, g->rows, g->zchunk)) : build_graph(g);
+  // the staged step runs many steps per launch and needs no graph
+  const bool staged = !g->profiling && g->sg_G == 0.0 && use_staged(g);
+  const int batch = staged ? kStagedSteps : kGraphSteps;
+  st = g->profiling || staged ? ensure_partials(g, blocks_for(g, g->rows, g->zchunk)) : build_graph(g);
   if (st) return st;
   const int64_t s0 = g->hctrl->step;
   cudaError_t e = launch_run_start(g->ctrl, t_end, max_steps, INFINITY, g->stream);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "run start: %s", cudaGetErrorString(e));
-  // at most this many batches of kGraphSteps steps can be needed
-  const int64_t need = (max_steps + kGraphSteps - 1) / kGraphSteps;
+  // at most this many batches of steps can be needed
+  const int64_t need = max_steps / batch + (max_steps % batch != 0);
   if (g->profiling) {
     // profiled runs launch the same kernels eagerly, bracketed by events
     for (int64_t it = 0;; it++) {
@@ -799,22 +914,25 @@ msh_status msh_run(msh_grid *g, double t_end, int64_t max_steps, int64_t *steps,
       collect_profile(g, (int)(g->hctrl->step - before));
       if (g->hctrl->done) break;
     }
-  } else if (max_steps < kGraphSteps) {
-    // short runs: exactly max_steps launch pairs, no speculative batch
-    for (int64_t i = 0; i < max_steps; i++) {
-      st = launch_one_step(g, -1);
-      if (st) return st;
-    }
+  } else if (max_steps < batch) {
+    // short runs: exactly max_steps steps, no speculative batch
+    st = launch_steps(g, max_steps);
+    if (st) return st;
     st = read_ctrl(g);
     if (st) return st;
   } else {
-    // Two graph batches in flight: launch batch it, then wait for the completion flag of
+    // Two batches (graphs, or staged launches) in flight: launch batch it, then wait for the completion flag of
     // batch it-1, so the GPU never idles while the host polls.  Batches launched after
     // the run finished return immediately on the device.
     for (int64_t it = 0;; it++) {
       if (it > need + 1) return fail(MSH_E_STATE, "run did not terminate (device control inconsistent)");
       if (it < need) {
-        CUDA_TRY(cudaGraphLaunch(g->graph, g->stream));
+        if (staged) {
+          st = launch_steps(g, batch);
+          if (st) return st;
+        } else {
+          CUDA_TRY(cudaGraphLaunch(g->graph, g->stream));
+        }
         CUDA_TRY(cudaMemcpyAsync(&g->hdone[it & 1], &g->ctrl->done, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                  g->stream));
         CUDA_TRY(cudaEventRecord(g->ev_done[it & 1], g->stream));
@@ -1024,7 +1142,11 @@ msh_status msh_step_begin(msh_grid *g, double dt) {
   if (st) return st;
   cudaError_t e = launch_set_dt(g->ctrl, dt, g->stream);
   int nb = 0;
-  if (e == cudaSuccess) {
+  // every pass of a phased step takes the path of the first
+  g->phase_staged = !(g->test_fault == 1 && g->ndim == 3) && use_staged(g);
+  if (e == cudaSuccess && g->phase_staged) {
+    e = run_staged(g, 1, 0, &nb);
+  } else if (e == cudaSuccess) {
     const int32_t test_fault = g->test_fault;
     g->test_fault = 0;  // a test hook applies to one step
     if (g->prec == MSH_FP32) {
@@ -1052,7 +1174,9 @@ msh_status msh_step_retry(msh_grid *g, int32_t level) {
     return fail(MSH_E_INVALID_ARG, "fallback pass %d after pass %d (passes run in order 1 .. %d)", level,
                 g->phase_level, kFallbackPasses);
   cudaError_t e = launch_force_pass(g->ctrl, level, g->stream);
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && g->phase_staged) {
+    e = run_staged(g, 1, level, nullptr);
+  } else if (e == cudaSuccess) {
     if (g->prec == MSH_FP32) {
       StepArgs<float> a = make_args<float>(g);
       a.level = level;
@@ -1166,9 +1290,10 @@ msh_status msh_set_tiling(msh_grid *g, int32_t rows, int32_t zchunk) {
   if (zchunk > stream_len) zchunk = (int)stream_len;
   msh_status st = ensure_partials(g, blocks_for(g, rows, zchunk));
   if (st) return st;
-  if (rows != g->rows || zchunk != g->zchunk) drop_graph(g);
+  if (rows != g->rows || zchunk != g->zchunk || !g->tiling_set) drop_graph(g);
   g->rows = rows;
   g->zchunk = zchunk;
+  g->tiling_set = true;
   return MSH_OK;
 }
 
@@ -1235,8 +1360,12 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   for (int r : rows_c)
     for (int z : zcs)
       if (!(r == 16 && g->ndim == 3 && g->prec == MSH_FP64)) cands.push_back({r, z});
-  float best = 1e30f;
+  // the staged step is a candidate of its own (0, 0) where the grid's size allows it
+  g->tiling_set = false;
+  if (use_staged(g)) cands.push_back({0, 0});
+  float best = 1e30f, best_tile = 1e30f;
   std::pair<int, int> best_c = {g->rows, g->zchunk};
+  bool best_staged = false;
   const int reps = 3;
   if (st == MSH_OK && (cudaMemcpyAsync(save, g->U[cur], bytes, cudaMemcpyDeviceToDevice, g->stream) != cudaSuccess ||
                        cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) {
@@ -1245,12 +1374,14 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   const bool prof = g->profiling;
   g->profiling = false;
   for (size_t i = 0; st == MSH_OK && i < cands.size(); i++) {
-    st = msh_set_tiling(g, cands[i].first, cands[i].second);
+    const bool staged = cands[i].first == 0;
+    if (staged) g->tiling_set = false;
+    else st = msh_set_tiling(g, cands[i].first, cands[i].second);
     if (st) break;
     cudaError_t e = launch_run_start(g->ctrl, INFINITY, 1 << 30, INFINITY, g->stream);
-    for (int w = 0; st == MSH_OK && w < 1; w++) st = launch_one_step(g, -1);
+    st = launch_steps(g, 1);
     if (st == MSH_OK) e = cudaEventRecord(e0, g->stream);
-    for (int w = 0; st == MSH_OK && w < reps; w++) st = launch_one_step(g, -1);
+    if (st == MSH_OK) st = launch_steps(g, reps);
     if (st == MSH_OK) e = cudaEventRecord(e1, g->stream);
     if (st == MSH_OK && e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -1258,6 +1389,10 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
     if (st == MSH_OK && e != cudaSuccess) st = fail(MSH_E_CUDA, "autotune timing: %s", cudaGetErrorString(e));
     if (st == MSH_OK && ms < best) {
       best = ms;
+      best_staged = staged;
+    }
+    if (st == MSH_OK && !staged && ms < best_tile) {
+      best_tile = ms;
       best_c = cands[i];
     }
     // restore state and control block for the next candidate
@@ -1286,6 +1421,7 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   if (st) return st;
   st = msh_set_tiling(g, best_c.first, best_c.second);
   if (st) return st;
+  if (best_staged) g->tiling_set = false;  // the staged step goes on; the streaming shape is the best of its kind
   if (rows_out) *rows_out = g->rows;
   if (zchunk_out) *zchunk_out = g->zchunk;
   return MSH_OK;

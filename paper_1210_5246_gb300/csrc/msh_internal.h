@@ -74,6 +74,28 @@ template <typename T> struct StepArgs {
   int test_skip = 0;    // test hook: thread block 0 does not issue its bulk copy of plane -2
 };
 
+// Grid barrier of the staged step (msh_staged.cuh), zero between launches.
+struct GridBar {
+  unsigned arrived, left, dead;
+};
+
+// Arguments of a staged launch: the step's, and the staging buffers.
+template <typename T> struct StagedArgs {
+  StepArgs<T> s;
+  T *W[2];             // [NV][N] primitive state by step parity
+  T *lo, *hi;          // [ndim][NV][N] face states (stage B leaves the fluxes in lo)
+  T *ghost;            // [ndim][2 sides][NV][max_pencils] face states of the ghost cells
+  size_t max_pencils;  // cells of the grid's largest side
+  GridBar *bar;
+  int *newly;          // [blocks] cells newly tagged by the last pass
+  int max_iter;        // steps at most in this launch
+  int phase = -1;      // >= 0: only this pass of a phased step
+  T *seg = nullptr;    // recompute: states seg[0 .. max_iter], seg[0] given
+  const double *dts = nullptr;  // their time steps (device)
+  int64_t seg_step = 0;         // step number of seg[0] (fallback tags)
+};
+constexpr int kStagedMaxBlocks = 2048;  // blocks of a staged launch at most (partials, counts)
+
 constexpr int kTile1D = 128;   // threads per block of the 1D step kernel
 constexpr int kTileX = 30;     // interior cells per warp row of the 3D kernel
 constexpr int kStripX = 28;    // updated cells per warp strip of the 2D kernel
@@ -103,6 +125,8 @@ template <typename T, int SCH> cudaError_t launch_step_ctu(const StepArgs<T> &a,
                                                            cudaStream_t s, int *nblocks_out);
 // stage 1 or 2 of the Kurganov-Tadmor scheme (a.U1 must be set)
 template <typename T> cudaError_t launch_step_kt(const StepArgs<T> &a, int ndim, int rows, int stage, cudaStream_t s);
+// the staged step: SCH = 0 (HLL), 1 (central scheme), 3 (Roe-type), 4 (HLLC)
+template <typename T, int SCH> cudaError_t launch_staged(const StagedArgs<T> &a, int ndim, cudaStream_t s, int *nblk);
 template <typename T> int step_blocks(int ndim, int rows, int nx, int ny, int nz, int zchunk);
 template <typename T> size_t step_smem(int ndim, int rows, bool ctu, bool retry);
 // partials of cells [c0, c1) (c1 = 0: all N); maxf: the corner-transport-upwind CFL speed
@@ -190,9 +214,15 @@ struct msh_grid {
   // and the number of partials the step kernel wrote
   int phase_level = -1;
   int phase_nb = 0;
+  bool phase_staged = false;
   int32_t test_fault = 0;  // msh_set_test_fault: applied to the next eager step launch
   unsigned long long *tag_count = nullptr;  // device counter of msh_count_tags
   int rows = 8, zchunk = 32;
+  bool tiling_set = false;  // msh_set_tiling chose the streaming kernels' shape: they step the grid
+  // the staged step (msh_staged.cuh): its buffers in one allocation, made at the first step
+  // that uses it; stg_off: the allocation failed, the streaming kernels step the grid
+  void *stg_mem = nullptr;
+  bool stg_off = false;
   cudaGraphExec_t graph = nullptr;
   // profiling: eager launches with events around every step-kernel launch
   bool profiling = false;

@@ -1,0 +1,708 @@
+// msh_staged.cuh -- the step as grid-wide stages in one persistent cooperative launch.
+//
+// The streaming kernels of msh_step_kernels.cuh keep everything of a cell in registers and
+// shared memory, at the price of halo cells and chunk prologues that are reconstructed
+// again.  Two kinds of grids pay too much for that: FP64 grids, where a double-precision
+// warp instruction occupies its scheduler's pipe for 64 cycles on GB300 however few of its
+// lanes are active (measured: 64.7 cycles for DFMA with 32 lanes or 8), so every repeated
+// lane and every idle scheduler is time lost; and small FP32 grids, which cannot fill 608
+// schedulers with strips or tiles.  Here the same arithmetic runs as stages over flat lists
+// of items, one item per lane, with the intermediate face states in global memory (mostly
+// L2):
+//   P   primitive variables of U^n (at the start of a launch; later steps get them from C)
+//   A   per cell and direction: reconstruction -> lower and upper face state
+//   B   per face: flux, left in place of the face state that only this face reads
+//   C   per cell: flux divergence, update, source, realizability, signal speed
+// Every cell is reconstructed once per direction and every face flux formed once, the items
+// of a stage are dealt to all schedulers evenly, and a grid barrier separates the stages.
+// The last barrier of a step carries the reduction of the CFL speed: every block reduces
+// the blocks' partials and plans the next step itself, so a launch takes many steps without
+// the host, and the a-posteriori fallback passes run inside it only when cells were tagged.
+// The per-cell arithmetic is that of the streaming kernels (same device functions, same
+// order of the flux divergence), and the results agree with theirs bit for bit.
+#pragma once
+#include "msh_step_kernels.cuh"
+
+namespace msh {
+
+constexpr int kStagedThreads = 256;
+constexpr int kStagedWarps = kStagedThreads / 32;
+
+// ------------------------------------------------------------ grid barrier
+// Arrivals only grow within a launch; the last block to leave a launch clears them for the
+// next.  Waits are bounded: a block that waits longer than 2^33 clocks (about four seconds)
+// marks the barrier dead, every block leaves, and the launch reports MSH_E_TIMEOUT.
+__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool grid_barrier(GridBar *b, unsigned nblk, unsigned &epoch, int *s_dead) {
+  __syncthreads();
+  if (nblk == 1) return true;
+  epoch += nblk;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&b->arrived, 1u);
+    if (ld_acquire_u32(&b->arrived) < epoch) {
+      const long long t0 = clock64();
+      while (ld_acquire_u32(&b->arrived) < epoch) {
+        if (ld_acquire_u32(&b->dead) != 0u) break;
+        if (clock64() - t0 > (1ll << 33)) {
+          atomicExch(&b->dead, 1u);
+          break;
+        }
+      }
+    }
+    *s_dead = (int)ld_acquire_u32(&b->dead);
+    __threadfence();
+  }
+  __syncthreads();
+  return *s_dead == 0;
+}
+__device__ __forceinline__ void grid_leave(GridBar *b, unsigned nblk) {
+  if (nblk == 1 || threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(&b->left, 1u) == nblk - 1) {  // every block has passed its last barrier
+    b->arrived = 0u;
+    b->left = 0u;
+    b->dead = 0u;
+  }
+}
+
+// ------------------------------------------------------------------ helpers
+template <int D> __device__ __forceinline__ int axis_n(int nx, int ny, int nz) { return D == 0 ? nx : D == 1 ? ny : nz; }
+
+// Cell index and mirror flag of position j along D (j may be up to two cells outside) on the
+// pencil through cell c, whose own coordinate along D is i.
+template <typename T, int D>
+__device__ __forceinline__ int mapped_cell(const StepArgs<T> &s, int c, int i, int j, bool &mir) {
+  const int n = axis_n<D>(s.nx, s.ny, s.nz), st = D == 0 ? 1 : D == 1 ? s.nx : s.nx * s.ny;
+  return c + (map_index(j, n, s.bc[2 * D], s.bc[2 * D + 1], mir) - i) * st;
+}
+
+// Primitive state of cell c in the local frame of D (mirrored: u_n and P_nt negated).
+template <typename T, int D>
+__device__ __forceinline__ void load_frame(const T *W, size_t N, int c, bool mir, T (&w)[NV]) {
+#pragma unroll
+  for (int k = 0; k < NV; k++) w[k] = W[(size_t)Frame<D>::g(k) * N + c];
+  if (mir) {
+    w[1] = -w[1];
+    w[5] = -w[5];
+    w[6] = -w[6];
+  }
+}
+
+template <typename T> __device__ __forceinline__ bool cell_tag(const StepArgs<T> &s, int c, int32_t tag, int level) {
+  return tagged(s.flags[c], tag, level);
+}
+
+// Stage A of one cell (position j along D on the pencil of cell c; j = -1 and j = n are the
+// ghost cells of a side that is not periodic, whose face state the boundary face needs).
+template <typename T, int SCH, int D>
+__device__ __forceinline__ void stage_a_item(const StagedArgs<T> &a, const T *W, size_t N, T nu, int c, int i, int j,
+                                             int32_t tag, int level, T *lo_out, T *hi_out, size_t stride) {
+  const StepArgs<T> &s = a.s;
+  bool mm, m0, mp;
+  const int cm = mapped_cell<T, D>(s, c, i, j - 1, mm);
+  const int c0 = mapped_cell<T, D>(s, c, i, j, m0);
+  const int cp = mapped_cell<T, D>(s, c, i, j + 1, mp);
+  T wm[NV], w0[NV], wp[NV], lo[NV], hi[NV];
+  load_frame<T, D>(W, N, cm, mm, wm);
+  load_frame<T, D>(W, N, c0, m0, w0);
+  load_frame<T, D>(W, N, cp, mp, wp);
+  recon<SCH>(wm, w0, wp, nu, lo, hi);
+  if (kCharacteristic<SCH> && level > 0)
+    first_order_faces(cell_tag(s, cm, tag, level), cell_tag(s, c0, tag, level), cell_tag(s, cp, tag, level), w0, lo, hi);
+  if (lo_out != nullptr) {
+#pragma unroll
+    for (int k = 0; k < NV; k++) lo_out[k * stride] = lo[k];
+  }
+  if (hi_out != nullptr) {
+#pragma unroll
+    for (int k = 0; k < NV; k++) hi_out[k * stride] = hi[k];
+  }
+}
+
+// The pencil of cell c along D, and the first cell of pencil p.
+template <int D> __device__ __forceinline__ int pencil_of(int c, int nx, int ny) {
+  if (D == 0) return c / nx;
+  if (D == 1) {
+    const int z = c / (nx * ny);
+    return z * nx + (c - z * nx * ny) % nx;
+  }
+  return c % (nx * ny);
+}
+template <int D> __device__ __forceinline__ int pencil_cell(int p, int nx, int ny) {
+  if (D == 0) return p * nx;
+  if (D == 1) {
+    const int z = p / nx;
+    return z * nx * ny + (p - z * nx);
+  }
+  return p;
+}
+template <int D> __device__ __forceinline__ int coord(int c, int nx, int ny) {
+  return D == 0 ? c % nx : D == 1 ? (c / nx) % ny : c / (nx * ny);
+}
+
+// Face states of direction D are [NV][N] at a.lo / a.hi + D NV N; ghost states of its lower
+// and upper side [NV][pencils] at a.ghost + (2 D + side) NV max_pencils.
+template <typename T, int SCH, int D>
+__device__ __forceinline__ void stage_a(const StagedArgs<T> &a, const T *W, size_t N, T nu, int item, bool ghost,
+                                        int32_t tag, int level) {
+  const StepArgs<T> &s = a.s;
+  const int nx = s.nx, ny = s.ny;
+  if (!ghost) {
+    if (item >= (int)N) return;
+    T *lo = a.lo + (size_t)D * NV * N + item, *hi = a.hi + (size_t)D * NV * N + item;
+    const int i = coord<D>(item, nx, ny);
+    stage_a_item<T, SCH, D>(a, W, N, nu, item, i, i, tag, level, lo, hi, N);
+  } else {  // the two ghost cells of the pencils along a side that is not periodic
+    const int n = axis_n<D>(s.nx, s.ny, s.nz), np = (int)(N / n);
+    if (item >= 2 * np) return;
+    const int side = item >= np ? 1 : 0, p = item - side * np;
+    T *g = a.ghost + (size_t)(2 * D + side) * NV * a.max_pencils + p;
+    stage_a_item<T, SCH, D>(a, W, N, nu, pencil_cell<D>(p, nx, ny), 0, side ? n : -1, tag, level, side ? g : nullptr,
+                            side ? nullptr : g, a.max_pencils);
+  }
+}
+
+// Stage B: flux through the lower face of cell `item` along D, stored over its lower face
+// state; with `upper` the flux through the upper boundary face of pencil `item` (sides that
+// are not periodic), stored over the upper face state of the pencil's last cell.
+template <typename T, int SCH, int D>
+__device__ __forceinline__ void stage_b(const StagedArgs<T> &a, size_t N, int item, bool upper, int32_t tag,
+                                        int level) {
+  const StepArgs<T> &s = a.s;
+  const int nx = s.nx, ny = s.ny, n = axis_n<D>(s.nx, s.ny, s.nz), st = D == 0 ? 1 : D == 1 ? nx : nx * ny;
+  T *lo = a.lo + (size_t)D * NV * N, *hi = a.hi + (size_t)D * NV * N;
+  const T *pl, *pr;
+  size_t sl = N, sr = N;
+  T *out;
+  int c;
+  bool first = false;
+  if (!upper) {
+    if (item >= (int)N) return;
+    c = item;
+    const int i = coord<D>(c, nx, ny);
+    pr = lo + c;
+    out = lo + c;
+    if (i > 0 || s.bc[2 * D] == BC_PERIODIC) {
+      pl = hi + (i > 0 ? c - st : c + (n - 1) * st);
+    } else {
+      pl = a.ghost + (size_t)(2 * D) * NV * a.max_pencils + pencil_of<D>(c, nx, ny);
+      sl = a.max_pencils;
+    }
+    if ((SCH == 3 || SCH == 4) && level > 0) {
+      bool m;
+      first = cell_tag(s, mapped_cell<T, D>(s, c, i, i - 1, m), tag, level) || cell_tag(s, c, tag, level);
+    }
+  } else {
+    if (item >= (int)(N / n)) return;
+    c = pencil_cell<D>(item, nx, ny) + (n - 1) * st;
+    pl = hi + c;
+    out = hi + c;
+    pr = a.ghost + (size_t)(2 * D + 1) * NV * a.max_pencils + item;
+    sr = a.max_pencils;
+    if ((SCH == 3 || SCH == 4) && level > 0) first = cell_tag(s, c, tag, level);  // the ghost cell is its image
+  }
+  T wl[NV], wr[NV], F[NV];
+#pragma unroll
+  for (int k = 0; k < NV; k++) {
+    wl[k] = pl[k * sl];
+    wr[k] = pr[k * sr];
+  }
+  if constexpr (SCH == 3 || SCH == 4) {
+    if (first) hll(wl, wr, F);
+    else face_flux<SCH>(wl, wr, F);
+  } else {
+    face_flux<SCH>(wl, wr, F);
+  }
+#pragma unroll
+  for (int k = 0; k < NV; k++) out[k * N] = F[k];
+}
+
+// Lower (fl) and upper (fu) face flux of cell c along D, local frame.
+template <typename T, int D>
+__device__ __forceinline__ void load_fluxes(const StagedArgs<T> &a, size_t N, int c, T (&fl)[NV], T (&fu)[NV]) {
+  const StepArgs<T> &s = a.s;
+  const int nx = s.nx, ny = s.ny, n = axis_n<D>(s.nx, s.ny, s.nz), st = D == 0 ? 1 : D == 1 ? nx : nx * ny;
+  const T *lo = a.lo + (size_t)D * NV * N;
+  const int i = coord<D>(c, nx, ny);
+  const T *pu = i + 1 < n ? lo + c + st
+                          : (s.bc[2 * D + 1] == BC_PERIODIC ? lo + c - (n - 1) * st : a.hi + (size_t)D * NV * N + c);
+#pragma unroll
+  for (int k = 0; k < NV; k++) {
+    fl[k] = lo[k * N + c];
+    fu[k] = pu[k * N];
+  }
+}
+
+// Flux divergence of cell c in the global component order, the faces added in the order of
+// the streaming kernels (1D: x; 2D: lower y, x, upper y; 3D: lower z, x, lower y, upper z,
+// upper y), so that the sums round alike.
+template <typename T, int NDIM>
+__device__ __forceinline__ void divergence(const StagedArgs<T> &a, size_t N, int c, T idx, T idy, T idz, T (&acc)[NV]) {
+  T fl[NV], fu[NV], t[NV], u[NV];
+  if constexpr (NDIM == 1) {
+    load_fluxes<T, 0>(a, N, c, fl, fu);
+#pragma unroll
+    for (int k = 0; k < NV; k++) acc[k] = (fl[k] - fu[k]) * idx;
+  } else if constexpr (NDIM == 2) {
+    load_fluxes<T, 1>(a, N, c, fl, fu);
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+      t[Frame<1>::g(k)] = fl[k];
+      u[Frame<1>::g(k)] = fu[k];
+    }
+    v_mul(acc, t, idy);
+    load_fluxes<T, 0>(a, N, c, fl, fu);
+    v_sub(fl, fl, fu);
+    v_fma(acc, fl, idx, acc);
+    v_fma(acc, u, -idy, acc);
+  } else {
+    load_fluxes<T, 2>(a, N, c, fl, fu);
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+      t[Frame<2>::g(k)] = fl[k];
+      u[Frame<2>::g(k)] = fu[k];
+    }
+    v_mul(acc, t, idz);
+    load_fluxes<T, 0>(a, N, c, fl, fu);
+    v_sub(fl, fl, fu);
+    v_fma(acc, fl, idx, acc);
+    load_fluxes<T, 1>(a, N, c, fl, fu);
+#pragma unroll
+    for (int k = 0; k < NV; k++) t[Frame<1>::g(k)] = fl[k];
+    v_fma(acc, t, idy, acc);
+    v_fma(acc, u, -idz, acc);
+#pragma unroll
+    for (int k = 0; k < NV; k++) acc[Frame<1>::g(k)] -= fu[k] * idy;
+  }
+}
+
+// Sums of ten values over a warp with 12 additions per lane instead of 50: each step halves
+// the components a lane keeps.  Lane 2 m (even) ends with one component's sum; returns its
+// index in `comp` (or -1).
+__device__ __forceinline__ double warp_sum10(double (&v)[NV], int &comp) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+  double p[6];
+#pragma unroll
+  for (int k = 0; k < 5; k++) p[k] = (b4 ? v[k + 5] : v[k]) + __shfl_xor_sync(FULL, b4 ? v[k] : v[k + 5], 16);
+  p[5] = 0.0;
+  double q[4];
+#pragma unroll
+  for (int k = 0; k < 3; k++) q[k] = (b3 ? p[k + 3] : p[k]) + __shfl_xor_sync(FULL, b3 ? p[k] : p[k + 3], 8);
+  q[3] = 0.0;
+  double r[2];
+#pragma unroll
+  for (int k = 0; k < 2; k++) r[k] = (b2 ? q[k + 2] : q[k]) + __shfl_xor_sync(FULL, b2 ? q[k] : q[k + 2], 4);
+  double x = (b1 ? r[1] : r[0]) + __shfl_xor_sync(FULL, b1 ? r[0] : r[1], 2);
+  x += __shfl_xor_sync(FULL, x, 1);
+  const int in3 = (b2 ? 2 : 0) + (b1 ? 1 : 0), in5 = (b3 ? 3 : 0) + in3;
+  comp = (in3 < 3 && in5 < 5) ? (b4 ? 5 : 0) + in5 : -1;
+  return x;
+}
+
+// The time control of a launch, the same in every block.
+struct StagedTime {
+  double t, t_next, dt, dt_last, dt_cfl;
+  int64_t step;
+  int64_t first_bad;
+  int done, status, realizable, last_tagged, stop, newly, any_tagged;
+};
+
+// ------------------------------------------------------------------- kernel
+// SCH 0, 3, 4: the characteristic step with its fallback; 1: both stages of the central
+// scheme.  a.phase >= 0: only pass a.phase of a phased step (partials for the finalize
+// kernel, no time control).  a.seg: recompute a.max_iter states seg[1..] from seg[0] with
+// the given time steps.
+template <typename T, int NDIM, int SCH>
+__global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged_kernel(const StagedArgs<T> a) {
+  constexpr bool kKt = SCH == 1;
+  __shared__ StagedTime st;
+  __shared__ int s_dead, s_nbad;
+  __shared__ double s_red[kStagedWarps][NV];
+  __shared__ double s_max[kStagedWarps];
+  __shared__ long long s_bad[kStagedWarps];
+  const StepArgs<T> &s = a.s;
+  Ctrl *ctrl = s.ctrl;
+  if (a.seg == nullptr && ctrl->done) return;  // the same in every block: nothing writes it before the first barrier
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned nblk = gridDim.x, blk = blockIdx.x;
+  const size_t N = (size_t)s.nx * s.ny * s.nz;
+  const int ngrp = (int)((N + 31) / 32);
+  unsigned epoch = 0;
+  if (tid == 0) {
+    st.t = ctrl->t;
+    st.t_next = ctrl->t_next;
+    st.dt = ctrl->dt;
+    st.dt_last = ctrl->dt_last;
+    st.dt_cfl = ctrl->dt_cfl;
+    st.step = a.seg != nullptr ? a.seg_step : ctrl->step;
+    st.done = 0;
+    st.status = ctrl->status;
+    st.realizable = ctrl->realizable;
+    st.first_bad = ctrl->first_bad;
+    st.last_tagged = ctrl->last_tagged;
+    s_dead = 0;
+    s_nbad = 0;
+    if (a.seg != nullptr) st.dt = a.dts[0];
+  }
+  __syncthreads();
+  const double ddx0 = s.dx[0], ddx1 = s.dx[1], ddx2 = s.dx[2];
+  const T idx = (T)(1.0 / ddx0), idy = (T)(1.0 / ddx1), idz = (T)(1.0 / ddx2);
+  // groups of 32 items are dealt out warp by warp, blocks first, so that a short list
+  // spreads over the SMs and over the schedulers of each
+  const int w0 = warp * (int)nblk + (int)blk, wstep = kStagedWarps * (int)nblk;
+  int gh[NDIM], up[NDIM];  // groups of ghost cells and of upper boundary faces per direction
+  int ngh = 0, nup = 0;
+#pragma unroll
+  for (int d = 0; d < NDIM; d++) {
+    const int n = d == 0 ? s.nx : d == 1 ? s.ny : s.nz;
+    const int np = (int)(N / n);
+    gh[d] = s.bc[2 * d] == BC_PERIODIC ? 0 : (2 * np + 31) / 32;
+    up[d] = s.bc[2 * d] == BC_PERIODIC ? 0 : (np + 31) / 32;
+    ngh += gh[d];
+    nup += up[d];
+  }
+  bool alive = true;
+  T smax = T(0);
+  long long bad = LLONG_MAX;
+
+  auto stages_ab = [&](const T *W, double dt, int32_t tag, int level) {
+    const T nux = (T)(0.5 * dt / ddx0), nuy = (T)(0.5 * dt / ddx1), nuz = (T)(0.5 * dt / ddx2);
+    for (int g = w0; g < NDIM * ngrp + ngh; g += wstep) {
+      bool ghost = g >= NDIM * ngrp;
+      int d, it;
+      if (!ghost) {
+        d = g / ngrp;
+        it = g - d * ngrp;
+      } else {
+        it = g - NDIM * ngrp;
+        d = 0;
+#pragma unroll
+        for (int e = 0; e + 1 < NDIM; e++)
+          if (d == e && it >= gh[e]) {
+            it -= gh[e];
+            d = e + 1;
+          }
+      }
+      const int item = it * 32 + lane;
+      if (d == 0) stage_a<T, SCH, 0>(a, W, N, nux, item, ghost, tag, level);
+      else if (NDIM > 1 && d == 1) stage_a<T, SCH, 1>(a, W, N, nuy, item, ghost, tag, level);
+      else if (NDIM > 2) stage_a<T, SCH, 2>(a, W, N, nuz, item, ghost, tag, level);
+    }
+    alive = alive && grid_barrier(a.bar, nblk, epoch, &s_dead);
+    if (!alive) return;
+    for (int g = w0; g < NDIM * ngrp + nup; g += wstep) {
+      bool upper = g >= NDIM * ngrp;
+      int d, it;
+      if (!upper) {
+        d = g / ngrp;
+        it = g - d * ngrp;
+      } else {
+        it = g - NDIM * ngrp;
+        d = 0;
+#pragma unroll
+        for (int e = 0; e + 1 < NDIM; e++)
+          if (d == e && it >= up[e]) {
+            it -= up[e];
+            d = e + 1;
+          }
+      }
+      const int item = it * 32 + lane;
+      if (d == 0) stage_b<T, SCH, 0>(a, N, item, upper, tag, level);
+      else if (NDIM > 1 && d == 1) stage_b<T, SCH, 1>(a, N, item, upper, tag, level);
+      else if (NDIM > 2) stage_b<T, SCH, 2>(a, N, item, upper, tag, level);
+    }
+    alive = alive && grid_barrier(a.bar, nblk, epoch, &s_dead);
+  };
+
+  // stage C; CS: the scheme finish_cell sees (0 for the characteristic step, 1 and 2 for the
+  // stages of the central scheme)
+  auto stage_c = [&](auto csc, const T *src, const T *un0, T *dst, T *Wout, double ddt, int32_t tag, int level, T *ck) {
+    constexpr int CS = decltype(csc)::value;
+    const T dt = (T)ddt;
+    Acc<T> none;
+    for (int g = w0; g < ngrp; g += wstep) {
+      const int c = g * 32 + lane;
+      if (c >= (int)N) continue;
+      T acc[NV];
+      divergence<T, NDIM>(a, N, c, idx, idy, idz, acc);
+      finish_cell<T, NDIM, CS, false, false, true>(s, src + c, N, un0 + c, dst, N, (size_t)c, acc, dt, idx, idy, idz, none,
+                                                   smax, bad, tag, ck, level, Wout, &s_nbad);
+    }
+  };
+
+  // the block's CFL speed, first non-realizable cell and newly tagged cells to its partial,
+  // then (after the barrier) the grid's in every block
+  auto write_part = [&]() {
+    smax = warp_max_nonneg(smax);
+    if (__any_sync(FULL, bad != LLONG_MAX)) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) bad = min(bad, __shfl_xor_sync(FULL, bad, o));
+    }
+    if (lane == 0) {
+      s_max[warp] = (double)smax;
+      s_bad[warp] = bad;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double m = s_max[0];
+      long long b = s_bad[0];
+      for (int w = 1; w < kStagedWarps; w++) {
+        m = max_nonneg(m, s_max[w]);
+        b = min(b, s_bad[w]);
+      }
+      Partial *p = s.part + blk;
+      p->smax = m;
+      p->bad = b;
+      a.newly[blk] = s_nbad;
+      s_nbad = 0;
+    }
+    smax = T(0);
+    bad = LLONG_MAX;
+  };
+  auto reduce_parts = [&](double &m, long long &b, int &nb) {  // warp 0
+    m = 0.0;
+    b = LLONG_MAX;
+    nb = 0;
+    for (unsigned i = lane; i < nblk; i += 32) {
+      m = max_nonneg(m, __ldcg(&s.part[i].smax));
+      b = min(b, __ldcg(&s.part[i].bad));
+      nb += __ldcg(&a.newly[i]);
+    }
+    m = warp_max_nonneg(m);
+    nb = __reduce_add_sync(FULL, nb);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) b = min(b, __shfl_xor_sync(FULL, b, o));
+  };
+
+  {  // P
+    const T *U = a.seg != nullptr ? a.seg : s.U[st.step & 1];
+    T *W = a.W[st.step & 1];
+    for (int g = w0; g < ngrp; g += wstep) {
+      const int c = g * 32 + lane;
+      if (c >= (int)N) continue;
+      T u[NV], w[NV];
+#pragma unroll
+      for (int k = 0; k < NV; k++) u[k] = U[k * N + c];
+      cons_to_prim(u, w);
+#pragma unroll
+      for (int k = 0; k < NV; k++) W[k * N + c] = w[k];
+    }
+    alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
+  }
+
+  int taken = 0;
+  while (alive) {
+    const int64_t step = st.step;
+    const double dt = st.dt;
+    const int32_t tag = (int32_t)(step & 0x0fffffff) + 1;
+    const T *U0 = a.seg != nullptr ? a.seg + (size_t)taken * NV * N : s.U[step & 1];
+    T *Ud = a.seg != nullptr ? a.seg + (size_t)(taken + 1) * NV * N : s.U[(step + 1) & 1];
+    const T *W0 = a.W[step & 1];
+    T *Wn = a.W[(step + 1) & 1];
+    T *const ck = (kKt || a.seg != nullptr) ? nullptr : tape_slot(s, step, N);
+    if constexpr (kKt) {
+      stages_ab(W0, dt, tag, 0);
+      if (!alive) break;
+      // the first stage's primitive state goes to the next step's buffer, which the second
+      // stage replaces once every face state has been formed from it
+      stage_c(std::integral_constant<int, 1>{}, U0, U0, s.U1, Wn, dt, tag, 0, (T *)nullptr);
+      alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
+      if (!alive) break;
+      stages_ab(Wn, dt, tag, 0);
+      if (!alive) break;
+      stage_c(std::integral_constant<int, 2>{}, s.U1, U0, Ud, Wn, dt, tag, 0, (T *)nullptr);
+      write_part();
+    } else {
+      const int level = a.phase >= 0 ? a.phase : 0;
+      stages_ab(W0, dt, tag, level);
+      if (!alive) break;
+      stage_c(std::integral_constant<int, 0>{}, U0, U0, Ud, Wn, dt, tag, level, level == 0 ? ck : nullptr);
+      write_part();
+      if (a.phase >= 0) break;
+    }
+    alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
+    if (!alive) break;
+    double m;
+    long long b;
+    int nb;
+    if (warp == 0) {
+      reduce_parts(m, b, nb);
+      if (lane == 0) {
+        st.newly = nb;
+        st.any_tagged = nb;
+      }
+    }
+    __syncthreads();
+    // a-posteriori fallback: passes with first-order faces at the tagged cells, while the
+    // pass before tagged new ones
+    if (!kKt) {
+      for (int level = 1; level <= kFallbackPasses && st.newly > 0; level++) {
+        stages_ab(W0, dt, tag, level);
+        if (!alive) break;
+        stage_c(std::integral_constant<int, 0>{}, U0, U0, Ud, Wn, dt, tag, level, (T *)nullptr);
+        write_part();
+        alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
+        if (!alive) break;
+        if (warp == 0) {
+          reduce_parts(m, b, nb);
+          if (lane == 0) st.newly = nb;
+        }
+        __syncthreads();
+      }
+      if (!alive) break;
+    }
+    taken++;
+    if (tid == 0) {  // plan the next step, as the finalize kernel does
+      if (a.seg != nullptr) {
+        st.stop = taken >= a.max_iter;
+        if (!st.stop) st.dt = a.dts[taken];
+        st.step = step + 1;
+        if (blk == 0 && st.any_tagged > 0)
+          for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
+      } else {
+        st.last_tagged = st.any_tagged;
+        st.realizable = b == LLONG_MAX;
+        st.first_bad = b == LLONG_MAX ? -1 : b;
+        st.dt_cfl = ctrl->cfl / m;
+        if (blk == 0) {
+          const int64_t ti = step - ctrl->tape_base;
+          if (ctrl->tape_dt != nullptr && ti >= 0 && ti < ctrl->tape_len) {
+            ctrl->tape_dt[ti] = dt;
+            ctrl->tape_had[ti] = st.any_tagged > 0;
+          }
+          const int64_t hi_ = step - ctrl->hist_base;
+          if (ctrl->hist != nullptr && hi_ >= 0 && hi_ < ctrl->hist_cap) ctrl->hist[hi_] = dt;
+          if (st.any_tagged > 0)
+            for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
+        }
+        st.dt_last = dt;
+        st.t = st.t_next;
+        st.step = step + 1;
+        if (!st.realizable) {
+          st.status = 4;  // MSH_E_REALIZABILITY
+          st.done = 1;
+        } else if (st.t >= ctrl->t_end || st.step >= ctrl->max_step) {
+          st.done = 1;
+        } else {
+          double nd = st.dt_cfl;
+          if (nd > ctrl->dt_max) nd = ctrl->dt_max;
+          double tn = st.t + nd;
+          if (tn >= ctrl->t_end) {
+            nd = ctrl->t_end - st.t;
+            tn = ctrl->t_end;
+          }
+          st.dt = nd;
+          st.t_next = tn;
+        }
+        st.stop = st.done || taken >= a.max_iter;
+      }
+    }
+    __syncthreads();
+    if (st.stop) break;
+  }
+  if (!alive) {  // a barrier gave up: the result is void
+    if (tid == 0 && a.seg == nullptr) {
+      ctrl->status = 5;  // MSH_E_TIMEOUT
+      ctrl->done = 1;
+    }
+    grid_leave(a.bar, nblk);
+    return;
+  }
+  if (a.seg == nullptr) {
+    // FP64 totals of the state the launch leaves (only the last step's are observable)
+    const T *U = s.U[(a.phase >= 0 ? st.step + 1 : st.step) & 1];
+    double d[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) d[k] = 0.0;
+    for (int g = w0; g < ngrp; g += wstep) {
+      const int c = g * 32 + lane;
+      if (c >= (int)N) continue;
+#pragma unroll
+      for (int k = 0; k < NV; k++) d[k] += (double)U[k * N + c];
+    }
+    int comp;
+    const double x = warp_sum10(d, comp);
+    if (comp >= 0 && (lane & 1) == 0) s_red[warp][comp] = x;
+    __syncthreads();
+    if (tid < NV) {
+      double sum = 0.0;
+      for (int w = 0; w < kStagedWarps; w++) sum += s_red[w][tid];
+      s.part[blk].diag[tid] = sum;
+    }
+    if (a.phase < 0) {
+      __syncthreads();
+      alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
+      if (blk == 0) {
+        if (lane < NV) {
+          double sum = 0.0;
+          for (unsigned i = warp; i < nblk; i += kStagedWarps) sum += __ldcg(&s.part[i].diag[lane]);
+          s_red[warp][lane] = sum;
+        }
+        __syncthreads();
+        if (tid < NV) {
+          double sum = 0.0;
+          for (int w = 0; w < kStagedWarps; w++) sum += s_red[w][tid];
+          ctrl->totals[tid] = sum;
+        }
+        if (tid == 0) {
+          ctrl->t = st.t;
+          ctrl->t_next = st.t_next;
+          ctrl->dt = st.dt;
+          ctrl->dt_last = st.dt_last;
+          ctrl->dt_cfl = st.dt_cfl;
+          ctrl->step = st.step;
+          ctrl->realizable = st.realizable;
+          ctrl->first_bad = st.first_bad;
+          ctrl->last_tagged = st.last_tagged;
+          ctrl->force = 0;
+          ctrl->status = alive ? st.status : 5;
+          ctrl->done = alive ? st.done : 1;
+        }
+      }
+    }
+  }
+  grid_leave(a.bar, nblk);
+}
+
+// ----------------------------------------------------------------- launcher
+template <typename T, int NDIM, int SCH> cudaError_t launch_staged_nd(const StagedArgs<T> &a, cudaStream_t s, int *nblk) {
+  static std::atomic<int> occ{0};
+  int per_sm = occ.load(std::memory_order_relaxed);
+  if (per_sm == 0) {
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, staged_kernel<T, NDIM, SCH>, kStagedThreads, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    occ.store(per_sm, std::memory_order_relaxed);
+  }
+  // as many blocks as the SMs hold, but no more than give every scheduler a group of 32 items
+  // of stage A (four groups per block)
+  const size_t N = (size_t)a.s.nx * a.s.ny * a.s.nz;
+  const long long groups = (long long)NDIM * (long long)((N + 31) / 32);
+  const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)device_sms() * per_sm, (groups + 3) / 4));
+  if (nblk != nullptr) *nblk = blocks;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kStagedThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, staged_kernel<T, NDIM, SCH>, a);
+}
+
+template <typename T, int SCH> cudaError_t launch_staged(const StagedArgs<T> &a, int ndim, cudaStream_t s, int *nblk) {
+  if (ndim == 1) return launch_staged_nd<T, 1, SCH>(a, s, nblk);
+  if (ndim == 2) return launch_staged_nd<T, 2, SCH>(a, s, nblk);
+  return launch_staged_nd<T, 3, SCH>(a, s, nblk);
+}
+
+}  // namespace msh

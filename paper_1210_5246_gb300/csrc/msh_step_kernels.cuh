@@ -93,6 +93,24 @@ __device__ __forceinline__ T speed_sum(const T (&W)[NV], T idx, T idy, T idz) {
   return s;
 }
 
+// max of a running maximum m >= 0 and a signal speed s >= 0; a NaN s leaves m (fmax's rule).
+// FP64: on the bit patterns, which order like non-negative numbers -- integer instructions
+// instead of the double-precision pipe (64 cycles per warp instruction).
+__device__ __forceinline__ float max_nonneg(float m, float s) { return fmaxf(m, s); }
+__device__ __forceinline__ double max_nonneg(double m, double s) {
+  const long long a = __double_as_longlong(m), b = __double_as_longlong(s);
+  return (b > a && b <= 0x7ff0000000000000ll) ? s : m;
+}
+// the same over a warp, in every lane
+__device__ __forceinline__ float warp_max_nonneg(float m) {
+  return __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(m)));
+}
+__device__ __forceinline__ double warp_max_nonneg(double m) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max_nonneg(m, __shfl_xor_sync(FULL, m, o));
+  return m;
+}
+
 // Checkpoint slot of the adjoint tape that step `step` stores U^step into, or nullptr.
 template <typename T> __device__ __forceinline__ T *tape_slot(const StepArgs<T> &a, int64_t step, size_t N) {
   if (a.ck == nullptr) return nullptr;
@@ -108,11 +126,16 @@ template <typename T> __device__ __forceinline__ T *tape_slot(const StepArgs<T> 
 // SCH 0: U^{n+1} = U^n + dt L (MUSCL-Hancock); SCH 1: U1 = U^n + dt L(U^n) (the first
 // Runge-Kutta stage, stored without sources or partials); SCH 2: U^{n+1} =
 // (U^n + U1 + dt L(U1)) / 2 with src = U1 and un0 = U^n of the cell (fields N apart).
-template <typename T, int NDIM, int SCH, bool RETRY, bool CTU = false>
+// STAGED (msh_staged.cuh): pass `level` comes as an argument, the primitive state goes to
+// Wout too, newly tagged cells also count in *newly, and the totals are left out (formed once
+// at the end of the launch).
+template <typename T, int NDIM, int SCH, bool RETRY, bool CTU = false, bool STAGED = false>
 __device__ __forceinline__ void finish_cell(const StepArgs<T> &a, const T *src, size_t stride, const T *un0,
                                             T *__restrict__ Ud, size_t N, size_t c,
                                             const T (&acc)[NV], T dt, T idx, T idy, T idz, Acc<T> &diag,
-                                            T &smax, long long &bad, int32_t tag, T *__restrict__ ck) {
+                                            T &smax, long long &bad, int32_t tag, T *__restrict__ ck,
+                                            int level = -1, T *Wout = nullptr, int *newly = nullptr) {
+  if constexpr (!STAGED) level = a.level;
   T Un[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) {
@@ -124,6 +147,12 @@ __device__ __forceinline__ void finish_cell(const StepArgs<T> &a, const T *src, 
   if (SCH == 1) {
 #pragma unroll
     for (int k = 0; k < NV; k++) Ud[k * N + c] = Un[k];
+    if constexpr (STAGED) {
+      T W[NV];
+      cons_to_prim(Un, W);
+#pragma unroll
+      for (int k = 0; k < NV; k++) Wout[k * N + c] = W[k];
+    }
     return;
   }
   if (a.acc != nullptr) {
@@ -156,21 +185,26 @@ __device__ __forceinline__ void finish_cell(const StepArgs<T> &a, const T *src, 
   }
   T W[NV];
   cons_to_prim(Un, W);
+  if constexpr (STAGED) {
+#pragma unroll
+    for (int k = 0; k < NV; k++) Wout[k * N + c] = W[k];
+  }
   if (!realizable(W)) {
     bad = min(bad, (long long)c);
     if (!kCharacteristic<SCH>) goto done;  // the central scheme has no a-posteriori fallback
     {
     // tag the cell for the next fallback pass (a cell tagged by an earlier pass keeps its tag)
     const int32_t f = a.flags[c];
-    if (!((f >> 3) == tag && (f & 7) < a.level)) {
-      a.flags[c] = tag * 8 + a.level;
-      atomicAdd(&a.ctrl->nbad[a.level], 1);
+    if (!((f >> 3) == tag && (f & 7) < level)) {
+      a.flags[c] = tag * 8 + level;
+      atomicAdd(&a.ctrl->nbad[level], 1);
+      if constexpr (STAGED) atomicAdd(newly, 1);
     }
     }
   }
 done:
-  smax = fmax(smax, speed_sum<T, NDIM, CTU>(W, idx, idy, idz));
-  diag.add(Un);
+  smax = max_nonneg(smax, speed_sum<T, NDIM, CTU>(W, idx, idy, idz));
+  if constexpr (!STAGED) diag.add(Un);
 }
 
 template <typename T, int NT>

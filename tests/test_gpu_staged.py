@@ -1,0 +1,111 @@
+"""The staged step (the default of FP64 grids and of small FP32 grids) against the streaming
+step kernels (a grid whose tiling was set): the same arithmetic per cell and face, so the
+states, times and fallback tags have to agree bit for bit, at sizes around a group of 32
+items, with every kind of boundary, scheme, gravity and with fallback passes."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+BCS = {"per": (0, 0), "out": (1, 1), "ref": (2, 2), "mix": (2, 1)}
+
+
+@pytest.fixture(scope="module")
+def msh():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1210_5246_gb300 import msh as m
+    m.load()
+    return m
+
+
+def _state(shape, seed, extreme=False):
+    rng = np.random.default_rng(seed)
+    W = np.zeros((10,) + shape)
+    s = 2.0 if extreme else 0.5
+    W[0] = np.exp(rng.uniform(-s, s, shape))
+    W[1:4] = rng.uniform(-1.5, 1.5, (3,) + shape)
+    d = [rng.uniform(0.2, 1.0, shape) for _ in range(3)]
+    a, b, c = (rng.normal(0.0, 0.2, shape) for _ in range(3))
+    W[4], W[5], W[6] = d[0] ** 2, a * d[0], b * d[0]
+    W[7], W[8], W[9] = a * a + d[1] ** 2, a * b + c * d[1], b * b + c * c + d[2] ** 2
+    return W
+
+
+def _run(msh, n, bc, prec, scheme, W, steps, tiling, phi=None, G=0.0):
+    nd = len(n)
+    g = msh.Grid(n, (0.0,) * nd, (1.0, 1.5, 0.5)[:nd], (bc,) * nd, 0.3, prec)
+    if tiling:
+        g.set_tiling(8, 0 if nd == 3 else 4)
+    g.set_scheme(scheme)
+    if phi is not None:
+        g.set_potential(phi)
+    if G:
+        g.set_self_gravity(G)
+    g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+    dt = g.step()
+    n_, t = g.run(max_steps=steps)
+    out = (dt, n_, t, g.get_state(), g.diagnostics())
+    g.close()
+    return out
+
+
+def _same(a, b):
+    assert a[:3] == b[:3]
+    np.testing.assert_array_equal(a[3], b[3])
+    # the totals are summed in another order (FP32 streaming sums start in FP32)
+    scale = np.abs(b[4][0]).max()
+    assert np.abs(a[4][0] - b[4][0]).max() <= (1e-12 if a[3].dtype == np.float64 else 1e-6) * scale
+    assert a[4][1:] == b[4][1:]
+
+
+@pytest.mark.parametrize("prec", ["FP64", "FP32"])
+@pytest.mark.parametrize("scheme", ["MUSCL_HANCOCK", "MUSCL_HANCOCK_ROE", "MUSCL_HANCOCK_HLLC", "KT"])
+@pytest.mark.parametrize("n,bc", [((2,), "ref"), ((33,), "mix"), ((260,), "per"), ((31, 2), "out"), ((45, 33), "mix"),
+                                  ((64, 32), "per"), ((2, 3, 2), "ref"), ((33, 7, 19), "mix"), ((17, 32, 9), "per")])
+def test_staged_equals_streaming(msh, n, bc, scheme, prec):
+    W = _state(n[::-1] if len(n) == 3 else (1,) * (3 - len(n)) + n[::-1], sum(n))
+    p, s = getattr(msh, prec), getattr(msh, scheme)
+    if scheme == "KT":
+        W[1:4] *= 0.3
+    _same(_run(msh, n, BCS[bc], p, s, W, 20, False), _run(msh, n, BCS[bc], p, s, W, 20, True))
+
+
+@pytest.mark.parametrize("prec", ["FP64", "FP32"])
+@pytest.mark.parametrize("n", [(45, 33), (33, 7, 19)])
+def test_staged_gravity_equals_streaming(msh, n, prec):
+    W = _state((1,) * (3 - len(n)) + n[::-1], 3)
+    rng = np.random.default_rng(5)
+    pad = tuple(m + 2 for m in n[::-1])
+    phi = 0.01 * rng.uniform(-1.0, 1.0, (1,) * (3 - len(n)) + pad)
+    p = getattr(msh, prec)
+    _same(_run(msh, n, BCS["out"], p, 0, W, 20, False, phi), _run(msh, n, BCS["out"], p, 0, W, 20, True, phi))
+    _same(_run(msh, n, BCS["per"], p, 0, W, 40, False, phi, 0.2), _run(msh, n, BCS["per"], p, 0, W, 40, True, phi, 0.2))
+
+
+@pytest.mark.parametrize("prec", ["FP64", "FP32"])
+@pytest.mark.parametrize("scheme", ["MUSCL_HANCOCK", "MUSCL_HANCOCK_ROE", "MUSCL_HANCOCK_HLLC"])
+@pytest.mark.parametrize("n,bc", [((300,), "out"), ((60, 41), "mix"), ((25, 18, 12), "ref")])
+def test_staged_fallback_equals_streaming(msh, n, bc, scheme, prec):
+    """Extreme states over steps longer than the CFL rule allows: cells are tagged and fallback
+    passes run; tags counted per step and the states agree."""
+    W = _state((1,) * (3 - len(n)) + n[::-1], 7, extreme=True)
+    nd, out = len(n), []
+    for tiling in (False, True):
+        g = msh.Grid(n, (0.0,) * nd, (1.0,) * nd, (BCS[bc],) * nd, 0.5, getattr(msh, prec))
+        if tiling:
+            g.set_tiling(4, 5)
+        g.set_scheme(getattr(msh, scheme))
+        g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+        _, dt, _ = g.reduce_layers(0, n[-1])
+        tags = []
+        for f in (1.0, 1.2, 1.0):
+            try:
+                tags.append(g.step_dt(f * dt))
+            except msh.MshError as e:  # a cell that stays non-realizable: the state is kept
+                tags.append((e.status, str(e)))
+                break
+        out.append((tags, g.get_state()))
+        g.close()
+    assert out[0][0] == out[1][0] and out[0][0][0] != 0
+    np.testing.assert_array_equal(out[0][1], out[1][1])
