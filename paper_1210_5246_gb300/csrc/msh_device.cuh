@@ -37,14 +37,38 @@ template <> struct Frame<2> {
 
 // ---------------------------------------------------------- fast arithmetic
 // FP32: hardware approximate reciprocal and reciprocal square root (a few ulp, far
-// inside the FP32 tolerances); FP64: IEEE division and square root.
+// inside the FP32 tolerances).  FP64: IEEE division, and CUDA's rsqrt() (1 ulp) for the
+// square roots: a double-precision warp instruction holds its scheduler's pipe for 64 cycles
+// on GB300, and 1 / sqrt(x) took 930 of them where rsqrt(x) takes 377, sqrt(p / r) 1160 where
+// p rsqrt(p r) takes 505 (measured, independent chains).
 template <typename T> __device__ __forceinline__ T frcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float frcp<float>(float x) { return __fdividef(1.0f, x); }
-template <typename T> __device__ __forceinline__ T frsqrt(T x) { return T(1) / sqrt(x); }
-template <> __device__ __forceinline__ float frsqrt<float>(float x) { return rsqrtf(x); }
+__device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double frsqrt(double x) { return rsqrt(x); }
 // sqrt(p / r) for p, r > 0
-template <typename T> __device__ __forceinline__ T sqrt_ratio(T p, T r) { return sqrt(p / r); }
-template <> __device__ __forceinline__ float sqrt_ratio<float>(float p, float r) { return p * rsqrtf(p * r); }
+template <typename T> __device__ __forceinline__ T sqrt_ratio(T p, T r) { return p * frsqrt(p * r); }
+
+// x > 0, x >= 0 and min / max.  FP64: on the bit patterns (integer instructions; the
+// double-precision compare runs on the 64-cycle pipe).  A NaN is neither > 0 nor >= 0; the
+// min / max of a NaN is unspecified (its flux is NaN whatever they return).
+__device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool gt0(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool ge0(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool ge0(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b <= 0x7ff0000000000000ull || b == 0x8000000000000000ull;
+}
+__device__ __forceinline__ long long order_bits(double x) {  // orders like the numbers
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ float min_of(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double min_of(double a, double b) { return order_bits(a) < order_bits(b) ? a : b; }
+__device__ __forceinline__ double max_of(double a, double b) { return order_bits(a) > order_bits(b) ? a : b; }
 
 // Sum and product that are never contracted into a fused multiply-add.  Where an expression
 // leaves the compiler a choice of what to fuse, the Roe-type scheme states it, so that every
@@ -160,7 +184,7 @@ template <typename T> __device__ __forceinline__ bool realizable(const T (&W)[NV
   const T m2 = W[4] * W[7] - W[5] * W[5];
   const T m3 = W[4] * (W[7] * W[9] - W[8] * W[8]) - W[5] * (W[5] * W[9] - W[8] * W[6]) +
                W[6] * (W[5] * W[8] - W[7] * W[6]);
-  return W[0] > T(0) && m1 > T(0) && m2 > T(0) && m3 > T(0);
+  return gt0(W[0]) && gt0(m1) && gt0(m2) && gt0(m3);
 }
 
 // ----------------------------------------------------------- reconstruction
@@ -174,9 +198,23 @@ template <typename T> __device__ __forceinline__ T mc_limit(T dl, T dr) {
 // The same limiter doubled: 2 mc(dL, dR) = sign(dL) min(4|dL|, 4|dR|, |dL + dR|) for
 // same-sign differences, else 0.  Scaling by powers of two is exact, so this is exactly
 // twice mc_limit (two instructions cheaper).
-template <typename T> __device__ __forceinline__ T mc_limit2(T dl, T dr) {
-  const T m = fmin(T(4) * fmin(fabs(dl), fabs(dr)), fabs(dl + dr));
-  return (dl * dr > T(0)) ? copysign(m, dl) : T(0);
+__device__ __forceinline__ float mc_limit2(float dl, float dr) {
+  const float m = fminf(4.0f * fminf(fabsf(dl), fabsf(dr)), fabsf(dl + dr));
+  return (dl * dr > 0.0f) ? copysignf(m, dl) : 0.0f;
+}
+// FP64: the signs and the two minima on the bit patterns, so that two double-precision
+// instructions are left of six (the pipe's 64 cycles each; the limiter was a quarter of a
+// reconstruction's time).  A NaN difference gives 0, as dl dr > 0 does; differences whose
+// product underflows are not cut to 0.
+__device__ __forceinline__ double mc_limit2(double dl, double dr) {
+  constexpr long long kAbs = 0x7fffffffffffffffll, kInf = 0x7ff0000000000000ll, kSign = ~kAbs;
+  const long long bl = __double_as_longlong(dl), br = __double_as_longlong(dr);
+  const long long al = bl & kAbs, ar = br & kAbs;
+  const long long lo = al < ar ? al : ar, hi = al < ar ? ar : al;
+  const long long q = __double_as_longlong(4.0 * __longlong_as_double(lo));
+  const long long c = __double_as_longlong(dl + dr) & kAbs;
+  const bool on = (bl ^ br) >= 0 && lo != 0 && hi <= kInf;
+  return __longlong_as_double(on ? ((q < c ? q : c) | (bl & kSign)) : 0ll);
 }
 
 // The doubled limiter on every amplitude of a 10-vector (FP32: the sum, the product and the
@@ -218,21 +256,25 @@ template <typename T> struct Eig {
   }
   // characteristic amplitudes c = L d in wave order
   // (f-, sv-, sw-, c_rho, c_yy, c_yz, c_zz, sv+, sw+, f+)
+  // t = d_xx / (6 P_xx) is the pressure part of both fast waves; the contact amplitudes take
+  // 2 t.  The factors of the cell are formed once for its two projections.
   __device__ __forceinline__ void project(const T (&d)[NV], T (&c)[NV]) const {
-    const T e = d[4] * ip * T(1.0 / 3.0);
-    const T t1 = d[1] * icf2, t2 = T(0.5) * e;
-    c[0] = t2 - t1;
-    c[9] = t2 + t1;
-    const T qv = (d[2] - a * d[1]) * ics2, rv = T(0.5) * (d[5] - a * d[4]) * ip;
-    c[1] = rv - qv;
-    c[7] = rv + qv;
-    const T qw = (d[3] - b * d[1]) * ics2, rw = T(0.5) * (d[6] - b * d[4]) * ip;
-    c[2] = rw - qw;
-    c[8] = rw + qw;
-    c[3] = d[0] - rho * e;
-    c[4] = d[7] - T(2) * a * d[5] + (T(4) * a * Pxy - Pyy) * e;
-    c[5] = d[8] - b * d[5] - a * d[6] + (T(4) * a * Pxz - Pyz) * e;
-    c[6] = d[9] - T(2) * b * d[6] + (T(4) * b * Pxz - Pzz) * e;
+    const T ip6 = ip * T(1.0 / 6.0), hip = T(0.5) * ip, r2 = T(2) * rho, a2 = T(2) * a, b2 = T(2) * b;
+    const T k4 = T(2) * fma(T(4) * a, Pxy, -Pyy), k5 = T(2) * fma(T(4) * a, Pxz, -Pyz),
+            k6 = T(2) * fma(T(4) * b, Pxz, -Pzz);
+    const T t = d[4] * ip6;
+    c[0] = fma(-d[1], icf2, t);
+    c[9] = fma(d[1], icf2, t);
+    const T qv = fma(-a, d[1], d[2]), rv = fma(-a, d[4], d[5]) * hip;
+    c[1] = fma(-qv, ics2, rv);
+    c[7] = fma(qv, ics2, rv);
+    const T qw = fma(-b, d[1], d[3]), rw = fma(-b, d[4], d[6]) * hip;
+    c[2] = fma(-qw, ics2, rw);
+    c[8] = fma(qw, ics2, rw);
+    c[3] = fma(-r2, t, d[0]);
+    c[4] = fma(k4, t, fma(-a2, d[5], d[7]));
+    c[5] = fma(k5, t, fma(-a, d[6], fma(-b, d[5], d[8])));
+    c[6] = fma(k6, t, fma(-b2, d[6], d[9]));
   }
   // primitive vector R c
   __device__ __forceinline__ void back(const T (&c)[NV], T (&o)[NV]) const {
@@ -315,7 +357,7 @@ __device__ __forceinline__ void transverse(const T (&wm)[NV], const T (&w0)[NV],
 // order).
 template <typename T>
 __device__ __forceinline__ void face_state_check(const T (&w0)[NV], T (&lo)[NV], T (&hi)[NV]) {
-  const bool ok = hi[0] > T(0) && lo[0] > T(0) && hi[4] > T(0) && lo[4] > T(0);
+  const bool ok = gt0(hi[0]) && gt0(lo[0]) && gt0(hi[4]) && gt0(lo[4]);
   if (!ok) {
 #pragma unroll
     for (int k = 0; k < NV; k++) { hi[k] = w0[k]; lo[k] = w0[k]; }
@@ -470,21 +512,23 @@ __device__ __forceinline__ void phys(const T (&w)[NV], T (&U)[NV], T (&F)[NV]) {
 
 // HLL flux between local-frame face states wl | wr with signal speeds
 // S_L = min(u_L - cf_L, u_R - cf_R), S_R = max(u_L + cf_L, u_R + cf_R).
+// FP32 adds the two sides' physical fluxes and conserved states in packed instructions; FP64,
+// which pays per operation, uses F_K = u_K U_K + Pi_K (pi_terms), 84 instead of 98 operations
+// after the signal speeds.
+template <typename T>
+__device__ __forceinline__ void cons_pi(const T (&w)[NV], T (&U)[NV], T (&P)[NV]);
 template <typename T>
 __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
-  T Ul[NV], Fl[NV], Ur[NV], Fr[NV];
-  phys(wl, Ul, Fl);
-  phys(wr, Ur, Fr);
   const T cl = T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
   const T cr = T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
-  const T SL = fmin(wl[1] - cl, wr[1] - cr);
-  const T SR = fmax(wl[1] + cl, wr[1] + cr);
+  const T SL = min_of(wl[1] - cl, wr[1] - cr);
+  const T SR = max_of(wl[1] + cl, wr[1] + cr);
   // F = a Fl + b Fr + c (Ur - Ul): (1, 0, 0) for SL >= 0, (0, 1, 0) for SR <= 0, else
   // (SR, -SL, SL SR) / (SR - SL); the branch selects three scalars, not ten fluxes
   T a, b, c;
-  if (SL >= T(0)) {
+  if (ge0(SL)) {
     a = T(1); b = T(0); c = T(0);
-  } else if (SR <= T(0)) {
+  } else if (ge0(-SR)) {
     a = T(0); b = T(1); c = T(0);
   } else {
     const T inv = frcp(SR - SL);
@@ -492,7 +536,19 @@ __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)
     b = -SL * inv;
     c = SL * SR * inv;
   }
-  T t[NV];
+  if constexpr (sizeof(T) == 8) {
+    T Ul[NV], Pl[NV], Ur[NV], Pr[NV];
+    cons_pi(wl, Ul, Pl);
+    cons_pi(wr, Ur, Pr);
+    const T al = fma(a, wl[1], -c), br = fma(b, wr[1], c);
+    F[0] = fma(al, Ul[0], br * Ur[0]);
+#pragma unroll
+    for (int k = 1; k < NV; k++) F[k] = fma(al, Ul[k], fma(br, Ur[k], fma(a, Pl[k], b * Pr[k])));
+    return;
+  }
+  T Ul[NV], Fl[NV], Ur[NV], Fr[NV], t[NV];
+  phys(wl, Ul, Fl);
+  phys(wr, Ur, Fr);
   v_sub(t, Ur, Ul);
   v_mul(t, t, c);
   v_fma(t, Fr, b, t);
@@ -604,6 +660,12 @@ __device__ __forceinline__ void pi_terms(T u, T v, T w, T pxx, T pxy, T pxz, T (
   P[9] = T(2) * pxz * w;
 }
 
+// Conserved state and Pi of a local-frame primitive state.
+template <typename T> __device__ __forceinline__ void cons_pi(const T (&w)[NV], T (&U)[NV], T (&P)[NV]) {
+  prim_to_cons(w, U);
+  pi_terms(w[1], w[2], w[3], w[4], w[5], w[6], P);
+}
+
 // Three-wave HLLC flux for the ten-moment system (local frame).  Outer waves S_L, S_R as in
 // HLL (they carry the fast and shear waves), the contact S_M in between (it carries rho and
 // the transverse stresses).  Every pair (u_i, P_ix) takes one star value on both sides of
@@ -619,8 +681,8 @@ template <typename T>
 __device__ __forceinline__ void hllc_flux(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
   const T cl = T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
   const T cr = T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
-  const T SL = fmin(wl[1] - cl, wr[1] - cr);
-  const T SR = fmax(wl[1] + cl, wr[1] + cr);
+  const T SL = min_of(wl[1] - cl, wr[1] - cr);
+  const T SR = max_of(wl[1] + cl, wr[1] + cr);
   const T CL = wl[0] * (SL - wl[1]), CR = wr[0] * (SR - wr[1]);
   const T inv = frcp(CR - CL);
   T us[3], ps[3];
@@ -634,13 +696,13 @@ __device__ __forceinline__ void hllc_flux(const T (&wl)[NV], const T (&wr)[NV], 
     hll(wl, wr, F);
     return;
   }
-  const bool left = SM >= T(0);
+  const bool left = ge0(SM);
   T wk[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) wk[k] = left ? wl[k] : wr[k];
   const T SK = left ? SL : SR, uk = wk[1];
   T a, b, c;
-  if (SL >= T(0) || SR <= T(0)) {
+  if (ge0(SL) || ge0(-SR)) {
     a = uk; b = T(1); c = T(0);
   } else {
     const T i2 = frcp(SK - SM);

@@ -281,35 +281,12 @@ __device__ __forceinline__ void divergence(const StagedArgs<T> &a, size_t N, int
   }
 }
 
-// Sums of ten values over a warp with 12 additions per lane instead of 50: each step halves
-// the components a lane keeps.  Lane 2 m (even) ends with one component's sum; returns its
-// index in `comp` (or -1).
-__device__ __forceinline__ double warp_sum10(double (&v)[NV], int &comp) {
-  const int lane = threadIdx.x & 31;
-  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
-  double p[6];
-#pragma unroll
-  for (int k = 0; k < 5; k++) p[k] = (b4 ? v[k + 5] : v[k]) + __shfl_xor_sync(FULL, b4 ? v[k] : v[k + 5], 16);
-  p[5] = 0.0;
-  double q[4];
-#pragma unroll
-  for (int k = 0; k < 3; k++) q[k] = (b3 ? p[k + 3] : p[k]) + __shfl_xor_sync(FULL, b3 ? p[k] : p[k + 3], 8);
-  q[3] = 0.0;
-  double r[2];
-#pragma unroll
-  for (int k = 0; k < 2; k++) r[k] = (b2 ? q[k + 2] : q[k]) + __shfl_xor_sync(FULL, b2 ? q[k] : q[k + 2], 4);
-  double x = (b1 ? r[1] : r[0]) + __shfl_xor_sync(FULL, b1 ? r[0] : r[1], 2);
-  x += __shfl_xor_sync(FULL, x, 1);
-  const int in3 = (b2 ? 2 : 0) + (b1 ? 1 : 0), in5 = (b3 ? 3 : 0) + in3;
-  comp = (in3 < 3 && in5 < 5) ? (b4 ? 5 : 0) + in5 : -1;
-  return x;
-}
-
 // The time control of a launch, the same in every block.
 struct StagedTime {
   double t, t_next, dt, dt_last, dt_cfl;
   int64_t step;
   int64_t first_bad;
+  double nu[3];  // dt / (2 dx)
   int done, status, realizable, last_tagged, stop, newly, any_tagged;
 };
 
@@ -351,8 +328,10 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     if (a.seg != nullptr) st.dt = a.dts[0];
   }
   __syncthreads();
-  const double ddx0 = s.dx[0], ddx1 = s.dx[1], ddx2 = s.dx[2];
-  const T idx = (T)(1.0 / ddx0), idy = (T)(1.0 / ddx1), idz = (T)(1.0 / ddx2);
+  __shared__ double sc[6];
+  step_factors(s.dx, st.dt, sc);
+  const T idx = (T)sc[3], idy = (T)sc[4], idz = (T)sc[5];
+  if (tid < 3) st.nu[tid] = sc[tid];  // first read after a barrier
   // groups of 32 items are dealt out warp by warp, blocks first, so that a short list
   // spreads over the SMs and over the schedulers of each
   const int w0 = warp * (int)nblk + (int)blk, wstep = kStagedWarps * (int)nblk;
@@ -371,8 +350,8 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
   T smax = T(0);
   long long bad = LLONG_MAX;
 
-  auto stages_ab = [&](const T *W, double dt, int32_t tag, int level) {
-    const T nux = (T)(0.5 * dt / ddx0), nuy = (T)(0.5 * dt / ddx1), nuz = (T)(0.5 * dt / ddx2);
+  auto stages_ab = [&](const T *W, int32_t tag, int level) {
+    const T nux = (T)st.nu[0], nuy = (T)st.nu[1], nuz = (T)st.nu[2];
     for (int g = w0; g < NDIM * ngrp + ngh; g += wstep) {
       bool ghost = g >= NDIM * ngrp;
       int d, it;
@@ -507,20 +486,20 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     T *Wn = a.W[(step + 1) & 1];
     T *const ck = (kKt || a.seg != nullptr) ? nullptr : tape_slot(s, step, N);
     if constexpr (kKt) {
-      stages_ab(W0, dt, tag, 0);
+      stages_ab(W0, tag, 0);
       if (!alive) break;
       // the first stage's primitive state goes to the next step's buffer, which the second
       // stage replaces once every face state has been formed from it
       stage_c(std::integral_constant<int, 1>{}, U0, U0, s.U1, Wn, dt, tag, 0, (T *)nullptr);
       alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
       if (!alive) break;
-      stages_ab(Wn, dt, tag, 0);
+      stages_ab(Wn, tag, 0);
       if (!alive) break;
       stage_c(std::integral_constant<int, 2>{}, s.U1, U0, Ud, Wn, dt, tag, 0, (T *)nullptr);
       write_part();
     } else {
       const int level = a.phase >= 0 ? a.phase : 0;
-      stages_ab(W0, dt, tag, level);
+      stages_ab(W0, tag, level);
       if (!alive) break;
       stage_c(std::integral_constant<int, 0>{}, U0, U0, Ud, Wn, dt, tag, level, level == 0 ? ck : nullptr);
       write_part();
@@ -543,7 +522,7 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     // pass before tagged new ones
     if (!kKt) {
       for (int level = 1; level <= kFallbackPasses && st.newly > 0; level++) {
-        stages_ab(W0, dt, tag, level);
+        stages_ab(W0, tag, level);
         if (!alive) break;
         stage_c(std::integral_constant<int, 0>{}, U0, U0, Ud, Wn, dt, tag, level, (T *)nullptr);
         write_part();
@@ -605,6 +584,8 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     }
     __syncthreads();
     if (st.stop) break;
+    if (tid < 3) st.nu[tid] = 0.5 * st.dt / (tid == 0 ? s.dx[0] : tid == 1 ? s.dx[1] : s.dx[2]);
+    __syncthreads();
   }
   if (!alive) {  // a barrier gave up: the result is void
     if (tid == 0 && a.seg == nullptr) {

@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(256) scan_kernel(const T *__restrict__ U, size
     for (int k = 0; k < NV; k++) Uc[k] = U[k * N + c];
     cons_to_prim(Uc, W);
     if (!realizable(W)) bad = min(bad, (long long)c);
-    smax = fmax(smax, speed_sum<T, NDIM, MAXF>(W, idx, idy, idz));
+    smax = max_nonneg(smax, speed_sum<T, NDIM, MAXF>(W, idx, idy, idz));
 #pragma unroll
     for (int k = 0; k < NV; k++) diag[k] += (double)Uc[k];
   }
@@ -74,30 +74,40 @@ __device__ void plan(Ctrl *c) {
 __global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, const Partial *part,
                                                                     int nparts, int mode) {
   if (mode == 0 && ctrl->done) return;
-  __shared__ double sd[kFinalizeThreads][NV + 1];
-  __shared__ long long sb[kFinalizeThreads];
-  const int t = threadIdx.x;
+  constexpr int kWarps = kFinalizeThreads / 32;
+  __shared__ double sd[kWarps][NV + 1], stot[NV];
+  __shared__ long long sb[kWarps];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   double d[NV];
   for (int k = 0; k < NV; k++) d[k] = 0.0;
   double smax = 0.0;
   long long bad = LLONG_MAX;
   for (int i = t; i < nparts; i += kFinalizeThreads) {
     for (int k = 0; k < NV; k++) d[k] += part[i].diag[k];
-    smax = fmax(smax, part[i].smax);
+    smax = max_nonneg(smax, part[i].smax);
     bad = min(bad, part[i].bad);
   }
-  for (int k = 0; k < NV; k++) sd[t][k] = d[k];
-  sd[t][NV] = smax;
-  sb[t] = bad;
-  __syncthreads();
-  for (int s = kFinalizeThreads / 2; s > 0; s >>= 1) {  // pairwise, fixed order
-    if (t < s) {
-      for (int k = 0; k < NV; k++) sd[t][k] += sd[t + s][k];
-      sd[t][NV] = fmax(sd[t][NV], sd[t + s][NV]);
-      sb[t] = min(sb[t], sb[t + s]);
-    }
-    __syncthreads();
+  // fixed order: strided sums per thread, warps, then one thread per component over the warps
+  int comp;
+  const double x = warp_sum10(d, comp);
+  smax = warp_max_nonneg(smax);
+  for (int o = 16; o > 0; o >>= 1) bad = min(bad, __shfl_xor_sync(FULL, bad, o));
+  if (comp >= 0 && (lane & 1) == 0) sd[warp][comp] = x;
+  if (lane == 0) {
+    sd[warp][NV] = smax;
+    sb[warp] = bad;
   }
+  __syncthreads();
+  if (t < NV) {
+    double sum = sd[0][t];
+    for (int w = 1; w < kWarps; w++) sum += sd[w][t];
+    stot[t] = sum;
+  }
+  for (int w = 0; w < kWarps; w++) {
+    smax = max_nonneg(smax, sd[w][NV]);
+    bad = min(bad, sb[w]);
+  }
+  __syncthreads();
   if (t != 0) return;
   Ctrl *c = ctrl;
   if (mode == 0 && c->stage_timeout) {  // the step kernel gave up waiting for staged data
@@ -105,11 +115,11 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, 
     c->done = 1;
     return;
   }
-  for (int k = 0; k < NV; k++) c->totals[k] = sd[0][k];
-  const long long b = sb[0];
+  for (int k = 0; k < NV; k++) c->totals[k] = stot[k];
+  const long long b = bad;
   c->realizable = (b == LLONG_MAX);
   c->first_bad = (b == LLONG_MAX) ? -1 : b;
-  c->dt_cfl = c->cfl / sd[0][NV];
+  c->dt_cfl = c->cfl / smax;
   if (mode == 1) {
     c->done = 1;
     return;

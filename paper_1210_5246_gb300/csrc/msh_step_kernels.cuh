@@ -41,6 +41,52 @@ namespace msh {
 constexpr unsigned FULL = 0xffffffffu;
 
 // ------------------------------------------------------------ block partials
+// max of a running maximum m >= 0 and a signal speed s >= 0; a NaN s leaves m (fmax's rule).
+// FP64: on the bit patterns, which order like non-negative numbers -- integer instructions
+// instead of the double-precision pipe (64 cycles per warp instruction).
+__device__ __forceinline__ float max_nonneg(float m, float s) { return fmaxf(m, s); }
+__device__ __forceinline__ double max_nonneg(double m, double s) {
+  const long long a = __double_as_longlong(m), b = __double_as_longlong(s);
+  return (b > a && b <= 0x7ff0000000000000ll) ? s : m;
+}
+// the same over a warp, in every lane
+__device__ __forceinline__ float warp_max_nonneg(float m) {
+  return __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(m)));
+}
+__device__ __forceinline__ double warp_max_nonneg(double m) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max_nonneg(m, __shfl_xor_sync(FULL, m, o));
+  return m;
+}
+
+// Sums of ten values over a warp with 12 additions per lane instead of 50: each step halves
+// the components a lane keeps.  Lane 2 m (even) ends with one component's sum; returns its
+// index in `comp` (or -1).
+__device__ __forceinline__ double warp_sum10(double (&v)[NV], int &comp) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+  double p[6];
+#pragma unroll
+  for (int k = 0; k < 5; k++) p[k] = (b4 ? v[k + 5] : v[k]) + __shfl_xor_sync(FULL, b4 ? v[k] : v[k + 5], 16);
+  p[5] = 0.0;
+  double q[4];
+#pragma unroll
+  for (int k = 0; k < 3; k++) q[k] = (b3 ? p[k + 3] : p[k]) + __shfl_xor_sync(FULL, b3 ? p[k] : p[k + 3], 8);
+  q[3] = 0.0;
+  double r[2];
+#pragma unroll
+  for (int k = 0; k < 2; k++) r[k] = (b2 ? q[k + 2] : q[k]) + __shfl_xor_sync(FULL, b2 ? q[k] : q[k + 2], 4);
+  double x = (b1 ? r[1] : r[0]) + __shfl_xor_sync(FULL, b1 ? r[0] : r[1], 2);
+  x += __shfl_xor_sync(FULL, x, 1);
+  const int in3 = (b2 ? 2 : 0) + (b1 ? 1 : 0), in5 = (b3 ? 3 : 0) + in3;
+  comp = (in3 < 3 && in5 < 5) ? (b4 ? 5 : 0) + in5 : -1;
+  return x;
+}
+
+// Partial of a block of NT threads: totals (plus `base`), signal speed, first bad cell.  The
+// FP64 additions are few on purpose: 12 per warp (warp_sum10), then ten threads sum one
+// component each over the warps; every one holds a scheduler's FP64 pipe for 64 cycles or
+// more, also in FP32 kernels (one thread adding ten components of 16 warps took 6 us).
 template <int NT>
 __device__ __forceinline__ void block_partial(double (&diag)[NV], double smax, long long bad,
                                               Partial *out, const double *base = nullptr) {
@@ -49,31 +95,33 @@ __device__ __forceinline__ void block_partial(double (&diag)[NV], double smax, l
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const int warp = tid >> 5;
+  int comp;
+  const double x = warp_sum10(diag, comp);
+  smax = warp_max_nonneg(smax);
+  if (__any_sync(FULL, bad != LLONG_MAX)) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < NV; k++) diag[k] += __shfl_down_sync(FULL, diag[k], o);
-    smax = fmax(smax, __shfl_down_sync(FULL, smax, o));
-    bad = min(bad, __shfl_down_sync(FULL, bad, o));
+    for (int o = 16; o > 0; o >>= 1) bad = min(bad, __shfl_xor_sync(FULL, bad, o));
   }
+  if (comp >= 0 && (lane & 1) == 0) red[warp][comp] = x;
   if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; k++) red[warp][k] = diag[k];
     red[warp][NV] = smax;
     redb[warp] = bad;
   }
   __syncthreads();
-  if (tid == 0) {
-    Partial p;
-    for (int k = 0; k < NV; k++) p.diag[k] = base != nullptr ? base[k] : 0.0;
-    p.smax = 0.0;
-    p.bad = LLONG_MAX;
-    for (int w = 0; w < NT / 32; w++) {
-      for (int k = 0; k < NV; k++) p.diag[k] += red[w][k];
-      p.smax = fmax(p.smax, red[w][NV]);
-      p.bad = min(p.bad, redb[w]);
+  if (tid < NV) {
+    double sum = base != nullptr ? base[tid] : 0.0;
+    for (int w = 0; w < NT / 32; w++) sum += red[w][tid];
+    out->diag[tid] = sum;
+  }
+  if (tid == NT - 1) {
+    double m = red[0][NV];
+    long long b = redb[0];
+    for (int w = 1; w < NT / 32; w++) {
+      m = max_nonneg(m, red[w][NV]);
+      b = min(b, redb[w]);
     }
-    *out = p;
+    out->smax = m;
+    out->bad = b;
   }
 }
 
@@ -93,22 +141,16 @@ __device__ __forceinline__ T speed_sum(const T (&W)[NV], T idx, T idy, T idz) {
   return s;
 }
 
-// max of a running maximum m >= 0 and a signal speed s >= 0; a NaN s leaves m (fmax's rule).
-// FP64: on the bit patterns, which order like non-negative numbers -- integer instructions
-// instead of the double-precision pipe (64 cycles per warp instruction).
-__device__ __forceinline__ float max_nonneg(float m, float s) { return fmaxf(m, s); }
-__device__ __forceinline__ double max_nonneg(double m, double s) {
-  const long long a = __double_as_longlong(m), b = __double_as_longlong(s);
-  return (b > a && b <= 0x7ff0000000000000ll) ? s : m;
-}
-// the same over a warp, in every lane
-__device__ __forceinline__ float warp_max_nonneg(float m) {
-  return __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(m)));
-}
-__device__ __forceinline__ double warp_max_nonneg(double m) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_nonneg(m, __shfl_xor_sync(FULL, m, o));
-  return m;
+// nu_d = dt / (2 dx_d) and 1 / dx_d, rounded from FP64: one lane per quotient and a broadcast
+// through shared memory.  (Every thread dividing for itself took six FP64 divisions, 580
+// pipe cycles each, per warp of every block.)
+__device__ __forceinline__ void step_factors(const double (&dx)[3], double dt, double *sc) {
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  if (tid < 6) {
+    const int d = tid < 3 ? tid : tid - 3;
+    sc[tid] = (tid < 3 ? 0.5 * dt : 1.0) / (d == 0 ? dx[0] : d == 1 ? dx[1] : dx[2]);
+  }
+  __syncthreads();
 }
 
 // Checkpoint slot of the adjoint tape that step `step` stores U^step into, or nullptr.
@@ -222,14 +264,14 @@ __device__ __forceinline__ void write_partial(const Acc<T> &diag, T smax, long l
   block_partial<NT>(d, (double)smax, bad, out, base);
 }
 
-// FP64 running totals of a thread block, in shared memory (thread 0 writes them).
+// FP64 running totals of a thread block, in shared memory (threads 0 to 9 write one each).
 __device__ __forceinline__ double *block_totals() {
   __shared__ double tot[NV];
   return tot;
 }
 
 // Move the threads' running sums into the block's FP64 totals (fixed order: warps by
-// shuffles, then thread 0 over the warps) and restart them from zero.  Every thread of the
+// shuffles, then one thread per component over the warps) and restart them from zero.  Every thread of the
 // block calls it.
 template <typename T, int NT> __device__ __forceinline__ void flush_totals(Acc<T> &diag, double *tot) {
   __shared__ double red[NT / 32][NV];
@@ -237,19 +279,14 @@ template <typename T, int NT> __device__ __forceinline__ void flush_totals(Acc<T
   diag.get(d);
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < NV; k++) d[k] += __shfl_down_sync(FULL, d[k], o);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; k++) red[tid >> 5][k] = d[k];
-  }
+  int comp;
+  const double x = warp_sum10(d, comp);
+  if (comp >= 0 && (lane & 1) == 0) red[tid >> 5][comp] = x;
   __syncthreads();
-  if (tid == 0) {
-    for (int w = 0; w < NT / 32; w++)
-      for (int k = 0; k < NV; k++) tot[k] += red[w][k];
+  if (tid < NV) {
+    double sum = tot[tid];
+    for (int w = 0; w < NT / 32; w++) sum += red[w][tid];
+    tot[tid] = sum;
   }
   diag.zero();
 }
@@ -276,7 +313,9 @@ __global__ void __launch_bounds__(kTile1D) step1d_kernel(StepArgs<T> a) {
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
   const double dtd = ctrl->dt;
-  const T dt = (T)dtd, nu = (T)(0.5 * dtd / a.dx[0]), idx = (T)(1.0 / a.dx[0]);
+  __shared__ double sc[6];
+  step_factors(a.dx, dtd, sc);
+  const T dt = (T)dtd, nu = (T)sc[0], idx = (T)sc[3];
   __shared__ T sW[NV][SXX];
   __shared__ T sH[NV][B];
   const int t = threadIdx.x;
@@ -461,10 +500,12 @@ __global__ void __launch_bounds__(32 * BY, (BY <= 8 && !CTU && sizeof(T) == 4 ? 
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
   const double dtd = ctrl->dt;
+  __shared__ double sc[6];
+  step_factors(a.dx, dtd, sc);
   const T dt = (T)dtd;
-  const T nux = (T)(0.5 * dtd / a.dx[0]), idx = (T)(1.0 / a.dx[0]);
-  const T nuy = (T)(0.5 * dtd / a.dx[1]), idy = (T)(1.0 / a.dx[1]);
-  const T nuz = (T)(0.5 * dtd / a.dx[2]), idz = (T)(1.0 / a.dx[2]);
+  const T nux = (T)sc[0], idx = (T)sc[3];
+  const T nuy = (T)sc[1], idy = (T)sc[4];
+  const T nuz = (T)sc[2], idz = (T)sc[5];
   T *const ck = (RETRY || SCH != 0) ? nullptr : tape_slot(a, step, (size_t)a.nx * a.ny * a.nz);
   // shared memory: RAW raw conserved planes filled one plane ahead (bulk tensor copies or
   // cp.async), three primitive planes (ring), the y-sweep face states and fluxes, per staged
@@ -1004,9 +1045,11 @@ __global__ void __launch_bounds__(32 * WARPS) step_strip2d_kernel(StepArgs<T> a)
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
   const double dtd = ctrl->dt;
+  __shared__ double sc[6];
+  step_factors(a.dx, dtd, sc);
   const T dt = (T)dtd;
-  const T nux = (T)(0.5 * dtd / a.dx[0]), idx = (T)(1.0 / a.dx[0]);
-  const T nuy = (T)(0.5 * dtd / a.dx[1]), idy = (T)(1.0 / a.dx[1]);
+  const T nux = (T)sc[0], idx = (T)sc[3];
+  const T nuy = (T)sc[1], idy = (T)sc[4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nx = a.nx, ny = a.ny, ych = a.zchunk;
   const size_t N = (size_t)nx * ny;
