@@ -478,18 +478,10 @@ int grid_blocks(size_t n) {
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
 }
 
-// One forward step src -> dst with the fixed dt (no finalize: the schedule is given).  The
-// fallback passes are launched only when `passes` is set, i.e. when the step is known (or
-// not yet known) to tag cells; a step that tagged none recomputes identically without them.
-template <typename T>
-cudaError_t forward_step(msh_grid *g, Ctrl *ctl, Partial *part, T *src, T *dst, int64_t step, double dt,
-                         bool passes) {
-  adj_setup_kernel<<<1, 1, 0, g->stream>>>(ctl, step, dt);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+// Step arguments of the recomputed forward steps (no tape, no second stage).
+template <typename T> StepArgs<T> forward_args(msh_grid *g, Ctrl *ctl, Partial *part) {
   StepArgs<T> a;
-  a.U[step & 1] = src;
-  a.U[(step + 1) & 1] = dst;
+  a.U[0] = a.U[1] = nullptr;
   a.acc = (const T *)g->acc;
   a.ctrl = ctl;
   a.part = part;
@@ -500,11 +492,27 @@ cudaError_t forward_step(msh_grid *g, Ctrl *ctl, Partial *part, T *src, T *dst, 
   for (int i = 0; i < 6; i++) a.bc[i] = g->bc[i];
   for (int i = 0; i < 3; i++) a.dx[i] = g->dx[i];
   a.zchunk = g->zchunk;
+  a.level = 0;
   a.ck = nullptr;
   a.ck_base = 0;
   a.ck_len = 0;
   a.ck_K = 1;
   a.U1 = nullptr;
+  return a;
+}
+
+// One forward step src -> dst with the fixed dt (no finalize: the schedule is given).  The
+// fallback passes are launched only when `passes` is set, i.e. when the step is known (or
+// not yet known) to tag cells; a step that tagged none recomputes identically without them.
+template <typename T>
+cudaError_t forward_step(msh_grid *g, Ctrl *ctl, Partial *part, T *src, T *dst, int64_t step, double dt,
+                         bool passes) {
+  adj_setup_kernel<<<1, 1, 0, g->stream>>>(ctl, step, dt);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  StepArgs<T> a = forward_args<T>(g, ctl, part);
+  a.U[step & 1] = src;
+  a.U[(step + 1) & 1] = dst;
   for (int level = 0; level <= (passes ? kFallbackPasses : 0); level++) {
     a.level = level;
     e = launch_step<T>(a, g->ndim, g->rows, level > 0, g->stream, nullptr);
@@ -528,12 +536,19 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
   const int64_t seg_len = std::min<int64_t>(K, std::max<int64_t>(nsteps, 1));
   size_t Npad = 1;
   for (int d = 0; d < 3; d++) Npad *= (size_t)(g->n[d] + (d < g->ndim ? 4 : 0));
+  // partials of the recomputed steps (the streaming kernels' or a staged launch's blocks)
   const int nb = std::max(step_blocks<T>(g->ndim, g->rows, (int)g->n[0], (int)g->n[1], (int)g->n[2], g->zchunk),
-                          1);
+                          kStagedMaxBlocks);
   T *seg = nullptr, *la = nullptr, *lb = nullptr, *scratch = nullptr;
   T *Wb = nullptr;
   Ctrl *ctl = nullptr;
   Partial *part = nullptr;
+  double *dts_d = nullptr;
+  const bool staged = nsteps > 0 && use_staged(g);
+  if (staged) {
+    A_TRY(cudaMalloc(&dts_d, sizeof(double) * (size_t)nsteps));
+    A_TRY(cudaMemcpyAsync(dts_d, dts, sizeof(double) * (size_t)nsteps, cudaMemcpyHostToDevice, g->stream));
+  }
   A_TRY(cudaMalloc(&seg, S * (size_t)seg_len));
   A_TRY(cudaMalloc(&la, S));
   A_TRY(cudaMalloc(&lb, S));
@@ -545,9 +560,11 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
   A_TRY(cudaMemcpyAsync(la, lamN, S, in_kind, g->stream));
   for (int64_t sg = nck - 1; sg >= 0; sg--) {
     const int64_t n0 = sg * K, n1 = std::min<int64_t>(n0 + K, nsteps);
-    // recompute the segment's states U^{n0} .. U^{n1-1}
+    // recompute the segment's states U^{n0} .. U^{n1-1}: in one staged launch, or step by step
     A_TRY(cudaMemcpyAsync(seg, ck + (size_t)sg * N * NV, S, cudaMemcpyDeviceToDevice, g->stream));
-    for (int64_t n = n0; n + 1 < n1; n++)
+    if (staged && n1 - n0 > 1)
+      A_TRY(staged_segment<T>(g, forward_args<T>(g, ctl, part), seg, dts_d + n0, n0, (int)(n1 - n0 - 1), nullptr));
+    for (int64_t n = n0; !staged && n + 1 < n1; n++)
       A_TRY(forward_step<T>(g, ctl, part, seg + (size_t)(n - n0) * N * NV, seg + (size_t)(n - n0 + 1) * N * NV, n,
                             dts[n], had[n] != 0));
     for (int64_t n = n1 - 1; n >= n0; n--) {
@@ -599,7 +616,8 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
   A_TRY(cudaStreamSynchronize(g->stream));
 done:
   cudaStreamSynchronize(g->stream);
-  for (void *p : {(void *)seg, (void *)la, (void *)lb, (void *)scratch, (void *)Wb, (void *)ctl, (void *)part})
+  for (void *p : {(void *)seg, (void *)la, (void *)lb, (void *)scratch, (void *)Wb, (void *)ctl, (void *)part,
+                  (void *)dts_d})
     if (p) cudaFree(p);
   return st;
 }
@@ -614,16 +632,25 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
   const size_t S = N * NV * sizeof(T);
   const cudaMemcpyKind in_kind = where == MSH_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const int64_t nck = nsteps > 0 ? (nsteps + K - 1) / K : 1;
+  // partials of the recomputed steps (the streaming kernels' or a staged launch's blocks)
   const int nb = std::max(step_blocks<T>(g->ndim, g->rows, (int)g->n[0], (int)g->n[1], (int)g->n[2], g->zchunk),
-                          1);
+                          kStagedMaxBlocks);
   T *ck = nullptr, *bufA = nullptr, *bufB = nullptr, *W0 = nullptr;
+  double *dts_d = nullptr;
   Ctrl *ctl = nullptr;
   Partial *part = nullptr;
   int32_t *had = nullptr;
   std::vector<int32_t> had_h((size_t)std::max<int64_t>(nsteps, 1), 0);
+  const bool staged = nsteps > 0 && use_staged(g);
   A_TRY(cudaMalloc(&ck, S * nck));
-  A_TRY(cudaMalloc(&bufA, S));
-  A_TRY(cudaMalloc(&bufB, S));
+  if (staged) {  // the states of one segment and the schedule
+    A_TRY(cudaMalloc(&bufA, S * (size_t)(std::min<int64_t>(K, nsteps) + 1)));
+    A_TRY(cudaMalloc(&dts_d, sizeof(double) * (size_t)nsteps));
+    A_TRY(cudaMemcpyAsync(dts_d, dts, sizeof(double) * (size_t)nsteps, cudaMemcpyHostToDevice, g->stream));
+  } else {
+    A_TRY(cudaMalloc(&bufA, S));
+    A_TRY(cudaMalloc(&bufB, S));
+  }
   A_TRY(cudaMalloc(&ctl, sizeof(Ctrl)));
   A_TRY(cudaMalloc(&part, sizeof(Partial) * (size_t)nb));
   A_TRY(cudaMalloc(&had, sizeof(int32_t) * had_h.size()));
@@ -636,7 +663,16 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
     A_TRY(cudaMemcpyAsync(W0, ck, S, cudaMemcpyDeviceToDevice, g->stream));
     A_TRY(launch_convert<T>(ck, N, 0, g->stream));
   }
-  {
+  if (staged) {
+    for (int64_t s = 0; s < nsteps; s += K) {  // segment by segment; its last state is the next checkpoint
+      const int len = (int)std::min<int64_t>(K, nsteps - s);
+      A_TRY(cudaMemcpyAsync(bufA, ck + (size_t)(s / K) * N * NV, S, cudaMemcpyDeviceToDevice, g->stream));
+      A_TRY(staged_segment<T>(g, forward_args<T>(g, ctl, part), bufA, dts_d + s, s, len, had + s));
+      if (s + K < nsteps)
+        A_TRY(cudaMemcpyAsync(ck + (size_t)(s / K + 1) * N * NV, bufA + (size_t)len * N * NV, S,
+                              cudaMemcpyDeviceToDevice, g->stream));
+    }
+  } else {
     const T *cur = ck;
     for (int64_t s = 0; s < nsteps; s++) {
       T *dst = (s & 1) ? bufB : bufA;
@@ -653,12 +689,15 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
   A_TRY(cudaStreamSynchronize(g->stream));
   cudaFree(bufA);
   cudaFree(bufB);
+  cudaFree(dts_d);
   bufA = bufB = nullptr;
+  dts_d = nullptr;
   st = reverse_sweep<T>(g, ck, nsteps, dts, had_h.data(), K, lamN, lam0, where, W0);
 done:
   cudaMemsetAsync(g->flags, 0, N * sizeof(int32_t), g->stream);
   cudaStreamSynchronize(g->stream);
-  for (void *p : {(void *)ck, (void *)bufA, (void *)bufB, (void *)W0, (void *)ctl, (void *)part, (void *)had})
+  for (void *p : {(void *)ck, (void *)bufA, (void *)bufB, (void *)dts_d, (void *)W0, (void *)ctl, (void *)part,
+                  (void *)had})
     if (p) cudaFree(p);
   return st;
 }

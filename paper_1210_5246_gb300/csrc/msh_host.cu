@@ -178,9 +178,10 @@ bool staged_wanted(const msh_grid *g) {
   return g->N <= kStagedMaxCells32[g->ndim - 1];
 }
 
-// Whether the staged step takes this grid's steps; allocates its buffers at the first use.
-// Where they do not fit, the streaming kernels go on.
-bool use_staged(msh_grid *g) {
+}  // namespace
+
+// Where the buffers do not fit, the streaming kernels go on.
+bool msh::use_staged(msh_grid *g) {
   if (!staged_wanted(g)) return false;
   if (g->stg_mem) return true;
   const StagedLayout l(g);
@@ -200,6 +201,8 @@ bool use_staged(msh_grid *g) {
   }
   return true;
 }
+
+namespace {
 
 template <typename T> StagedArgs<T> make_staged(msh_grid *g, const StepArgs<T> &s, int max_iter) {
   const StagedLayout l(g);
@@ -239,6 +242,25 @@ cudaError_t run_staged(msh_grid *g, int max_iter, int phase, int *nblk) {
   a.phase = phase;
   return dispatch_staged<double>(g, a, nblk);
 }
+
+}  // namespace
+
+template <typename T>
+cudaError_t msh::staged_segment(msh_grid *g, const StepArgs<T> &args, T *seg, const double *dts, int64_t step0,
+                                int steps, int32_t *had) {
+  StagedArgs<T> a = make_staged<T>(g, args, steps);
+  a.seg = seg;
+  a.dts = dts;
+  a.seg_step = step0;
+  a.had = had;
+  return dispatch_staged<T>(g, a, nullptr);
+}
+template cudaError_t msh::staged_segment<float>(msh_grid *, const StepArgs<float> &, float *, const double *, int64_t,
+                                                int, int32_t *);
+template cudaError_t msh::staged_segment<double>(msh_grid *, const StepArgs<double> &, double *, const double *,
+                                                 int64_t, int, int32_t *);
+
+namespace {
 
 msh_status launch_one_step(msh_grid *g, int ev_slot) {
   g->phase_level = -1;  // a whole step closes a phased one that was left open

@@ -93,6 +93,7 @@ template <typename T> struct StagedArgs {
   T *seg = nullptr;    // recompute: states seg[0 .. max_iter], seg[0] given
   const double *dts = nullptr;  // their time steps (device)
   int64_t seg_step = 0;         // step number of seg[0] (fallback tags)
+  int32_t *had = nullptr;       // had[i]: whether step i tagged cells (may be null)
 };
 constexpr int kStagedMaxBlocks = 2048;  // blocks of a staged launch at most (partials, counts)
 
@@ -240,6 +241,13 @@ struct msh_grid {
 };
 
 namespace msh {
+// Whether the staged step takes this grid's steps (allocates its buffers at the first use).
+bool use_staged(msh_grid *g);
+// The `steps` states after seg[0], written to seg[1 .. steps] ([NV][N] each, device), with the
+// given time steps (device) by one staged launch; tags carry the step numbers from step0 on.
+template <typename T>
+cudaError_t staged_segment(msh_grid *g, const StepArgs<T> &args, T *seg, const double *dts, int64_t step0, int steps,
+                           int32_t *had);
 // self-gravity (msh_selfgrav.cu): the per-step potential and acceleration, the history
 // flag, plans and buffers
 cudaError_t launch_self_gravity(msh_grid *g, cudaStream_t s);

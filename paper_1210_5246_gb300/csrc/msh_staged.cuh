@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
         st.stop = taken >= a.max_iter;
         if (!st.stop) st.dt = a.dts[taken];
         st.step = step + 1;
+        if (blk == 0 && a.had != nullptr) a.had[taken - 1] = st.any_tagged > 0;
         if (blk == 0 && st.any_tagged > 0)
           for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
       } else {
