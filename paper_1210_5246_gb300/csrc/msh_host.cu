@@ -89,6 +89,14 @@ template <typename T> StepArgs<T> make_args(msh_grid *g) {
   return a;
 }
 
+// The default shape of the streaming kernels, unless msh_set_tiling chose one.
+void default_shape(msh_grid *g) {
+  if (g->tiling_set) return;
+  const Tiling t = default_tiling(g->ndim, g->n, g->prec, g->ctu);
+  g->rows = t.rows;
+  g->zchunk = t.zchunk;
+}
+
 int blocks_for(msh_grid *g, int rows, int zchunk) {
   if (g->prec == MSH_FP32) return step_blocks<float>(g->ndim, rows, (int)g->n[0], (int)g->n[1], (int)g->n[2], zchunk);
   return step_blocks<double>(g->ndim, rows, (int)g->n[0], (int)g->n[1], (int)g->n[2], zchunk);
@@ -517,8 +525,7 @@ msh_status msh_init_grid(msh_grid **out, int32_t ndim, const int64_t n[3], const
   g->esize = precision == MSH_FP32 ? 4 : 8;
   g->cfl = cfl;
   g->N = (size_t)n[0] * n[1] * n[2];
-  g->zchunk = default_chunk(ndim, n);
-  g->rows = 8;
+  default_shape(g);
   auto cleanup = [&](msh_status s) {
     msh_destroy(g);
     return s;
@@ -821,6 +828,7 @@ msh_status msh_set_ctu(msh_grid *g, int32_t on) {
   if ((bool)on == g->ctu) return MSH_OK;
   drop_graph(g);
   g->ctu = on != 0;
+  default_shape(g);
   // the CFL rule changed: plan the next step of the current state again
   if (g->has_state) return prime(g, cur_buf(g));
   return MSH_OK;

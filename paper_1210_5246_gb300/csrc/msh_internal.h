@@ -101,13 +101,13 @@ constexpr int kTile1D = 128;   // threads per block of the 1D step kernel
 constexpr int kTileX = 30;     // interior cells per warp row of the 3D kernel
 constexpr int kStripX = 28;    // updated cells per warp strip of the 2D kernel
 
-// Default length of the chunk a thread block streams: rows (2D); 3D: 0, the balanced
-// tiling (work units of equal plane counts, one per resident block).
-inline int default_chunk(int ndim, const int64_t n[3]) {
-  if (ndim == 3) return 0;
-  if (ndim == 2) return (int)(n[1] < 16 ? n[1] : 16);
-  return 1;
-}
+// Tile shape of the streaming step kernels: thread rows (3D) or warps per block (2D), and the
+// planes or rows streamed per block or warp (0 in 3D: the balanced tiling).
+struct Tiling {
+  int rows, zchunk;
+};
+// The default shape for a grid (msh_step.cu).
+Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu);
 constexpr int kFinalizeThreads = 256;
 
 // launchers (msh_step.cu)

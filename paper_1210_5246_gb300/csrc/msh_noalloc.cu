@@ -80,14 +80,15 @@ msh_status noalloc_step(int ndim, const int64_t n[3], const double dx[3], const 
   a.nz = (int)n[2];
   for (int i = 0; i < 6; i++) a.bc[i] = i < 2 * ndim ? bc[i] : MSH_BC_PERIODIC;
   for (int i = 0; i < 3; i++) a.dx[i] = dx[i];
-  a.zchunk = default_chunk(ndim, n);
   a.level = 0;
   a.ck = nullptr;  // no adjoint tape
   a.ck_base = 0;
   a.ck_len = 0;
   a.ck_K = 1;
   a.U1 = nullptr;
-  const int rows = 8;
+  const Tiling shape = default_tiling(ndim, n, sizeof(T) == 4 ? MSH_FP32 : MSH_FP64, false);
+  const int rows = shape.rows;
+  a.zchunk = shape.zchunk;
   const int nb = step_blocks<T>(ndim, rows, a.nx, a.ny, a.nz, a.zchunk);
   if ((size_t)nb > kNoallocMaxBlocks)
     return set_error_text("msh_step_noalloc: grid needs more thread blocks than the fixed scratch holds"),

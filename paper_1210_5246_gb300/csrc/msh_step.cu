@@ -264,6 +264,87 @@ cudaError_t launch_ensemble_end(const Ctrl *ctrl, int32_t *status, cudaStream_t 
   return cudaGetLastError();
 }
 
+// ----------------------------------------------------------- default tiling
+// Planes a unit of the balanced 3D tiling streams plus p for each of its prologues, at most
+// over the units (the same hand-out as step_tile_kernel).
+static double balanced_cost(long long ncols, long long nz, long long units, double p) {
+  const long long nfull = ncols / units, nrcol = ncols - nfull * units, nrest = nrcol * nz;
+  const long long wz = std::max<long long>(1, (nrest + units - 1) / units), nwf = nz / wz, wlast = nz - nwf * wz;
+  double worst = 0.0;
+  for (long long u = 0; u < units; u++) {
+    double cost = (double)nfull * (nz + p);
+    long long rp = nrest * u / units;
+    const long long rend = nrest * (u + 1) / units;
+    while (rp < rend) {
+      const long long inwhole = nrcol * wz * nwf;
+      const long long left = rp < inwhole ? wz - rp % wz : wlast - (rp - inwhole) % wlast;
+      const long long len = std::min(left, rend - rp);
+      cost += (double)len + p;
+      rp += len;
+    }
+    worst = std::max(worst, cost);
+  }
+  return worst;
+}
+
+// The shape with the least estimated time.  The estimates are fits to timed sweeps over grid
+// sizes (step kernel, GB300):
+//   3D FP32  a block of 16 rows takes 5.5 us per plane with one block per SM, one of 8 rows
+//            6.3 us with two per SM (corner transport upwind: 10 us and 6.4 us, one per SM);
+//            a prologue costs as much as 6 planes.  256^3: 16 rows balanced 1.60 ms against
+//            2.14 ms with 8 rows; 160^3: two chunks of 80 planes per column 0.47 ms, balanced
+//            0.70 ms (its last windows are 8 planes long); 48^3 CTU: 8 rows in chunks of 6.
+//   2D FP32  a row of a strip takes 2.7 us while a scheduler has up to two warps, 3.2 us with
+//            three and 3.7 us with four; a chunk's prologue, partial and start cost as much as
+//            3.6 rows.  512^2: 4 rows 28 us, 8 rows 31 us, 16 rows 54 us; 1024^2: 16 rows 73 us.
+//   FP64     the double-precision pipe is the bound: time goes with the warps per scheduler,
+//            a prologue costs about one row or plane.
+Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu) {
+  if (ndim == 1) return {8, 1};
+  const bool f32 = prec == MSH_FP32;
+  const long long sms = device_sms();
+  Tiling best = {8, ndim == 3 ? 0 : 16};
+  double best_cost = 1e300;
+  auto offer = [&](int rows, int zchunk, double cost) {
+    if (cost < 0.995 * best_cost) {  // near ties keep the earlier candidate
+      best_cost = cost;
+      best = {rows, zchunk};
+    }
+  };
+  if (ndim == 2) {
+    const long long strips = (n[0] + kStripX - 1) / kStripX;
+    for (int rows : {8, 4, 16})
+      for (int c = 1; c <= 64 && c <= n[1]; c++) {
+        const long long warps = strips * ((n[1] + c - 1) / c), blocks = (warps + rows - 1) / rows;
+        double cost;
+        if (f32) {
+          const long long slots = sms * (16 / rows), waves = blocks / slots, rest = blocks - waves * slots;
+          const double w = (double)((rest + sms - 1) / sms) * rows / 4.0;  // warps per scheduler, last wave
+          cost = (c + 3.6) * (3.7 * (double)waves + (rest == 0 ? 0.0 : w <= 2.0 ? 2.7 : w <= 3.0 ? 3.2 : 3.7));
+        } else {
+          cost = (c + 1.0) * (double)((blocks + sms - 1) / sms) * rows / 4.0;
+        }
+        offer(rows, c, cost);
+      }
+    return best;
+  }
+  const double p = f32 ? 6.0 : 1.0;
+  const long long tilesx = (n[0] + kTileX - 1) / kTileX;
+  for (int rows : {16, 8}) {
+    if (rows == 16 && !f32) continue;
+    const long long slots = rows == 8 && f32 && !ctu ? 2 * sms : sms;
+    const double plane = !f32 ? 1.0 : ctu ? (rows == 16 ? 10.0 : 6.4) : (rows == 16 ? 5.5 : 6.3);
+    const long long ncols = tilesx * ((n[1] + rows - 3) / (rows - 2));
+    const long long units = std::max<long long>(1, std::min<long long>(slots, ncols * n[2] / kMinUnitPlanes));
+    offer(rows, 0, plane * balanced_cost(ncols, n[2], units, p));
+    for (long long m = 1; m <= 64 && m <= n[2]; m++) {
+      const long long z = (n[2] + m - 1) / m, u = ncols * ((n[2] + z - 1) / z);
+      offer(rows, (int)z, plane * (double)((u + slots - 1) / slots) * ((double)z + p));
+    }
+  }
+  return best;
+}
+
 // ------------------------------------------------------------- conversions
 template <typename T>
 __global__ void convert_kernel(T *U, size_t N, int to_primitive) {
