@@ -57,8 +57,14 @@ constexpr int kGraphSteps = 16;
 constexpr int kStagedSteps = 64;  // steps of one staged launch at most
 // the staged step's buffers (2 + 2 ndim states) stay below this; larger grids stream
 constexpr size_t kStagedMaxBytes = size_t(2) << 30;
-// FP32 grids of up to this many cells (1D, 2D, 3D) take the staged step
-constexpr size_t kStagedMaxCells32[3] = {size_t(1) << 24, 400000, 600000};
+// FP32 grids of up to this many cells (1D, 2D, 3D) may take the staged step (beyond, its face
+// states leave L2); in 2D and 3D where its estimated time is the shorter one.  Fits to timed
+// steps: staged 2D 13.7 us + 0.97e-4 us per cell (64^2 13.7, 256^2 20.1, 512^2 39), 3D 14.7 us +
+// 2e-4 us per cell (32^3 21, 64^3 67, 97x61x45 72); a streaming step adds 8 us of launches to its
+// kernel (256^2 27.7 us, 512^2 38, 64^3 74, 97x61x45 73.5).
+constexpr size_t kStagedMaxCells32[3] = {size_t(1) << 24, 400000, 400000};
+constexpr double kStagedBase[3] = {0.0, 13.7, 14.7}, kStagedPerCell[3] = {0.0, 0.97e-4, 2.0e-4};
+constexpr double kStreamLaunches = 8.0;
 
 }  // namespace
 
@@ -95,6 +101,7 @@ void default_shape(msh_grid *g) {
   const Tiling t = default_tiling(g->ndim, g->n, g->prec, g->ctu);
   g->rows = t.rows;
   g->zchunk = t.zchunk;
+  g->tile_us = t.us;
 }
 
 int blocks_for(msh_grid *g, int rows, int zchunk) {
@@ -183,7 +190,9 @@ bool staged_wanted(const msh_grid *g) {
   if (g->ctu || g->tiling_set || g->stg_off) return false;
   if (StagedLayout(g).bytes > kStagedMaxBytes) return false;
   if (g->prec == MSH_FP64) return true;
-  return g->N <= kStagedMaxCells32[g->ndim - 1];
+  const int d = g->ndim - 1;
+  if (g->N > kStagedMaxCells32[d]) return false;
+  return d == 0 || kStagedBase[d] + kStagedPerCell[d] * (double)g->N < kStreamLaunches + g->tile_us;
 }
 
 }  // namespace

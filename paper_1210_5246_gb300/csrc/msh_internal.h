@@ -105,6 +105,7 @@ constexpr int kStripX = 28;    // updated cells per warp strip of the 2D kernel
 // planes or rows streamed per block or warp (0 in 3D: the balanced tiling).
 struct Tiling {
   int rows, zchunk;
+  double us;  // estimated time of a step's kernel (FP32)
 };
 // The default shape for a grid (msh_step.cu).
 Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu);
@@ -224,6 +225,7 @@ struct msh_grid {
   // that uses it; stg_off: the allocation failed, the streaming kernels step the grid
   void *stg_mem = nullptr;
   bool stg_off = false;
+  double tile_us = 0.0;  // estimated step time of the streaming kernels' default shape
   cudaGraphExec_t graph = nullptr;
   // profiling: eager launches with events around every step-kernel launch
   bool profiling = false;

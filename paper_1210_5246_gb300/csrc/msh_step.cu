@@ -300,20 +300,20 @@ static double balanced_cost(long long ncols, long long nz, long long units, doub
 //   FP64     the double-precision pipe is the bound: time goes with the warps per scheduler,
 //            a prologue costs about one row or plane.
 Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu) {
-  if (ndim == 1) return {8, 1};
+  if (ndim == 1) return {8, 1, 0.0};
   const bool f32 = prec == MSH_FP32;
   const long long sms = device_sms();
-  Tiling best = {8, ndim == 3 ? 0 : 16};
+  Tiling best = {8, ndim == 3 ? 0 : 16, 0.0};
   double best_cost = 1e300;
   auto offer = [&](int rows, int zchunk, double cost) {
     if (cost < 0.995 * best_cost) {  // near ties keep the earlier candidate
       best_cost = cost;
-      best = {rows, zchunk};
+      best = {rows, zchunk, cost};
     }
   };
   if (ndim == 2) {
     const long long strips = (n[0] + kStripX - 1) / kStripX;
-    for (int rows : {8, 4, 16})
+    for (int rows : {16, 8, 4})
       for (int c = 1; c <= 64 && c <= n[1]; c++) {
         const long long warps = strips * ((n[1] + c - 1) / c), blocks = (warps + rows - 1) / rows;
         double cost;
