@@ -544,8 +544,12 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
   Ctrl *ctl = nullptr;
   Partial *part = nullptr;
   double *dts_d = nullptr;
+  T *gwork = nullptr;  // ghost cells' parts of the staged reverse steps
   const bool staged = nsteps > 0 && use_staged(g);
   if (staged) {
+    size_t pencils = 1;
+    for (int d = 0; d < g->ndim; d++) pencils = std::max(pencils, N / (size_t)g->n[d]);
+    A_TRY(cudaMalloc(&gwork, pencils * NV * 4 * (size_t)g->ndim * sizeof(T)));
     A_TRY(cudaMalloc(&dts_d, sizeof(double) * (size_t)nsteps));
     A_TRY(cudaMemcpyAsync(dts_d, dts, sizeof(double) * (size_t)nsteps, cudaMemcpyHostToDevice, g->stream));
   }
@@ -557,6 +561,7 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
   A_TRY(cudaMalloc(&ctl, sizeof(Ctrl)));
   A_TRY(cudaMalloc(&part, sizeof(Partial) * (size_t)nb));
   A_TRY(cudaMemcpyAsync(ctl, g->hctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, g->stream));
+  A_TRY(cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), g->stream));
   A_TRY(cudaMemcpyAsync(la, lamN, S, in_kind, g->stream));
   for (int64_t sg = nck - 1; sg >= 0; sg--) {
     const int64_t n0 = sg * K, n1 = std::min<int64_t>(n0 + K, nsteps);
@@ -567,6 +572,17 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
     for (int64_t n = n0; !staged && n + 1 < n1; n++)
       A_TRY(forward_step<T>(g, ctl, part, seg + (size_t)(n - n0) * N * NV, seg + (size_t)(n - n0 + 1) * N * NV, n,
                             dts[n], had[n] != 0));
+    bool any_tags = false;
+    for (int64_t n = n0; n < n1; n++) any_tags = any_tags || had[n] != 0;
+    if (staged && !any_tags) {  // the segment's reverse steps in one staged launch, lam in place
+      StagedArgs<T> a = staged_args<T>(g, forward_args<T>(g, ctl, part));
+      a.seg = seg;
+      a.dts = dts_d + n0;
+      T *const self[3] = {a.W[1], scratch, Wb};
+      A_TRY(launch_staged_reverse<T>(a, g->ndim, la, self, gwork, gwork + a.max_pencils * NV * 2 * g->ndim, (int)(n1 - n0),
+                                     g->stream));
+      continue;
+    }
     for (int64_t n = n1 - 1; n >= n0; n--) {
       T *Un = seg + (size_t)(n - n0) * N * NV;
       // restore the fallback tags of step n (only a step that tagged cells has any)
@@ -613,11 +629,19 @@ msh_status reverse_sweep(msh_grid *g, const T *ck, int64_t nsteps, const double 
     std::swap(la, lb);
   }
   A_TRY(cudaMemcpyAsync(lam0, la, S, out_kind, g->stream));
-  A_TRY(cudaStreamSynchronize(g->stream));
+  {
+    Ctrl c;
+    A_TRY(cudaMemcpyAsync(&c, ctl, sizeof c, cudaMemcpyDeviceToHost, g->stream));
+    A_TRY(cudaStreamSynchronize(g->stream));
+    if (c.status == MSH_E_TIMEOUT && staged) {
+      st = afail(MSH_E_TIMEOUT, "a staged launch gave up waiting at a grid barrier");
+      goto done;
+    }
+  }
 done:
   cudaStreamSynchronize(g->stream);
   for (void *p : {(void *)seg, (void *)la, (void *)lb, (void *)scratch, (void *)Wb, (void *)ctl, (void *)part,
-                  (void *)dts_d})
+                  (void *)dts_d, (void *)gwork})
     if (p) cudaFree(p);
   return st;
 }
@@ -640,6 +664,7 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
   Ctrl *ctl = nullptr;
   Partial *part = nullptr;
   int32_t *had = nullptr;
+  int32_t fwd_status = 0;
   std::vector<int32_t> had_h((size_t)std::max<int64_t>(nsteps, 1), 0);
   const bool staged = nsteps > 0 && use_staged(g);
   A_TRY(cudaMalloc(&ck, S * nck));
@@ -655,6 +680,7 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
   A_TRY(cudaMalloc(&part, sizeof(Partial) * (size_t)nb));
   A_TRY(cudaMalloc(&had, sizeof(int32_t) * had_h.size()));
   A_TRY(cudaMemcpyAsync(ctl, g->hctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, g->stream));
+  A_TRY(cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), g->stream));
   // fallback tags are step numbers: start from a clean slate (and leave one behind)
   A_TRY(cudaMemsetAsync(g->flags, 0, N * sizeof(int32_t), g->stream));
   A_TRY(cudaMemcpyAsync(ck, U0, S, in_kind, g->stream));
@@ -686,7 +712,12 @@ msh_status adjoint_impl(msh_grid *g, const void *U0, int64_t nsteps, const doubl
   }
   if (nsteps > 0)
     A_TRY(cudaMemcpyAsync(had_h.data(), had, sizeof(int32_t) * (size_t)nsteps, cudaMemcpyDeviceToHost, g->stream));
+  A_TRY(cudaMemcpyAsync(&fwd_status, &ctl->status, sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
   A_TRY(cudaStreamSynchronize(g->stream));
+  if (staged && fwd_status == MSH_E_TIMEOUT) {
+    st = afail(MSH_E_TIMEOUT, "a staged launch gave up waiting at a grid barrier");
+    goto done;
+  }
   cudaFree(bufA);
   cudaFree(bufB);
   cudaFree(dts_d);

@@ -11,7 +11,7 @@ namespace msh {
 // W = W(U): rho, u = m/rho, P = E - m m^T / rho.  Accumulates Ub += (dW/dU)^T Wb.
 template <typename T>
 __device__ __forceinline__ void cons_to_prim_vjp(const T (&U)[NV], const T (&Wb)[NV], T (&Ub)[NV]) {
-  const T ir = T(1) / U[0];
+  const T ir = frcp(U[0]);
   const T u0 = U[1] * ir, u1 = U[2] * ir, u2 = U[3] * ir;
   Ub[0] += Wb[0] - (Wb[1] * u0 + Wb[2] * u1 + Wb[3] * u2) * ir + Wb[4] * u0 * u0 + Wb[5] * u0 * u1 +
            Wb[6] * u0 * u2 + Wb[7] * u1 * u1 + Wb[8] * u1 * u2 + Wb[9] * u2 * u2;
@@ -90,43 +90,50 @@ __device__ __forceinline__ void hll_vjp(const T (&wl)[NV], const T (&wr)[NV], co
   T Ul[NV], Fl[NV], Ur[NV], Fr[NV];
   phys(wl, Ul, Fl);
   phys(wr, Ur, Fr);
-  const T cl = T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
-  const T cr = T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
+  // c = sqrt(3 P / rho) = sqrt(3) P s, s = 1 / sqrt(P rho)
+  const T sl = frsqrt(wl[4] * wl[0]), sr = frsqrt(wr[4] * wr[0]);
+  const T cl = T(1.7320508075688772) * (wl[4] * sl);
+  const T cr = T(1.7320508075688772) * (wr[4] * sr);
   const T aL = wl[1] - cl, aR = wr[1] - cr, bL = wl[1] + cl, bR = wr[1] + cr;
-  const T SL = fmin(aL, aR), SR = fmax(bL, bR);
+  const T SL = min_of(aL, aR), SR = max_of(bL, bR);
   T zero[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) zero[k] = T(0);
-  if (SL >= T(0)) {
+  if (ge0(SL)) {
     phys_vjp(wl, zero, Fb, wlb);
     return;
   }
-  if (SR <= T(0)) {
+  if (ge0(-SR)) {
     phys_vjp(wr, zero, Fb, wrb);
     return;
   }
-  const T inv = T(1) / (SR - SL);
+  // F = (SR Fl - SL Fr + SL SR dU) inv: the speeds' adjoints need three sums over the fields
+  const T inv = frcp(SR - SL);
+  const T ca = SR * inv, cb = -SL * inv, cc = SL * SR * inv;
   T Flb[NV], Frb[NV], Urb[NV], Ulb[NV];
-  T SLb = T(0), SRb = T(0);
+  T X = T(0), Y = T(0), Z = T(0);
 #pragma unroll
   for (int k = 0; k < NV; k++) {
-    const T dU = Ur[k] - Ul[k];
-    const T F = (SR * Fl[k] - SL * Fr[k] + SL * SR * dU) * inv;
-    Flb[k] = SR * inv * Fb[k];
-    Frb[k] = -SL * inv * Fb[k];
-    Urb[k] = SL * SR * inv * Fb[k];
+    X = fma(Fb[k], Fl[k], X);
+    Y = fma(Fb[k], Fr[k], Y);
+    Z = fma(Fb[k], Ur[k] - Ul[k], Z);
+    Flb[k] = ca * Fb[k];
+    Frb[k] = cb * Fb[k];
+    Urb[k] = cc * Fb[k];
     Ulb[k] = -Urb[k];
-    SRb += Fb[k] * ((Fl[k] + SL * dU) * inv - F * inv);
-    SLb += Fb[k] * ((-Fr[k] + SR * dU) * inv + F * inv);
   }
+  const T G = ca * X + cb * Y + cc * Z;  // sum of Fb F
+  const T SRb = inv * (X + SL * Z - G), SLb = inv * (SR * Z - Y + G);
   T clb = T(0), crb = T(0);
-  if (aL <= aR) { wlb[1] += SLb; clb -= SLb; } else { wrb[1] += SLb; crb -= SLb; }
-  if (bL >= bR) { wlb[1] += SRb; clb += SRb; } else { wrb[1] += SRb; crb += SRb; }
-  // c = sqrt(3 P / rho): dc/dP = c / (2P), dc/drho = -c / (2 rho)
-  wlb[4] += clb * cl / (T(2) * wl[4]);
-  wlb[0] -= clb * cl / (T(2) * wl[0]);
-  wrb[4] += crb * cr / (T(2) * wr[4]);
-  wrb[0] -= crb * cr / (T(2) * wr[0]);
+  if (!gt0(aL - aR)) { wlb[1] += SLb; clb -= SLb; } else { wrb[1] += SLb; crb -= SLb; }
+  if (!gt0(bR - bL)) { wlb[1] += SRb; clb += SRb; } else { wrb[1] += SRb; crb += SRb; }
+  // dc/dP = c / (2 P) = (sqrt(3)/2) s,  dc/drho = -c / (2 rho) = -(sqrt(3)/2) s P / rho, where
+  // P / rho = (P s)^2
+  const T hl = T(0.8660254037844386) * sl, hr = T(0.8660254037844386) * sr, ql = wl[4] * sl, qr = wr[4] * sr;
+  wlb[4] += clb * hl;
+  wlb[0] -= clb * hl * (ql * ql);
+  wrb[4] += crb * hr;
+  wrb[0] -= crb * hr * (qr * qr);
   phys_vjp(wl, Ulb, Flb, wlb);
   phys_vjp(wr, Urb, Frb, wrb);
 }
@@ -214,13 +221,14 @@ __device__ __forceinline__ void back_vjp(const Eig<T> &E, const T (&c)[NV], cons
 // Reverse of Eig::init: adds the adjoints of the eigen-quantities into w0b (local frame).
 template <typename T>
 __device__ __forceinline__ void eig_init_vjp(const Eig<T> &E, const EigBar<T> &Eb, T (&w0b)[NV]) {
-  const T q = E.Pxx / E.rho;
-  const T rs = frsqrt(q);
+  const T q = E.cs * E.cs;        // P_xx / rho
+  const T rs = T(2) * E.ics2;     // 1 / cs
+  const T ir = q * E.ip;          // 1 / rho
   const T csb = Eb.cs + T(1.7320508075688772) * Eb.cf;
-  T rsb = T(0.28867513459481287) * Eb.icf2 + T(0.5) * Eb.ics2 + csb * q;
-  T qb = csb * rs - T(0.5) * rsb * rs / q;
-  T Pxxb = Eb.Pxx + qb / E.rho;
-  const T rhob = Eb.rho - qb * q / E.rho;
+  const T rsb = T(0.28867513459481287) * Eb.icf2 + T(0.5) * Eb.ics2 + csb * q;
+  const T qb = csb * rs - T(0.5) * rsb * rs * (rs * rs);
+  T Pxxb = Eb.Pxx + qb * ir;
+  const T rhob = Eb.rho - qb * q * ir;
   const T ipb = Eb.ip + Eb.a * E.Pxy + Eb.b * E.Pxz;
   Pxxb -= ipb * E.ip * E.ip;
   w0b[0] += rhob;
@@ -231,6 +239,28 @@ __device__ __forceinline__ void eig_init_vjp(const Eig<T> &E, const EigBar<T> &E
   w0b[7] += Eb.Pyy;
   w0b[8] += Eb.Pyz;
   w0b[9] += Eb.Pzz;
+}
+
+// Derivatives of the limited amplitude mc(l, r) with its forward selection frozen: 2 on the
+// smaller side, 1/2 on both where the central difference is taken, 0 for differences of
+// opposite sign (ties go to the left side, then to the centre).
+__device__ __forceinline__ void mc_weights(float l, float r, float &fl, float &fr) {
+  const float al = fabsf(l), ar = fabsf(r), c = fabsf(l + r);
+  const bool on = l * r > 0.0f, left = al <= ar, side = left ? 4.0f * al <= c : 4.0f * ar < c;
+  fl = !on ? 0.0f : side ? (left ? 2.0f : 0.0f) : 0.5f;
+  fr = !on ? 0.0f : side ? (left ? 0.0f : 2.0f) : 0.5f;
+}
+__device__ __forceinline__ void mc_weights(double l, double r, double &fl, double &fr) {
+  // on the bit patterns, as mc_limit2
+  constexpr long long kAbs = 0x7fffffffffffffffll, kInf = 0x7ff0000000000000ll;
+  const long long bl = __double_as_longlong(l), br = __double_as_longlong(r), al = bl & kAbs, ar = br & kAbs;
+  const long long c = __double_as_longlong(l + r) & kAbs;
+  const bool left = al <= ar;
+  const long long lo = left ? al : ar, hi = left ? ar : al;
+  const long long q = __double_as_longlong(4.0 * __longlong_as_double(lo));
+  const bool on = (bl ^ br) >= 0 && lo != 0 && hi <= kInf, side = left ? q <= c : q < c;
+  fl = !on ? 0.0 : side ? (left ? 2.0 : 0.0) : 0.5;
+  fr = !on ? 0.0 : side ? (left ? 0.0 : 2.0) : 0.5;
 }
 
 // Reverse of reconstruct() (local frame) plus the a-posteriori first-order overrides
@@ -261,21 +291,17 @@ __device__ __forceinline__ void reconstruct_vjp(const T (&wm)[NV], const T (&w0)
   }
   E.project(dL, cl);
   E.project(dR, cr);
+  mc_limit2_v(cl, cr, m);
 #pragma unroll
-  for (int k = 0; k < NV; k++) m[k] = mc_limit(cl[k], cr[k]);
+  for (int k = 0; k < NV; k++) m[k] *= T(0.5);
   lm[0] = -E.cf * m[0]; lm[1] = -E.cs * m[1]; lm[2] = -E.cs * m[2];
   lm[3] = T(0); lm[4] = T(0); lm[5] = T(0); lm[6] = T(0);
   lm[7] = E.cs * m[7]; lm[8] = E.cs * m[8]; lm[9] = E.cf * m[9];
-  E.back(m, dw);
-  E.back(lm, g);
+  E.back2(m, dw, g);
   {
-    T hi0 = T(0), lo0 = T(0), hi4 = T(0), lo4 = T(0);
-    const T adw0 = E.u * dw[0] + g[0], adw4 = E.u * dw[4] + g[4];
-    hi0 = w0[0] - nu * adw0 + T(0.5) * dw[0];
-    lo0 = w0[0] - nu * adw0 - T(0.5) * dw[0];
-    hi4 = w0[4] - nu * adw4 + T(0.5) * dw[4];
-    lo4 = w0[4] - nu * adw4 - T(0.5) * dw[4];
-    if (!(hi0 > T(0) && lo0 > T(0) && hi4 > T(0) && lo4 > T(0))) {  // face-state fallback: lo = hi = w0
+    const T pr0 = w0[0] - nu * (E.u * dw[0] + g[0]), pr4 = w0[4] - nu * (E.u * dw[4] + g[4]);
+    const T h0 = T(0.5) * dw[0], h4 = T(0.5) * dw[4];
+    if (!(gt0(pr0 + h0) && gt0(pr0 - h0) && gt0(pr4 + h4) && gt0(pr4 - h4))) {  // face-state fallback: lo = hi = w0
 #pragma unroll
       for (int k = 0; k < NV; k++) w0b[k] += lob[k] + hib[k];
       return;
@@ -307,15 +333,10 @@ __device__ __forceinline__ void reconstruct_vjp(const T (&wm)[NV], const T (&w0)
   T clb[NV], crb[NV];
 #pragma unroll
   for (int k = 0; k < NV; k++) {
-    clb[k] = T(0);
-    crb[k] = T(0);
-    const T l = cl[k], r = cr[k];
-    if (l * r > T(0)) {
-      const T al = T(2) * fabs(l), ac = fabs(T(0.5) * (l + r)), ar = T(2) * fabs(r);
-      if (al <= ac && al <= ar) clb[k] = T(2) * mb[k];
-      else if (ac <= ar) { clb[k] = T(0.5) * mb[k]; crb[k] = T(0.5) * mb[k]; }
-      else crb[k] = T(2) * mb[k];
-    }
+    T fl, fr;
+    mc_weights(cl[k], cr[k], fl, fr);
+    clb[k] = fl * mb[k];
+    crb[k] = fr * mb[k];
   }
   T dLb[NV], dRb[NV];
 #pragma unroll

@@ -272,6 +272,11 @@ cudaError_t msh::staged_segment(msh_grid *g, const StepArgs<T> &args, T *seg, co
   a.had = had;
   return dispatch_staged<T>(g, a, nullptr);
 }
+template <typename T> StagedArgs<T> msh::staged_args(msh_grid *g, const StepArgs<T> &args) {
+  return make_staged<T>(g, args, 0);
+}
+template StagedArgs<float> msh::staged_args<float>(msh_grid *, const StepArgs<float> &);
+template StagedArgs<double> msh::staged_args<double>(msh_grid *, const StepArgs<double> &);
 template cudaError_t msh::staged_segment<float>(msh_grid *, const StepArgs<float> &, float *, const double *, int64_t,
                                                 int, int32_t *);
 template cudaError_t msh::staged_segment<double>(msh_grid *, const StepArgs<double> &, double *, const double *,

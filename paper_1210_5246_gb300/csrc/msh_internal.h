@@ -250,6 +250,13 @@ bool use_staged(msh_grid *g);
 template <typename T>
 cudaError_t staged_segment(msh_grid *g, const StepArgs<T> &args, T *seg, const double *dts, int64_t step0, int steps,
                            int32_t *had);
+// The staged arguments of a grid (its buffers) with the given step arguments.
+template <typename T> StagedArgs<T> staged_args(msh_grid *g, const StepArgs<T> &args);
+// Reverse steps of a segment without tagged cells (msh_adj_staged.cu): lam^{n0+len} -> lam^{n0} in
+// place; a.seg and a.dts as for staged_segment; self, gself, gout: work space.
+template <typename T>
+cudaError_t launch_staged_reverse(const StagedArgs<T> &a, int ndim, T *lam, T *const (&self)[3], T *gself, T *gout,
+                                  int len, cudaStream_t s);
 // self-gravity (msh_selfgrav.cu): the per-step potential and acceleration, the history
 // flag, plans and buffers
 cudaError_t launch_self_gravity(msh_grid *g, cudaStream_t s);

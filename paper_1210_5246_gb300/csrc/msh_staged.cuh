@@ -589,9 +589,9 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     __syncthreads();
   }
   if (!alive) {  // a barrier gave up: the result is void
-    if (tid == 0 && a.seg == nullptr) {
+    if (tid == 0) {
       ctrl->status = 5;  // MSH_E_TIMEOUT
-      ctrl->done = 1;
+      if (a.seg == nullptr) ctrl->done = 1;
     }
     grid_leave(a.bar, nblk);
     return;
