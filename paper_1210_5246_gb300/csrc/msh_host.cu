@@ -109,6 +109,12 @@ int blocks_for(msh_grid *g, int rows, int zchunk) {
   return step_blocks<double>(g->ndim, rows, (int)g->n[0], (int)g->n[1], (int)g->n[2], zchunk);
 }
 
+msh_status read_ctrl(msh_grid *g) {
+  CUDA_TRY(cudaMemcpyAsync(g->hctrl, g->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, g->stream));
+  CUDA_TRY(cudaStreamSynchronize(g->stream));
+  return MSH_OK;
+}
+
 msh_status ensure_partials(msh_grid *g, int need) {
   if (need <= g->part_cap) return MSH_OK;
   if (g->part) cudaFree(g->part);
@@ -342,6 +348,38 @@ msh_status launch_one_step(msh_grid *g, int ev_slot) {
   return MSH_OK;
 }
 
+// One whole step whose result the host reads anyway: the streaming characteristic step's
+// fallback passes are launched only if the control block says that cells were tagged (four
+// launches less otherwise).
+msh_status step_and_read(msh_grid *g) {
+  const bool test = g->test_fault == 1 && g->ndim == 3;
+  if (g->scheme == MSH_SCHEME_KT || g->sg_G > 0.0 || test || use_staged(g)) {
+    msh_status st = launch_one_step(g, -1);
+    return st ? st : read_ctrl(g);
+  }
+  g->phase_level = -1;
+  int nb = 0;
+  for (int level = 0; level <= kFallbackPasses; level++) {
+    cudaError_t e;
+    if (g->prec == MSH_FP32) {
+      StepArgs<float> a = make_args<float>(g);
+      a.level = level;
+      e = launch_characteristic(g, a, level > 0, level > 0 ? nullptr : &nb);
+    } else {
+      StepArgs<double> a = make_args<double>(g);
+      a.level = level;
+      e = launch_characteristic(g, a, level > 0, level > 0 ? nullptr : &nb);
+    }
+    if (e != cudaSuccess) return fail(MSH_E_CUDA, "step launch: %s", cudaGetErrorString(e));
+    if (level != 0 && level != kFallbackPasses) continue;
+    e = launch_finalize(g->ctrl, g->part, nb, level == 0 ? 2 : 0, g->stream);
+    if (e != cudaSuccess) return fail(MSH_E_CUDA, "finalize launch: %s", cudaGetErrorString(e));
+    msh_status st = read_ctrl(g);
+    if (st || g->hctrl->nbad[0] == 0) return st;
+  }
+  return MSH_OK;
+}
+
 // n steps in a row (the device control stops them): as few launches as the path allows.
 msh_status launch_steps(msh_grid *g, int64_t n) {
   if (g->sg_G > 0.0 || (g->test_fault == 1 && g->ndim == 3) || !use_staged(g)) {
@@ -388,12 +426,6 @@ msh_status build_graph(msh_grid *g) {
   return MSH_OK;
 }
 
-msh_status read_ctrl(msh_grid *g) {
-  CUDA_TRY(cudaMemcpyAsync(g->hctrl, g->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, g->stream));
-  CUDA_TRY(cudaStreamSynchronize(g->stream));
-  return MSH_OK;
-}
-
 void collect_profile(msh_grid *g, int slots) {
   if (!g->profiling) return;
   for (int i = 0; i < slots; i++) {
@@ -410,21 +442,35 @@ void collect_profile(msh_grid *g, int slots) {
   }
 }
 
-// Scan the buffer `which` and run the finalize kernel in mode 1 (no time advance).
+// One pass over src (launch_scan) into the grid's control block or `ctrl`.
+cudaError_t scan(msh_grid *g, const void *src, void *dst, bool prim, int32_t *flags, Ctrl *ctrl, size_t c0 = 0,
+                 size_t c1 = 0) {
+  const ScanEnd end = {ctrl, &ctrl->scan_count, 0, 0.0, 0.0};
+  if (g->prec == MSH_FP32)
+    return launch_scan<float>((const float *)src, (float *)dst, prim, flags, g->N, g->ndim, g->dx, g->part, end,
+                              g->stream, c0, c1, g->ctu);
+  return launch_scan<double>((const double *)src, (double *)dst, prim, flags, g->N, g->ndim, g->dx, g->part, end,
+                             g->stream, c0, c1, g->ctu);
+}
+
+// CFL step, totals and realizability of the buffer `which` (no time advance).
 msh_status prime(msh_grid *g, int which) {
   msh_status st = ensure_partials(g, kScanBlocks);
   if (st) return st;
-  cudaError_t e;
-  if (g->prec == MSH_FP32)
-    e = launch_scan<float>((const float *)g->U[which], g->N, (int)g->n[0], (int)g->n[1], g->ndim, g->dx, g->part,
-                           kScanBlocks, g->stream, 0, 0, g->ctu);
-  else
-    e = launch_scan<double>((const double *)g->U[which], g->N, (int)g->n[0], (int)g->n[1], g->ndim, g->dx,
-                            g->part, kScanBlocks, g->stream, 0, 0, g->ctu);
+  const cudaError_t e = scan(g, g->U[which], nullptr, false, nullptr, g->ctrl);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "scan launch: %s", cudaGetErrorString(e));
-  e = launch_finalize(g->ctrl, g->part, kScanBlocks, 1, g->stream);
-  if (e != cudaSuccess) return fail(MSH_E_CUDA, "finalize launch: %s", cudaGetErrorString(e));
   return read_ctrl(g);
+}
+
+// Whether p points to memory of the current device that its kernels may read.
+bool device_readable(const void *p) {
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
 int cur_buf(msh_grid *g) { return (int)(g->hctrl->step & 1); }
@@ -624,16 +670,21 @@ msh_status msh_set_state(msh_grid *g, const void *U, int32_t where, int32_t kind
   if (st0) return st0;
   const int cur = cur_buf(g), nxt = cur ^ 1;
   const size_t bytes = g->N * 10 * g->esize;
-  CUDA_TRY(cudaMemcpyAsync(g->U[nxt], U, bytes, where == MSH_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                           g->stream));
-  if (kind == MSH_PRIMITIVE) {
-    cudaError_t e = g->prec == MSH_FP32 ? launch_convert<float>((float *)g->U[nxt], g->N, 0, g->stream)
-                                        : launch_convert<double>((double *)g->U[nxt], g->N, 0, g->stream);
-    if (e != cudaSuccess) return fail(MSH_E_CUDA, "convert: %s", cudaGetErrorString(e));
-  }
-  // fallback tags are step numbers; a new state must not see tags of an earlier trajectory
-  CUDA_TRY(cudaMemsetAsync(g->flags, 0, g->N * sizeof(int32_t), g->stream));
-  msh_status st = prime(g, nxt);
+  // One pass reads the state (a device state in place, a host state after its upload), converts
+  // it, checks it, clears the fallback tags (they are step numbers; a new state must not see
+  // those of an earlier trajectory) and writes it to the spare buffer; if it is realizable the
+  // device copies it on into the current one.
+  const bool direct = where == MSH_DEVICE && device_readable(U);
+  msh_status st = ensure_partials(g, kScanBlocks);
+  if (st) return st;
+  if (!direct)
+    CUDA_TRY(cudaMemcpyAsync(g->U[nxt], U, bytes, where == MSH_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
+                             g->stream));
+  const bool prim = kind == MSH_PRIMITIVE;
+  cudaError_t e = scan(g, direct ? U : g->U[nxt], direct || prim ? g->U[nxt] : nullptr, prim, g->flags, g->ctrl);
+  if (e == cudaSuccess) e = launch_accept(g->ctrl, g->U[nxt], g->U[cur], bytes, g->stream);
+  if (e != cudaSuccess) return fail(MSH_E_CUDA, "state scan: %s", cudaGetErrorString(e));
+  st = read_ctrl(g);
   if (st) return st;
   if (!g->hctrl->realizable) {
     const int64_t bad = g->hctrl->first_bad;
@@ -641,11 +692,6 @@ msh_status msh_set_state(msh_grid *g, const void *U, int32_t where, int32_t kind
     if (g->has_state) prime(g, cur);
     return fail(MSH_E_REALIZABILITY, "state not realizable at cell %lld (rho <= 0 or P not SPD)", (long long)bad);
   }
-  CUDA_TRY(cudaMemcpyAsync(g->U[cur], g->U[nxt], bytes, cudaMemcpyDeviceToDevice, g->stream));
-  // a new state has no previous self-gravity acceleration
-  g->hctrl->sg_hist = 0;
-  CUDA_TRY(cudaMemsetAsync(&g->ctrl->sg_hist, 0, sizeof(int32_t), g->stream));
-  CUDA_TRY(cudaStreamSynchronize(g->stream));
   g->has_state = true;
   return MSH_OK;
 }
@@ -704,19 +750,8 @@ msh_status msh_run_ensemble(msh_grid *g, int64_t count, const void *const *in, v
     CUDA_TRY(cudaEventRecord(ev_in[j], g->ens_in));
     // the steps, on the grid's stream
     CUDA_TRY(cudaStreamWaitEvent(g->stream, ev_in[j], 0));
-    cudaError_t e = cudaSuccess;
-    if (kind == MSH_PRIMITIVE)
-      e = fp32 ? launch_convert<float>((float *)slot, g->N, 0, g->stream)
-               : launch_convert<double>((double *)slot, g->N, 0, g->stream);
-    if (e != cudaSuccess) return fail(MSH_E_CUDA, "convert: %s", cudaGetErrorString(e));
     const int64_t s0 = base + k * nsteps;
-    void *src = g->U[s0 & 1];
-    CUDA_TRY(cudaMemcpyAsync(src, slot, bytes, cudaMemcpyDeviceToDevice, g->stream));
-    e = fp32 ? launch_scan<float>((const float *)src, g->N, (int)g->n[0], (int)g->n[1], g->ndim, g->dx, g->part,
-                                  kScanBlocks, g->stream, 0, 0, g->ctu)
-             : launch_scan<double>((const double *)src, g->N, (int)g->n[0], (int)g->n[1], g->ndim, g->dx, g->part,
-                                   kScanBlocks, g->stream, 0, 0, g->ctu);
-    if (e == cudaSuccess) e = launch_finalize(g->ctrl, g->part, kScanBlocks, 1, g->stream);
+    cudaError_t e = scan(g, slot, g->U[s0 & 1], kind == MSH_PRIMITIVE, nullptr, g->ctrl);
     if (e == cudaSuccess) e = launch_ensemble_start(g->ctrl, s0, nsteps, g->ens_status + k, g->stream);
     if (e != cudaSuccess) return fail(MSH_E_CUDA, "ensemble start: %s", cudaGetErrorString(e));
     st = launch_steps(g, nsteps);
@@ -913,9 +948,7 @@ msh_status msh_step(msh_grid *g, double dt_max, double *dt_taken) {
   if (st) return st;
   cudaError_t e = launch_run_start(g->ctrl, INFINITY, 1, dt_max, g->stream);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "run start: %s", cudaGetErrorString(e));
-  st = launch_one_step(g, -1);
-  if (st) return st;
-  st = read_ctrl(g);
+  st = step_and_read(g);
   if (st) return st;
   if (dt_taken) *dt_taken = g->hctrl->dt_last;
   if (g->hctrl->status == MSH_E_TIMEOUT)
@@ -1122,12 +1155,7 @@ msh_status msh_reduce_layers(msh_grid *g, int64_t start, int64_t count, double t
   CUDA_TRY(cudaMemcpyAsync(g->ctrl_aux, &c, sizeof c, cudaMemcpyHostToDevice, g->stream));
   const size_t c0 = (size_t)start * per, c1 = (size_t)(start + count) * per;
   const int which = cur_buf(g);
-  cudaError_t e = g->prec == MSH_FP32
-                      ? launch_scan<float>((const float *)g->U[which], g->N, (int)g->n[0], (int)g->n[1], g->ndim,
-                                           g->dx, g->part, kScanBlocks, g->stream, c0, c1, g->ctu)
-                      : launch_scan<double>((const double *)g->U[which], g->N, (int)g->n[0], (int)g->n[1], g->ndim,
-                                            g->dx, g->part, kScanBlocks, g->stream, c0, c1, g->ctu);
-  if (e == cudaSuccess) e = launch_finalize(g->ctrl_aux, g->part, kScanBlocks, 1, g->stream);
+  const cudaError_t e = scan(g, g->U[which], nullptr, false, nullptr, g->ctrl_aux, c0, c1);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "layer reduction: %s", cudaGetErrorString(e));
   CUDA_TRY(cudaMemcpyAsync(&c, g->ctrl_aux, sizeof c, cudaMemcpyDeviceToHost, g->stream));
   CUDA_TRY(cudaStreamSynchronize(g->stream));
@@ -1147,9 +1175,7 @@ msh_status msh_step_dt(msh_grid *g, double dt, int32_t *tagged_cells) {
   if (st) return st;
   cudaError_t e = launch_set_dt(g->ctrl, dt, g->stream);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "set dt: %s", cudaGetErrorString(e));
-  st = launch_one_step(g, -1);
-  if (st) return st;
-  st = read_ctrl(g);
+  st = step_and_read(g);
   if (st) return st;
   g->dt_stale = false;  // the finalize planned from the new state
   if (tagged_cells) *tagged_cells = g->hctrl->last_tagged;

@@ -42,6 +42,7 @@ struct Ctrl {
   int64_t tape_base, tape_len;
   int32_t last_tagged;  // cells the a-posteriori fallback tagged in the last step
   int32_t sg_hist;      // self-gravity: the previous step's acceleration is stored
+  unsigned scan_count;  // blocks of a running scan that have written their partial
   int32_t stage_timeout;  // a 3D step kernel's bounded wait for a bulk tensor copy ran out
                           // (the step's result is void; finalize reports MSH_E_TIMEOUT)
 };
@@ -131,11 +132,24 @@ template <typename T> cudaError_t launch_step_kt(const StepArgs<T> &a, int ndim,
 template <typename T, int SCH> cudaError_t launch_staged(const StagedArgs<T> &a, int ndim, cudaStream_t s, int *nblk);
 template <typename T> int step_blocks(int ndim, int rows, int nx, int ny, int nz, int zchunk);
 template <typename T> size_t step_smem(int ndim, int rows, bool ctu, bool retry);
-// partials of cells [c0, c1) (c1 = 0: all N); maxf: the corner-transport-upwind CFL speed
-template <typename T> cudaError_t launch_scan(const T *U, size_t N, int nx, int ny, int ndim,
-                                              const double *dx, Partial *part, int nparts,
-                                              cudaStream_t s, size_t c0 = 0, size_t c1 = 0,
-                                              bool maxf = false);
+// What the last block of a scan does with the partials: the CFL step and totals of the state
+// (kind 0), or (kind 1) a fresh control block for one step with dt <= dt_max (msh_noalloc.cu).
+struct ScanEnd {
+  Ctrl *ctrl;
+  unsigned *count;  // zero between scans
+  int kind;
+  double cfl, dt_max;
+};
+// One pass over cells [c0, c1) (c1 = 0: all N) of src: conversion of a primitive state (prim),
+// copy to dst (nullptr: none), fallback tags cleared (flags, nullptr: kept), signal speed,
+// totals and realizability; maxf: the corner-transport-upwind CFL speed.
+template <typename T>
+cudaError_t launch_scan(const T *src, T *dst, bool prim, int32_t *flags, size_t N, int ndim, const double *dx,
+                        Partial *part, const ScanEnd &end, cudaStream_t s, size_t c0 = 0, size_t c1 = 0,
+                        bool maxf = false);
+// copy `bytes` (a multiple of 8) from src to dst if the scan found the state realizable; a new
+// state has no previous self-gravity acceleration
+cudaError_t launch_accept(Ctrl *ctrl, const void *src, void *dst, size_t bytes, cudaStream_t s);
 cudaError_t launch_set_dt(Ctrl *ctrl, double dt, cudaStream_t s);
 // phased steps of slabs that share the a-posteriori fallback (msh_step_begin / _retry / _end)
 cudaError_t launch_force_pass(Ctrl *ctrl, int level, cudaStream_t s);

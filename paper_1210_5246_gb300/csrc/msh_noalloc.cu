@@ -26,7 +26,7 @@ constexpr size_t kNoallocMaxBlocks = 16384;           // per-block reduction par
 constexpr size_t kNoallocCtrlBytes = 512;
 constexpr size_t kNoallocBytes =
     kNoallocCtrlBytes + kNoallocMaxBlocks * sizeof(Partial) + kNoallocMaxCells * sizeof(int32_t);
-static_assert(sizeof(Ctrl) <= kNoallocCtrlBytes, "control block does not fit its slot");
+static_assert(sizeof(Ctrl) <= kNoallocCtrlBytes - 16, "control block and scan counter do not fit their slot");
 static_assert(sizeof(Partial) % 8 == 0, "partials must keep 8-byte alignment");
 
 // The scratch memory.  In host code this name is only a host-side stand-in: the device
@@ -38,27 +38,6 @@ constexpr int kMaxDevices = 64;
 // device address of g_noalloc_scratch per device; two host threads making the first call on
 // a device at once both store the same address
 std::atomic<void *> g_scratch_addr[kMaxDevices] = {};
-
-// Start the step after the scan of U_in: a non-realizable input (rho <= 0 or P not positive
-// definite in some cell; the scan's finalize has set ctrl->realizable and first_bad) is not
-// stepped: the step kernels see done = 1 and return, U_out is not written, and the status is
-// MSH_E_REALIZABILITY.  Otherwise the step is planned as a one-step run with dt <= dt_max.
-__global__ void noalloc_start_kernel(Ctrl *c, double dt_max) {
-  if (!c->realizable) {
-    c->done = 1;
-    c->status = MSH_E_REALIZABILITY;
-    return;
-  }
-  c->t_end = INFINITY;
-  c->max_step = c->step + 1;
-  c->dt_max = dt_max;
-  c->done = 0;
-  c->status = 0;
-  double dt = c->dt_cfl;
-  if (dt > dt_max) dt = dt_max;
-  c->dt = dt;
-  c->t_next = c->t + dt;
-}
 
 template <typename T>
 msh_status noalloc_step(int ndim, const int64_t n[3], const double dx[3], const int32_t bc[6], double cfl,
@@ -93,31 +72,26 @@ msh_status noalloc_step(int ndim, const int64_t n[3], const double dx[3], const 
   if ((size_t)nb > kNoallocMaxBlocks)
     return set_error_text("msh_step_noalloc: grid needs more thread blocks than the fixed scratch holds"),
            MSH_E_INVALID_ARG;
-  // clear the control block and the tags of these cells (the array keeps the last call's data)
-  Ctrl init;
-  memset(&init, 0, sizeof init);
-  init.cfl = cfl;
-  init.t_end = INFINITY;
-  init.dt_max = INFINITY;
-  init.done = 1;
-  init.first_bad = -1;
-  cudaError_t e = cudaMemcpyAsync(ctrl, &init, sizeof init, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, N * sizeof(int32_t), s);
-  // CFL dt of the input state, then one step with dt = min(CFL dt, dt_max)
-  if (e == cudaSuccess) e = launch_scan<T>(Uin, N, a.nx, a.ny, ndim, dx, part, kScanBlocks, s);
-  if (e == cudaSuccess) e = launch_finalize(ctrl, part, kScanBlocks, 1, s);
-  if (e == cudaSuccess) {
-    noalloc_start_kernel<<<1, 1, 0, s>>>(ctrl, dt_max);
-    e = cudaGetLastError();
-  }
-  for (int level = 0; e == cudaSuccess && level <= kFallbackPasses; level++) {
-    a.level = level;
-    e = launch_step<T>(a, ndim, rows, level > 0, s, nullptr);
-  }
-  if (e == cudaSuccess) e = launch_finalize(ctrl, part, nb, 0, s);
+  // One scan of the input clears the tags of these cells (the array keeps the last call's
+  // data), sets up the control block and plans the step with dt = min(CFL dt, dt_max); a
+  // non-realizable input leaves done = 1 and nothing is stepped.  The step and its finalize
+  // follow; the fallback passes only if the host reads that cells were tagged.
+  const ScanEnd end = {ctrl, reinterpret_cast<unsigned *>(base + kNoallocCtrlBytes - 16), 1, cfl, dt_max};
   Ctrl out;
+  cudaError_t e = launch_scan<T>(Uin, nullptr, false, flags, N, ndim, dx, part, end, s);
+  if (e == cudaSuccess) e = launch_step<T>(a, ndim, rows, false, s, nullptr);
+  if (e == cudaSuccess) e = launch_finalize(ctrl, part, nb, 2, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&out, ctrl, sizeof out, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess && out.done == 0) {  // cells were tagged: the finalize waited
+    for (int level = 1; e == cudaSuccess && level <= kFallbackPasses; level++) {
+      a.level = level;
+      e = launch_step<T>(a, ndim, rows, true, s, nullptr);
+    }
+    if (e == cudaSuccess) e = launch_finalize(ctrl, part, nb, 0, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&out, ctrl, sizeof out, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
   if (e != cudaSuccess) {
     set_error_text(cudaGetErrorString(e));
     return MSH_E_CUDA;

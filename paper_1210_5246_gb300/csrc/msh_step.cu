@@ -10,31 +10,6 @@
 
 namespace msh {
 
-// ----------------------------------------------------------------- scan kernel
-// Partials (totals, max signal speed sum, first non-realizable cell) of the cells
-// [c0, c1) of a state whose fields are N apart.  MAXF: the corner-transport-upwind speed
-// (the maximum over the dims instead of the sum).
-template <typename T, int NDIM, bool MAXF>
-__global__ void __launch_bounds__(256) scan_kernel(const T *__restrict__ U, size_t N, size_t c0, size_t c1, T idx,
-                                                   T idy, T idz, Partial *part) {
-  double diag[NV];
-#pragma unroll
-  for (int k = 0; k < NV; k++) diag[k] = 0.0;
-  T smax = T(0);
-  long long bad = LLONG_MAX;
-  for (size_t c = c0 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < c1; c += (size_t)gridDim.x * blockDim.x) {
-    T Uc[NV], W[NV];
-#pragma unroll
-    for (int k = 0; k < NV; k++) Uc[k] = U[k * N + c];
-    cons_to_prim(Uc, W);
-    if (!realizable(W)) bad = min(bad, (long long)c);
-    smax = max_nonneg(smax, speed_sum<T, NDIM, MAXF>(W, idx, idy, idz));
-#pragma unroll
-    for (int k = 0; k < NV; k++) diag[k] += (double)Uc[k];
-  }
-  block_partial<256>(diag, (double)smax, bad, part + blockIdx.x);
-}
-
 // Acceleration a = -grad Phi by central differences from the potential with one ghost
 // layer, stored [3][N] in the state's precision.
 template <typename T>
@@ -70,10 +45,9 @@ __device__ void plan(Ctrl *c) {
 }
 
 // mode 0: after a step (advance time, record dt, stop on a non-realizable cell, plan the
-// next step); mode 1: after set_state (CFL dt and totals of the state only).
-__global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, const Partial *part,
-                                                                    int nparts, int mode) {
-  if (mode == 0 && ctrl->done) return;
+// next step); mode 1: after set_state (CFL dt and totals of the state only).  Run by one block
+// of kFinalizeThreads threads.
+__device__ void finalize_block(Ctrl *ctrl, const Partial *part, int nparts, int mode) {
   constexpr int kWarps = kFinalizeThreads / 32;
   __shared__ double sd[kWarps][NV + 1], stot[NV];
   __shared__ long long sb[kWarps];
@@ -143,6 +117,101 @@ __global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, 
     return;
   }
   plan(c);
+}
+
+// mode 2: mode 0 unless the step tagged cells (the host then runs the fallback passes and mode 0)
+__global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, const Partial *part, int nparts,
+                                                                    int mode) {
+  if (mode != 1 && ctrl->done) return;
+  if (mode == 2 && ctrl->nbad[0] != 0 && !ctrl->stage_timeout) return;
+  finalize_block(ctrl, part, nparts, mode == 1 ? 1 : 0);
+}
+
+// ----------------------------------------------------------------- scan kernel
+// One pass over the cells [c0, c1) of a state whose fields are N apart (see launch_scan); every
+// block writes its partial, and the last one to finish (a counter) finalizes, which spares a
+// launch.  MAXF: the corner-transport-upwind speed (the maximum over the dims instead of the
+// sum).  Bound by the FP64 sums of the totals (ten conversions and additions per cell), not by
+// the copy: the grid has one block per 256 cells up to four per SM.
+template <typename T, int NDIM, bool MAXF>
+__global__ void __launch_bounds__(kFinalizeThreads) scan_kernel(const T *src, T *dst, int prim, int32_t *flags,
+                                                                size_t N, size_t c0, size_t c1, T idx, T idy, T idz,
+                                                                Partial *part, ScanEnd end) {
+  double diag[NV];
+#pragma unroll
+  for (int k = 0; k < NV; k++) diag[k] = 0.0;
+  T smax = T(0);
+  long long bad = LLONG_MAX;
+  for (size_t c = c0 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < c1; c += (size_t)gridDim.x * blockDim.x) {
+    T Uc[NV], W[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) Uc[k] = src[k * N + c];
+    if (prim) {
+#pragma unroll
+      for (int k = 0; k < NV; k++) W[k] = Uc[k];
+      prim_to_cons(W, Uc);
+    }
+    if (dst != nullptr) {
+#pragma unroll
+      for (int k = 0; k < NV; k++) dst[k * N + c] = Uc[k];
+    }
+    if (flags != nullptr) flags[c] = 0;
+    cons_to_prim(Uc, W);
+    if (!realizable(W)) bad = min(bad, (long long)c);
+    smax = max_nonneg(smax, speed_sum<T, NDIM, MAXF>(W, idx, idy, idz));
+#pragma unroll
+    for (int k = 0; k < NV; k++) diag[k] += (double)Uc[k];
+  }
+  block_partial<kFinalizeThreads>(diag, (double)smax, bad, part + blockIdx.x);
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(end.count, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  Ctrl *ctrl = end.ctrl;
+  if (threadIdx.x == 0) {
+    *end.count = 0u;
+    if (end.kind == 1) {
+      Ctrl c = {};
+      c.cfl = end.cfl;
+      c.t_end = INFINITY;
+      c.dt_max = INFINITY;
+      c.done = 1;
+      c.first_bad = -1;
+      *ctrl = c;
+    }
+  }
+  __syncthreads();
+  finalize_block(ctrl, part, (int)gridDim.x, 1);
+  if (end.kind == 1 && threadIdx.x == 0) {
+    if (!ctrl->realizable) {  // a non-realizable input is not stepped
+      ctrl->status = MSH_E_REALIZABILITY;
+    } else {
+      ctrl->max_step = 1;
+      ctrl->dt_max = end.dt_max;
+      ctrl->done = 0;
+      double dt = ctrl->dt_cfl;
+      if (dt > end.dt_max) dt = end.dt_max;
+      ctrl->dt = dt;
+      ctrl->t_next = dt;
+    }
+  }
+}
+
+__global__ void accept_kernel(Ctrl *ctrl, const uint2 *src, uint2 *dst, size_t n) {
+  if (!ctrl->realizable) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->sg_hist = 0;
+  if (n % 2 == 0) {
+    const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
+    uint4 *d4 = reinterpret_cast<uint4 *>(dst);
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x)
+      d4[i] = s4[i];
+  } else {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+      dst[i] = src[i];
+  }
 }
 
 // One step with a given dt: no CFL limit, no end time.
@@ -366,15 +435,25 @@ cudaError_t launch_step(const StepArgs<T> &a, int ndim, int rows, bool retry, cu
 }
 
 template <typename T>
-cudaError_t launch_scan(const T *U, size_t N, int nx, int ny, int ndim, const double *dx, Partial *part,
-                        int nparts, cudaStream_t s, size_t c0, size_t c1, bool maxf) {
+cudaError_t launch_scan(const T *src, T *dst, bool prim, int32_t *flags, size_t N, int ndim, const double *dx,
+                        Partial *part, const ScanEnd &end, cudaStream_t s, size_t c0, size_t c1, bool maxf) {
+  static_assert(kFinalizeThreads == 256, "scan blocks finalize");
   const T ix = (T)(1.0 / dx[0]), iy = (T)(1.0 / dx[1]), iz = (T)(1.0 / dx[2]);
   if (c1 == 0) c1 = N;
-  if (ndim == 1) scan_kernel<T, 1, false><<<nparts, 256, 0, s>>>(U, N, c0, c1, ix, iy, iz, part);
-  else if (ndim == 2 && maxf) scan_kernel<T, 2, true><<<nparts, 256, 0, s>>>(U, N, c0, c1, ix, iy, iz, part);
-  else if (ndim == 2) scan_kernel<T, 2, false><<<nparts, 256, 0, s>>>(U, N, c0, c1, ix, iy, iz, part);
-  else if (maxf) scan_kernel<T, 3, true><<<nparts, 256, 0, s>>>(U, N, c0, c1, ix, iy, iz, part);
-  else scan_kernel<T, 3, false><<<nparts, 256, 0, s>>>(U, N, c0, c1, ix, iy, iz, part);
+  const int nb = (int)std::max<size_t>(1, std::min<size_t>((c1 - c0 + 255) / 256, (size_t)kScanBlocks)), p = prim;
+  if (ndim == 1) scan_kernel<T, 1, false><<<nb, 256, 0, s>>>(src, dst, p, flags, N, c0, c1, ix, iy, iz, part, end);
+  else if (ndim == 2 && maxf)
+    scan_kernel<T, 2, true><<<nb, 256, 0, s>>>(src, dst, p, flags, N, c0, c1, ix, iy, iz, part, end);
+  else if (ndim == 2) scan_kernel<T, 2, false><<<nb, 256, 0, s>>>(src, dst, p, flags, N, c0, c1, ix, iy, iz, part, end);
+  else if (maxf) scan_kernel<T, 3, true><<<nb, 256, 0, s>>>(src, dst, p, flags, N, c0, c1, ix, iy, iz, part, end);
+  else scan_kernel<T, 3, false><<<nb, 256, 0, s>>>(src, dst, p, flags, N, c0, c1, ix, iy, iz, part, end);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_accept(Ctrl *ctrl, const void *src, void *dst, size_t bytes, cudaStream_t s) {
+  const size_t n = bytes / 8;
+  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((n / 2 + 255) / 256, 8 * (size_t)kScanBlocks));
+  accept_kernel<<<blocks, 256, 0, s>>>(ctrl, static_cast<const uint2 *>(src), static_cast<uint2 *>(dst), n);
   return cudaGetLastError();
 }
 
@@ -410,8 +489,8 @@ template <typename T> cudaError_t launch_convert(T *U, size_t N, int to_primitiv
   template cudaError_t launch_step<T>(const StepArgs<T> &, int, int, bool, cudaStream_t, int *);     \
   template int step_blocks<T>(int, int, int, int, int, int);                                         \
   template size_t step_smem<T>(int, int, bool, bool);                                                    \
-  template cudaError_t launch_scan<T>(const T *, size_t, int, int, int, const double *, Partial *, int, \
-                                      cudaStream_t, size_t, size_t, bool);                           \
+  template cudaError_t launch_scan<T>(const T *, T *, bool, int32_t *, size_t, int, const double *, Partial *, \
+                                      const ScanEnd &, cudaStream_t, size_t, size_t, bool);           \
   template cudaError_t launch_convert<T>(T *, size_t, int, cudaStream_t);                            \
   template cudaError_t launch_gravity_field<T>(const double *, T *, int, int, int, int, const double *, cudaStream_t);
 MSH_INST(float)
