@@ -6,12 +6,17 @@
 // into shared memory and advances it to its own t_end with a block-local CFL reduction;
 // the tube never leaves shared memory until it is finished.  In shared memory a tube is held
 // in primitive variables W, so the reconstruction reads its three cells without
-// conversions; per step the block sweeps the tube in chunks of NT cells: reconstruction of
-// the chunk's cells, HLL fluxes through their lower faces, and the conservative update
-// U^{n+1} = U(W^n) - dt/dx (F_{i+1/2} - F_{i-1/2}) of the cell one behind the chunk front (a
-// cell is updated once both of its faces are known; its W^n is the thread's left neighbour,
-// already in registers), stored as W^{n+1} into the second tube buffer; the buffers swap
-// roles after each step, so W^n stays intact for the fallback passes without a copy.
+// conversions; per step every warp sweeps segments of 30 cells on its own (tube_pass) into
+// the second tube buffer, and the buffers swap roles, so W^n stays intact for the fallback
+// passes without a copy.  A step costs two block barriers; between them one thread plans the
+// time step.  Tubes go to the kernel in up to three classes by length, launched side by side:
+// long tubes need a whole SM's shared memory for their two buffers (16 warps, one block per
+// SM), shorter ones two or four blocks per SM with 8 or 4 warps each, which hide each other's
+// time control and fill the SMs that the long tubes leave.
+// Bound: instruction issue.  4096 tubes of 128 to 2048 cells to t = 0.1 (7.4e8 cell updates):
+// 27.9 ms with one tube per block of 256 threads, three barriers per chunk and every thread
+// planning the time step; 19.6 ms now (14.7 + 3.8 + 1.1 for the three classes one after another),
+// 0.58 instructions per scheduler and cycle.
 // The step is the same as the grid kernels': MUSCL-Hancock on the characteristic
 // variables (Sec. 3.3), HLL flux, outflow boundaries by index clamping, CFL time step
 // dt = C dx / max(|u| + sqrt(3 P_xx/rho)) with the last step clipped to t_end.
@@ -37,13 +42,13 @@ template <typename T> struct TubeArgs {
   const int32_t *len;      // [ntubes]
   const double *t_end;     // [ntubes]
   const int32_t *order;    // [ntubes] processing order (longest first)
-  int32_t *queue;          // work-queue head
+  int32_t *queue;          // work-queue head: tubes order[first + *queue] .. order[last - 1]
+  int32_t first, last;
   int64_t *steps;          // [ntubes] out
   double *t_out;           // [ntubes] out
   int32_t *status;         // [ntubes] out: 0 ok, 4 non-realizable, 5 step cap reached
   int64_t *fallback;       // [ntubes] out: steps whose second-order update tagged cells
   int64_t total;
-  int32_t ntubes;
   int32_t cap;             // shared-memory capacity in cells (>= max len)
   double cfl;
   int64_t max_steps;
@@ -55,34 +60,38 @@ template <typename T> __device__ __forceinline__ void load_w(const T *sW, int ca
   for (int k = 0; k < NV; k++) W[k] = sW[k * cap + cc];
 }
 
-template <typename T, int NT> __device__ __forceinline__ T block_max(T v, T *red) {
+__device__ __forceinline__ float warp_max_speed(float v) {  // v >= 0
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double warp_max_speed(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) red[w] = v;
-  __syncthreads();
-  T m = red[0];
-#pragma unroll
-  for (int i = 1; i < NT / 32; i++) m = fmax(m, red[i]);
-  __syncthreads();
-  return m;
+  for (int o = 16; o > 0; o >>= 1) v = max_of(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
 }
 
-// One sweep of a tube over all its faces: reconstruction, HLL fluxes and the conservative
-// update, chunk by chunk.  src holds W^n; dst receives W^{n+1} (a different buffer).  With FALLBACK, every face that
-// touches a cell tagged by an earlier pass (sFl == 2) takes first-order states.  Cells whose
-// update is not realizable and that carry no active tag are tagged (sFl = 1) and *s_nbad
-// is set.  Returns the thread's maximum signal-speed sum of the new state.
+template <typename T> __device__ __forceinline__ T tube_speed(const T (&W)[NV], T idx) {
+  return (fabs(W[1]) + T(1.7320508075688772) * sqrt_ratio(W[4], W[0])) * idx;
+}
+
+// One sweep of a tube, segment by segment of kTubeSeg cells, the warps of the block taking
+// segments in turn.  Lane l of a warp holds cell first - 1 + l: it reconstructs its cell from
+// shared memory, takes the upper face state of its left neighbour and the flux through its
+// upper face by warp shuffles, and (lanes 1 .. 30) updates its cell into dst, so no warp waits
+// for another within a sweep.  src holds W^n; dst (another buffer) receives W^{n+1}.  With
+// FALLBACK, every face that touches a cell tagged by an earlier pass (sFl == 2) takes
+// first-order states.  Cells whose update is not realizable and that carry no active tag are
+// tagged (sFl = 1) and *s_nbad is set.  Returns the lane's maximum signal speed of the new state.
+constexpr int kTubeSeg = 30;
 template <typename T, int NT, bool FALLBACK>
-__device__ T tube_pass(const T *src, T *dst, unsigned char *sFl, int n, int cap, T nu, T dtdx, T idx, T *sF,
-                       T *sH, T *sHc, int *s_nbad, int *s_any) {
-  const int t = threadIdx.x;
+__device__ __forceinline__ T tube_pass(const T *src, T *dst, unsigned char *sFl, int n, int cap, T nu, T dtdx, T idx,
+                                       int *s_nbad, int *s_any) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   T smax = T(0);
-  for (int b = -1; b <= n; b += NT) {
-    const int c = b + t;
-    T lo[NV], hi[NV], wm[NV];  // wm: W^n of the cell this thread updates (c - 1)
-    if (c <= n) {
-      T w0[NV], wp[NV];
+  for (int b = warp * kTubeSeg; b < n; b += (NT / 32) * kTubeSeg) {
+    const int c = b - 1 + lane;
+    T lo[NV], hi[NV], w0[NV], F[NV];
+    {
+      T wm[NV], wp[NV];
       load_w(src, cap, c - 1, n, wm);
       load_w(src, cap, c, n, w0);
       load_w(src, cap, c + 1, n, wp);
@@ -91,78 +100,63 @@ __device__ T tube_pass(const T *src, T *dst, unsigned char *sFl, int n, int cap,
         auto f = [&](int i) { return sFl[min(max(i, 0), n - 1)] == 2; };
         first_order_faces(f(c - 1), f(c), f(c + 1), w0, lo, hi);
       }
-#pragma unroll
-      for (int v = 0; v < NV; v++) sH[v * NT + t] = hi[v];
     }
-    __syncthreads();
-    if (c >= 0 && c <= n) {
-      T hl[NV], F[NV];
+    {
+      T hl[NV];
 #pragma unroll
-      for (int v = 0; v < NV; v++) hl[v] = (t > 0) ? sH[v * NT + t - 1] : sHc[v];
-      hll(hl, lo, F);
-#pragma unroll
-      for (int v = 0; v < NV; v++) sF[v * (NT + 1) + t + 1] = F[v];
+      for (int v = 0; v < NV; v++) hl[v] = __shfl_up_sync(0xffffffffu, hi[v], 1);
+      hll(hl, lo, F);  // flux through the lower face (lane 0: not used)
     }
-    __syncthreads();
-    // the last thread hands its hi face state to the next chunk (read after the next
-    // barrier; every read of the current carry happened before the barrier above)
-    if (t == NT - 1 && c <= n) {
+    T U[NV], W[NV];
+    prim_to_cons(w0, U);
 #pragma unroll
-      for (int v = 0; v < NV; v++) sHc[v] = hi[v];
-    }
-    const int cu = b - 1 + t;  // cell whose two faces are now known (= c - 1: its W^n is wm)
-    if (cu >= 0 && cu < n) {
-      T U[NV], W[NV];
-      prim_to_cons(wm, U);
-#pragma unroll
-      for (int v = 0; v < NV; v++) U[v] -= dtdx * (sF[v * (NT + 1) + t + 1] - sF[v * (NT + 1) + t]);
+    for (int v = 0; v < NV; v++) U[v] -= dtdx * (__shfl_down_sync(0xffffffffu, F[v], 1) - F[v]);
+    if (lane >= 1 && lane <= kTubeSeg && c < n) {
       cons_to_prim(U, W);
 #pragma unroll
-      for (int v = 0; v < NV; v++) dst[v * cap + cu] = W[v];
+      for (int v = 0; v < NV; v++) dst[v * cap + c] = W[v];
       if (!realizable(W)) {
         *s_any = 1;
-        if (sFl[cu] != 2) {  // newly failing cell: tag it for the next pass
-          sFl[cu] = 1;
+        if (sFl[c] != 2) {  // newly failing cell: tag it for the next pass
+          sFl[c] = 1;
           *s_nbad = 1;
         }
       }
-      smax = fmax(smax, (fabs(W[1]) + T(1.7320508075688772) * sqrt_ratio(W[4], W[0])) * idx);
-    }
-    __syncthreads();
-    if (t == 0) {  // the last face of this chunk is the lower face of the next chunk's first update
-#pragma unroll
-      for (int v = 0; v < NV; v++) sF[v * (NT + 1)] = sF[v * (NT + 1) + NT];
+      smax = fmax(smax, tube_speed(W, idx));
     }
   }
   return smax;
 }
 
+// What the block does next with its tube (thread 0 decides between the passes).
+enum { TUBE_DONE = 0, TUBE_STEP = 1, TUBE_RETRY = 2 };
+
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT) tubes_kernel(TubeArgs<T> a) {
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tubes_kernel(TubeArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cap = a.cap;
   // two tube buffers (primitive): a step reads W^n from one and writes W^{n+1} to the other
   // (the fallback passes re-read the untouched W^n), then the two swap roles
   T *sU = reinterpret_cast<T *>(smem_raw);  // [NV][cap]
   T *sUo = sU + (size_t)NV * cap;           // [NV][cap]
-  T *sF = sUo + (size_t)NV * cap;           // [NV][NT+1]: sF[0] = carried face, sF[t+1] = lower face of cell b+t
-  T *sH = sF + NV * (NT + 1);               // [NV][NT]: hi face states of the chunk
-  T *sHc = sH + NV * NT;                    // [NV]: hi face state of the cell before the chunk
-  unsigned char *sFl = reinterpret_cast<unsigned char *>(sHc + NV);  // [cap] fallback tags
-  __shared__ T red[NT / 32];
-  __shared__ int s_q;
+  unsigned char *sFl = reinterpret_cast<unsigned char *>(sUo + (size_t)NV * cap);  // [cap] fallback tags
+  constexpr int kWarps = NT / 32;
+  __shared__ T red[kWarps];
+  __shared__ T s_dt;
+  __shared__ int s_q, s_act, s_swap, s_clear;
   __shared__ int s_nbad, s_any;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (;;) {
     if (t == 0) s_q = atomicAdd(a.queue, 1);
     __syncthreads();
-    const int q = s_q;
-    __syncthreads();
-    if (q >= a.ntubes) break;
+    const int q = a.first + s_q;
+    if (q >= a.last) break;
     const int k = a.order[q];
     const int n = a.len[k];
     const int64_t off = a.off[k];
     T *cur = sU, *nxt = sUo;  // W^n and W^{n+1} of the current step
+    const T idx = (T)n, half_idx = T(0.5) * idx;
+    T smax = T(0);  // signal speed of the initial state
     for (int c = t; c < n; c += NT) {
       T U[NV], W[NV];
 #pragma unroll
@@ -171,55 +165,88 @@ __global__ void __launch_bounds__(NT) tubes_kernel(TubeArgs<T> a) {
 #pragma unroll
       for (int v = 0; v < NV; v++) cur[v * cap + c] = W[v];
       sFl[c] = 0;
+      smax = fmax(smax, tube_speed(W, idx));
     }
-    __syncthreads();
-    const T idx = (T)n, half_idx = T(0.5) * idx;
-    // signal-speed sum of the initial state
-    T sm = T(0);
-    for (int c = t; c < n; c += NT) {
-      T W[NV];
-      load_w(cur, cap, c, n, W);
-      sm = fmax(sm, (fabs(W[1]) + T(1.7320508075688772) * sqrt_ratio(W[4], W[0])) * idx);
-    }
-    sm = block_max<T, NT>(sm, red);
-    double tt = 0.0;
+    // the time control, in thread 0 alone: its FP64 arithmetic (a division, sums, conversions)
+    // would hold every scheduler's FP64 pipe for each warp that repeats it
+    double tt = 0.0, tn = 0.0;
     const double te = a.t_end[k];
     int64_t steps = 0, fb_steps = 0;
-    int status = 0;
-    while (tt < te) {
-      if (steps >= a.max_steps) { status = 5; break; }
-      double dt = a.cfl / (double)sm;
-      double tn = tt + dt;
-      if (tn >= te) { dt = te - tt; tn = te; }
-      const T nu = (T)dt * half_idx, dtdx = (T)dt * idx;
-      if (t == 0) { s_nbad = 0; s_any = 0; }
+    int status = 0, pass = 0, started = 0;
+    if (t == 0) {
+      s_nbad = 0;
+      s_any = 0;
+    }
+    for (;;) {
+      smax = warp_max_speed(smax);
+      if (lane == 0) red[warp] = smax;
       __syncthreads();
-      T smax = tube_pass<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
-      sm = block_max<T, NT>(smax, red);  // its barriers also order the carries and s_nbad
-      fb_steps += s_nbad != 0;
-      // a-posteriori fallback: redo the step from U^n with first-order faces at every tagged
-      // cell; cells still failing are tagged too (at most kFallbackPasses passes)
-      for (int pass = 1; pass <= kFallbackPasses && s_nbad; pass++) {
+      if (t == 0) {
+        int act = TUBE_STEP;
+        s_swap = 0;
+        s_clear = 0;
+        if (started) {
+          if (pass == 0) fb_steps += s_nbad != 0;
+          if (s_nbad && pass < kFallbackPasses) {
+            // a-posteriori fallback: redo the step from W^n with first-order faces at every
+            // tagged cell; cells still failing are tagged too
+            act = TUBE_RETRY;
+            pass++;
+          } else {  // the step stands
+            s_swap = 1;
+            s_clear = pass > 0 || s_nbad;
+            tt = tn;
+            steps++;
+            pass = 0;
+            if (s_any) {
+              status = 4;
+              act = TUBE_DONE;
+            }
+          }
+        }
+        if (act == TUBE_STEP && !(tt < te)) act = TUBE_DONE;
+        if (act == TUBE_STEP && steps >= a.max_steps) {
+          status = 5;
+          act = TUBE_DONE;
+        }
+        if (act == TUBE_STEP) {
+          T sm = red[0];
+          for (int w = 1; w < kWarps; w++) sm = fmax(sm, red[w]);
+          double dt = a.cfl / (double)sm;
+          tn = tt + dt;
+          if (tn >= te) {
+            dt = te - tt;
+            tn = te;
+          }
+          s_dt = (T)dt;
+        }
+        started = 1;
+        s_act = act;
+        s_nbad = 0;
+        s_any = 0;
+      }
+      __syncthreads();
+      const int act = s_act;
+      if (s_swap) {
+        T *sw = cur;  // W^{n+1} becomes the next step's W^n
+        cur = nxt;
+        nxt = sw;
+      }
+      if (s_clear) {
+        for (int c = t; c < n; c += NT) sFl[c] = 0;
         __syncthreads();
-        if (t == 0) { s_nbad = 0; s_any = 0; }
-        __syncthreads();
+      }
+      if (act == TUBE_DONE) break;
+      const T dt = s_dt, nu = dt * half_idx, dtdx = dt * idx;
+      if (act == TUBE_RETRY) {
         for (int c = t; c < n; c += NT)
           if (sFl[c] == 1) sFl[c] = 2;  // tags of earlier passes become active
         __syncthreads();
-        smax = tube_pass<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
-        sm = block_max<T, NT>(smax, red);
+        smax = tube_pass<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
+      } else {
+        smax = tube_pass<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
       }
-      const bool still_bad = s_any != 0;  // some cell of the last pass is not realizable
-      for (int c = t; c < n; c += NT) sFl[c] = 0;
-      __syncthreads();
-      T *sw = cur;  // U^{n+1} becomes the next step's U^n
-      cur = nxt;
-      nxt = sw;
-      if (still_bad) { status = 4; tt = tn; steps++; break; }
-      tt = tn;
-      steps++;
     }
-    __syncthreads();
     for (int c = t; c < n; c += NT) {
       T W[NV], U[NV];
 #pragma unroll
@@ -238,34 +265,26 @@ __global__ void __launch_bounds__(NT) tubes_kernel(TubeArgs<T> a) {
   }
 }
 
-template <typename T> size_t tube_smem(int cap, int nt) {
-  return sizeof(T) * (2 * (size_t)NV * cap + (size_t)NV * (nt + 1) + (size_t)NV * nt + NV) + (size_t)cap;
-}
+template <typename T> size_t tube_smem(int cap) { return sizeof(T) * 2 * (size_t)NV * cap + (size_t)cap; }
 
-template <typename T, int NT> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, int blocks, cudaStream_t s) {
-  const size_t smem = tube_smem<T>(a.cap, NT);
+template <typename T, int NT> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, cudaStream_t s) {
+  const size_t smem = tube_smem<T>(a.cap);
   cudaError_t e = cudaFuncSetAttribute(tubes_kernel<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int dev = 0, sms = 0, per_sm = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tubes_kernel<T, NT>, NT, smem);
   if (e != cudaSuccess) return e;
+  const int blocks = std::min(sms * std::max(1, per_sm), (int)(a.last - a.first));
   tubes_kernel<T, NT><<<blocks, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T> int tube_blocks(int cap, int nt) {
-  int dev = 0, sms = 0, maxsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  const size_t per = tube_smem<T>(cap, nt) + 1024;
-  int per_sm = (int)(maxsm / per);
-  per_sm = std::max(1, std::min(per_sm, 2048 / nt));
-  return sms * per_sm;
-}
-
 template <typename T> cudaError_t launch_tubes(const TubeArgs<T> &a, int nt, cudaStream_t s) {
-  const int blocks = std::min(tube_blocks<T>(a.cap, nt), (int)a.ntubes);
-  if (nt == 128) return launch_tubes_nt<T, 128>(a, blocks, s);
-  if (nt == 512) return launch_tubes_nt<T, 512>(a, blocks, s);
-  return launch_tubes_nt<T, 256>(a, blocks, s);
+  if (nt == 64) return launch_tubes_nt<T, 64>(a, s);
+  if (nt == 128) return launch_tubes_nt<T, 128>(a, s);
+  if (nt == 512) return launch_tubes_nt<T, 512>(a, s);
+  return launch_tubes_nt<T, 256>(a, s);
 }
 
 }  // namespace msh
@@ -299,7 +318,9 @@ struct msh_batch {
   double cfl = 0.8;
   int64_t total = 0;
   int cap = 0;
-  int threads = 0;  // chosen block size (0 = not tuned yet)
+  std::vector<int32_t> order;
+  cudaStream_t aux[2] = {nullptr, nullptr};  // side streams of the shorter classes
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::vector<int32_t> len;
@@ -343,19 +364,54 @@ msh_status upload_initial(msh_batch *b) {
   return MSH_OK;
 }
 
-msh_status run_once(msh_batch *b, int nt, int64_t max_steps) {
-  B_TRY(cudaMemsetAsync(b->d_queue, 0, sizeof(int32_t), b->stream));
-  cudaError_t e;
-  if (b->prec == MSH_FP32) {
-    TubeArgs<float> a{(float *)b->U, b->d_off, b->d_len, b->d_tend, b->d_order, b->d_queue, b->d_steps, b->d_t,
-                      b->d_status, b->d_fallback, b->total, b->ntubes, b->cap, b->cfl, max_steps};
-    e = launch_tubes<float>(a, nt, b->stream);
-  } else {
-    TubeArgs<double> a{(double *)b->U, b->d_off, b->d_len, b->d_tend, b->d_order, b->d_queue, b->d_steps, b->d_t,
-                       b->d_status, b->d_fallback, b->total, b->ntubes, b->cap, b->cfl, max_steps};
-    e = launch_tubes<double>(a, nt, b->stream);
+// A class of tubes: order[first .. last) on blocks of nt threads.
+struct TubeClass {
+  int first, last, nt;
+};
+
+// threads > 0: every tube on blocks of that size.  0: by length.  FP32: 16 warps per tube above
+// 1024 cells, 8 above 512, 4 below (each class fills an SM with 16 warps); FP64, whose buffers
+// are twice as large and whose pipe two warps per scheduler saturate: 8, 4 and 2 warps at half
+// the lengths.
+std::vector<TubeClass> tube_classes(const msh_batch *b, int threads) {
+  std::vector<TubeClass> cls;
+  if (threads > 0) {
+    cls.push_back({0, b->ntubes, threads});
+    return cls;
   }
-  if (e != cudaSuccess) return bfail(MSH_E_CUDA, "tube kernel launch: %s", cudaGetErrorString(e));
+  const bool f32 = b->prec == MSH_FP32;
+  const int above[3] = {f32 ? 1024 : 512, f32 ? 512 : 256, 0}, nt[3] = {f32 ? 512 : 256, f32 ? 256 : 128, f32 ? 128 : 64};
+  int at = 0;
+  for (int i = 0; i < 3; i++) {
+    int end = at;
+    while (end < b->ntubes && b->len[b->order[end]] > above[i]) end++;
+    if (end > at) cls.push_back({at, end, nt[i]});
+    at = end;
+  }
+  return cls;
+}
+
+template <typename T> cudaError_t launch_class(msh_batch *b, const TubeClass &c, int i, int64_t max_steps, cudaStream_t s) {
+  TubeArgs<T> a{(T *)b->U, b->d_off, b->d_len, b->d_tend, b->d_order, b->d_queue + i, c.first, c.last, b->d_steps, b->d_t,
+                b->d_status, b->d_fallback, b->total, b->len[b->order[c.first]], b->cfl, max_steps};
+  return launch_tubes<T>(a, c.nt, s);
+}
+
+msh_status run_once(msh_batch *b, int threads, int64_t max_steps) {
+  const std::vector<TubeClass> cls = tube_classes(b, threads);
+  B_TRY(cudaMemsetAsync(b->d_queue, 0, 3 * sizeof(int32_t), b->stream));
+  if (cls.size() > 1) B_TRY(cudaEventRecord(b->ev_fork, b->stream));
+  for (size_t i = 0; i < cls.size(); i++) {
+    cudaStream_t s = i == 0 ? b->stream : b->aux[i - 1];
+    if (i > 0) B_TRY(cudaStreamWaitEvent(s, b->ev_fork, 0));
+    const cudaError_t e = b->prec == MSH_FP32 ? launch_class<float>(b, cls[i], (int)i, max_steps, s)
+                                              : launch_class<double>(b, cls[i], (int)i, max_steps, s);
+    if (e != cudaSuccess) return bfail(MSH_E_CUDA, "tube kernel launch: %s", cudaGetErrorString(e));
+    if (i > 0) {
+      B_TRY(cudaEventRecord(b->ev_join[i - 1], s));
+      B_TRY(cudaStreamWaitEvent(b->stream, b->ev_join[i - 1], 0));
+    }
+  }
   return MSH_OK;
 }
 
@@ -418,7 +474,8 @@ msh_status msh_batch_init(msh_batch **out, int32_t ntubes, const int32_t *len, c
     acc += len[k];
   }
   b->total = acc;
-  std::vector<int32_t> order(ntubes);
+  std::vector<int32_t> &order = b->order;
+  order.resize(ntubes);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return len[x] > len[y]; });
   b->init.resize((size_t)b->total * NV * b->esize);
@@ -434,11 +491,16 @@ msh_status msh_batch_init(msh_batch **out, int32_t ntubes, const int32_t *len, c
     e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     b->own_stream = true;
   }
+  for (auto &x : b->aux)
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+  for (auto &x : b->ev_join)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMalloc(&b->U, (size_t)b->total * NV * b->esize);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_off, sizeof(int64_t) * ntubes);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_len, sizeof(int32_t) * ntubes);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_order, sizeof(int32_t) * ntubes);
-  if (e == cudaSuccess) e = cudaMalloc(&b->d_queue, sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_queue, 3 * sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_status, sizeof(int32_t) * ntubes);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_tend, sizeof(double) * ntubes);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_t, sizeof(double) * ntubes);
@@ -471,45 +533,13 @@ msh_status msh_batch_run(msh_batch *b, int32_t threads, int64_t max_steps) {
   if (threads != 0 && threads != 128 && threads != 256 && threads != 512)
     return bfail(MSH_E_INVALID_ARG, "threads must be 0, 128, 256 or 512");
   if (max_steps < 1) return bfail(MSH_E_INVALID_ARG, "max_steps must be >= 1");
-  int nt = threads;
-  if (nt == 0 && b->threads == 0) {
-    // autotune: time each block size on a full run from the initial state
-    cudaEvent_t e0, e1;
-    B_TRY(cudaEventCreate(&e0));
-    B_TRY(cudaEventCreate(&e1));
-    float best = 1e30f;
-    int best_nt = 256;
-    for (int cand : {128, 256, 512}) {
-      const size_t need = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, cand) : tube_smem<double>(b->cap, cand);
-      if (need > 227 * 1024) continue;
-      msh_status st = upload_initial(b);
-      if (st) return st;
-      B_TRY(cudaEventRecord(e0, b->stream));
-      st = run_once(b, cand, max_steps);
-      if (st) return st;
-      B_TRY(cudaEventRecord(e1, b->stream));
-      B_TRY(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      B_TRY(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best) {
-        best = ms;
-        best_nt = cand;
-      }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    b->threads = best_nt;
-    msh_status st = upload_initial(b);
-    if (st) return st;
-  }
-  if (nt == 0) nt = b->threads;
-  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, nt) : tube_smem<double>(b->cap, nt);
-  if (smem > 227 * 1024) return bfail(MSH_E_INVALID_ARG, "tubes too long for %d threads (%zu B shared)", nt, smem);
-  // one persistent launch, captured in a CUDA graph (queue reset + kernel)
+  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap) : tube_smem<double>(b->cap);
+  if (smem > 227 * 1024) return bfail(MSH_E_INVALID_ARG, "tubes too long for shared memory (%zu B)", smem);
+  // one persistent launch per class of lengths, captured in a CUDA graph with the queue reset
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   B_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-  msh_status st = run_once(b, nt, max_steps);
+  msh_status st = run_once(b, threads, max_steps);
   cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
   if (st) {
     if (graph) cudaGraphDestroy(graph);
@@ -634,6 +664,11 @@ msh_status msh_batch_destroy(msh_batch *b) {
   cudaFree(b->d_t);
   cudaFree(b->d_steps);
   cudaFree(b->d_fallback);
+  for (auto x : b->aux)
+    if (x) cudaStreamDestroy(x);
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  for (auto x : b->ev_join)
+    if (x) cudaEventDestroy(x);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
   delete b;
   return MSH_OK;
