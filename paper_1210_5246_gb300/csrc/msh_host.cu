@@ -127,7 +127,8 @@ msh_status ensure_partials(msh_grid *g, int need) {
 
 void drop_graph(msh_grid *g) {
   if (g->graph) cudaGraphExecDestroy(g->graph);
-  g->graph = nullptr;
+  if (g->graph_lean) cudaGraphExecDestroy(g->graph_lean);
+  g->graph = g->graph_lean = nullptr;
 }
 
 // Copy the tape fields of the host mirror (the tail of Ctrl) to the device control block.
@@ -348,28 +349,47 @@ msh_status launch_one_step(msh_grid *g, int ev_slot) {
   return MSH_OK;
 }
 
+// Pass `level` of the streaming characteristic step.
+cudaError_t launch_pass(msh_grid *g, int level, int *nb) {
+  if (g->prec == MSH_FP32) {
+    StepArgs<float> a = make_args<float>(g);
+    a.level = level;
+    return launch_characteristic(g, a, level > 0, nb);
+  }
+  StepArgs<double> a = make_args<double>(g);
+  a.level = level;
+  return launch_characteristic(g, a, level > 0, nb);
+}
+
+// Whether this grid's steps are streaming characteristic ones whose fallback passes can be left
+// to the host.
+bool lean_steps(msh_grid *g) {
+  return g->scheme != MSH_SCHEME_KT && g->sg_G == 0.0 && !(g->test_fault == 1 && g->ndim == 3) && !use_staged(g);
+}
+
+// A step without its fallback passes (four launches that nearly always return at once): the
+// finalize stops the run with kStatusPending if cells were tagged.
+msh_status launch_lean_step(msh_grid *g) {
+  g->phase_level = -1;
+  int nb = 0;
+  cudaError_t e = launch_pass(g, 0, &nb);
+  if (e == cudaSuccess) e = launch_finalize(g->ctrl, g->part, nb, 3, g->stream);
+  if (e != cudaSuccess) return fail(MSH_E_CUDA, "step launch: %s", cudaGetErrorString(e));
+  return MSH_OK;
+}
+
 // One whole step whose result the host reads anyway: the streaming characteristic step's
 // fallback passes are launched only if the control block says that cells were tagged (four
 // launches less otherwise).
 msh_status step_and_read(msh_grid *g) {
-  const bool test = g->test_fault == 1 && g->ndim == 3;
-  if (g->scheme == MSH_SCHEME_KT || g->sg_G > 0.0 || test || use_staged(g)) {
+  if (!lean_steps(g)) {
     msh_status st = launch_one_step(g, -1);
     return st ? st : read_ctrl(g);
   }
   g->phase_level = -1;
   int nb = 0;
   for (int level = 0; level <= kFallbackPasses; level++) {
-    cudaError_t e;
-    if (g->prec == MSH_FP32) {
-      StepArgs<float> a = make_args<float>(g);
-      a.level = level;
-      e = launch_characteristic(g, a, level > 0, level > 0 ? nullptr : &nb);
-    } else {
-      StepArgs<double> a = make_args<double>(g);
-      a.level = level;
-      e = launch_characteristic(g, a, level > 0, level > 0 ? nullptr : &nb);
-    }
+    cudaError_t e = launch_pass(g, level, level > 0 ? nullptr : &nb);
     if (e != cudaSuccess) return fail(MSH_E_CUDA, "step launch: %s", cudaGetErrorString(e));
     if (level != 0 && level != kFallbackPasses) continue;
     e = launch_finalize(g->ctrl, g->part, nb, level == 0 ? 2 : 0, g->stream);
@@ -397,8 +417,9 @@ msh_status launch_steps(msh_grid *g, int64_t n) {
   return MSH_OK;
 }
 
-msh_status build_graph(msh_grid *g) {
-  if (g->graph) return MSH_OK;
+msh_status build_graph(msh_grid *g, bool lean) {
+  cudaGraphExec_t &exec = lean ? g->graph_lean : g->graph;
+  if (exec) return MSH_OK;
   const int32_t test_fault = g->test_fault;  // test hooks never enter a graph
   g->test_fault = 0;
   struct Restore {
@@ -412,7 +433,7 @@ msh_status build_graph(msh_grid *g) {
   cudaGraph_t graph;
   CUDA_TRY(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
   for (int i = 0; i < kGraphSteps; i++) {
-    st = launch_one_step(g, i);
+    st = lean ? launch_lean_step(g) : launch_one_step(g, i);
     if (st) {
       cudaStreamEndCapture(g->stream, &graph);
       if (graph) cudaGraphDestroy(graph);
@@ -420,7 +441,7 @@ msh_status build_graph(msh_grid *g) {
     }
   }
   CUDA_TRY(cudaStreamEndCapture(g->stream, &graph));
-  cudaError_t e = cudaGraphInstantiate(&g->graph, graph, 0);
+  cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
   return MSH_OK;
@@ -440,6 +461,46 @@ void collect_profile(msh_grid *g, int slots) {
       (void)cudaGetLastError();
     }
   }
+}
+
+// Launch a started run until the device control reports completion or `left` steps were
+// launched, and read the control block.
+msh_status run_batches(msh_grid *g, bool staged, bool lean, int64_t left, int batch) {
+  msh_status st = MSH_OK;
+  if (left < batch) {
+    // short runs: exactly that many steps, no speculative batch
+    if (lean)
+      for (int64_t i = 0; i < left && st == MSH_OK; i++) st = launch_lean_step(g);
+    else
+      st = launch_steps(g, left);
+    return st ? st : read_ctrl(g);
+  }
+  if (!staged) {
+    st = build_graph(g, lean);
+    if (st) return st;
+  }
+  // Two batches (graphs, or staged launches) in flight: launch batch it, then wait for the
+  // completion flag of batch it-1, so the GPU never idles while the host polls.  Batches
+  // launched after the run finished return immediately on the device.
+  const int64_t need = left / batch + (left % batch != 0);
+  for (int64_t it = 0;; it++) {
+    if (it > need + 1) return fail(MSH_E_STATE, "run did not terminate (device control inconsistent)");
+    if (it < need) {
+      if (staged) {
+        st = launch_steps(g, batch);
+        if (st) return st;
+      } else {
+        CUDA_TRY(cudaGraphLaunch(lean ? g->graph_lean : g->graph, g->stream));
+      }
+      CUDA_TRY(cudaMemcpyAsync(&g->hdone[it & 1], &g->ctrl->done, sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+      CUDA_TRY(cudaEventRecord(g->ev_done[it & 1], g->stream));
+    }
+    if (it >= 1) {
+      CUDA_TRY(cudaEventSynchronize(g->ev_done[(it - 1) & 1]));
+      if (g->hdone[(it - 1) & 1] || it >= need) break;
+    }
+  }
+  return read_ctrl(g);
 }
 
 // One pass over src (launch_scan) into the grid's control block or `ctrl`.
@@ -693,6 +754,7 @@ msh_status msh_set_state(msh_grid *g, const void *U, int32_t where, int32_t kind
     return fail(MSH_E_REALIZABILITY, "state not realizable at cell %lld (rho <= 0 or P not SPD)", (long long)bad);
   }
   g->has_state = true;
+  g->tags_seen = false;
   return MSH_OK;
 }
 
@@ -969,15 +1031,14 @@ msh_status msh_run(msh_grid *g, double t_end, int64_t max_steps, int64_t *steps,
   // the staged step runs many steps per launch and needs no graph
   const bool staged = !g->profiling && g->sg_G == 0.0 && use_staged(g);
   const int batch = staged ? kStagedSteps : kGraphSteps;
-  st = g->profiling || staged ? ensure_partials(g, blocks_for(g, g->rows, g->zchunk)) : build_graph(g);
+  st = ensure_partials(g, blocks_for(g, g->rows, g->zchunk));
   if (st) return st;
   const int64_t s0 = g->hctrl->step;
   cudaError_t e = launch_run_start(g->ctrl, t_end, max_steps, INFINITY, g->stream);
   if (e != cudaSuccess) return fail(MSH_E_CUDA, "run start: %s", cudaGetErrorString(e));
-  // at most this many batches of steps can be needed
-  const int64_t need = max_steps / batch + (max_steps % batch != 0);
   if (g->profiling) {
     // profiled runs launch the same kernels eagerly, bracketed by events
+    const int64_t need = max_steps / batch + (max_steps % batch != 0);
     for (int64_t it = 0;; it++) {
       if (it > need) return fail(MSH_E_STATE, "run did not terminate (device control inconsistent)");
       const int64_t before = g->hctrl->step;
@@ -991,36 +1052,27 @@ msh_status msh_run(msh_grid *g, double t_end, int64_t max_steps, int64_t *steps,
       collect_profile(g, (int)(g->hctrl->step - before));
       if (g->hctrl->done) break;
     }
-  } else if (max_steps < batch) {
-    // short runs: exactly max_steps steps, no speculative batch
-    st = launch_steps(g, max_steps);
-    if (st) return st;
-    st = read_ctrl(g);
-    if (st) return st;
   } else {
-    // Two batches (graphs, or staged launches) in flight: launch batch it, then wait for the completion flag of
-    // batch it-1, so the GPU never idles while the host polls.  Batches launched after
-    // the run finished return immediately on the device.
-    for (int64_t it = 0;; it++) {
-      if (it > need + 1) return fail(MSH_E_STATE, "run did not terminate (device control inconsistent)");
-      if (it < need) {
-        if (staged) {
-          st = launch_steps(g, batch);
-          if (st) return st;
-        } else {
-          CUDA_TRY(cudaGraphLaunch(g->graph, g->stream));
-        }
-        CUDA_TRY(cudaMemcpyAsync(&g->hdone[it & 1], &g->ctrl->done, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                 g->stream));
-        CUDA_TRY(cudaEventRecord(g->ev_done[it & 1], g->stream));
-      }
-      if (it >= 1) {
-        CUDA_TRY(cudaEventSynchronize(g->ev_done[(it - 1) & 1]));
-        if (g->hdone[(it - 1) & 1] || it >= need) break;
-      }
+    // Streaming characteristic steps go without their fallback passes until one tags cells; the
+    // run then stops, the host launches that step's passes, and the rest of the run (and later
+    // runs of this state) takes every step with its passes.
+    bool lean = !staged && !g->tags_seen && lean_steps(g);
+    int64_t left = max_steps;
+    for (;;) {
+      st = run_batches(g, staged, lean, left, batch);
+      if (st) return st;
+      if (!lean || g->hctrl->status != kStatusPending) break;
+      lean = false;
+      g->tags_seen = true;
+      e = launch_resume(g->ctrl, g->stream);
+      for (int level = 1; e == cudaSuccess && level <= kFallbackPasses; level++) e = launch_pass(g, level, nullptr);
+      if (e == cudaSuccess) e = launch_finalize(g->ctrl, g->part, blocks_for(g, g->rows, g->zchunk), 0, g->stream);
+      if (e != cudaSuccess) return fail(MSH_E_CUDA, "fallback passes: %s", cudaGetErrorString(e));
+      st = read_ctrl(g);
+      if (st) return st;
+      if (g->hctrl->done) break;
+      left = max_steps - (g->hctrl->step - s0);
     }
-    st = read_ctrl(g);
-    if (st) return st;
   }
   if (steps) *steps = g->hctrl->step - s0;
   if (t_out) *t_out = g->hctrl->t;

@@ -22,6 +22,9 @@ struct NvtxRange {
 
 // A-posteriori fallback passes per step (see the step kernels).
 constexpr int kFallbackPasses = 4;
+// Control-block status of a run that waits for the host to launch a step's fallback passes
+// (never returned to a caller).
+constexpr int32_t kStatusPending = 99;
 
 // Device-resident time control of a grid.  The step kernels read dt and the buffer
 // parity from here; the finalize kernel writes the next dt, so a run needs no host
@@ -158,6 +161,7 @@ cudaError_t launch_tags(Ctrl *ctrl, int32_t *flags, size_t c0, size_t c1, int32_
 cudaError_t launch_count_tags(const Ctrl *ctrl, const int32_t *flags, size_t c0, size_t c1, int level,
                               unsigned long long *count, cudaStream_t s);
 cudaError_t launch_finalize(Ctrl *ctrl, const Partial *part, int nparts, int mode, cudaStream_t s);
+cudaError_t launch_resume(Ctrl *ctrl, cudaStream_t s);
 cudaError_t launch_run_start(Ctrl *ctrl, double t_end, int64_t max_steps, double dt_max, cudaStream_t s);
 cudaError_t launch_ensemble_start(Ctrl *ctrl, int64_t step_base, int64_t nsteps, int32_t *status, cudaStream_t s);
 cudaError_t launch_ensemble_end(const Ctrl *ctrl, int32_t *status, cudaStream_t s);
@@ -240,7 +244,9 @@ struct msh_grid {
   void *stg_mem = nullptr;
   bool stg_off = false;
   double tile_us = 0.0;  // estimated step time of the streaming kernels' default shape
-  cudaGraphExec_t graph = nullptr;
+  // kGraphSteps steps with their fallback passes, and without (see msh_run)
+  cudaGraphExec_t graph = nullptr, graph_lean = nullptr;
+  bool tags_seen = false;  // a run since the last msh_set_state tagged cells
   // profiling: eager launches with events around every step-kernel launch
   bool profiling = false;
   std::vector<cudaEvent_t> ev;

@@ -119,11 +119,18 @@ __device__ void finalize_block(Ctrl *ctrl, const Partial *part, int nparts, int 
   plan(c);
 }
 
-// mode 2: mode 0 unless the step tagged cells (the host then runs the fallback passes and mode 0)
+// mode 2: mode 0 unless the step tagged cells (the host then runs the fallback passes and mode
+// 0); mode 3: the same in the middle of a run, which stops there with kStatusPending
 __global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, const Partial *part, int nparts,
                                                                     int mode) {
   if (mode != 1 && ctrl->done) return;
-  if (mode == 2 && ctrl->nbad[0] != 0 && !ctrl->stage_timeout) return;
+  if (mode >= 2 && ctrl->nbad[0] != 0 && !ctrl->stage_timeout) {
+    if (mode == 3 && threadIdx.x == 0) {
+      ctrl->status = kStatusPending;
+      ctrl->done = 1;
+    }
+    return;
+  }
   finalize_block(ctrl, part, nparts, mode == 1 ? 1 : 0);
 }
 
@@ -471,6 +478,17 @@ cudaError_t launch_gravity_field(const double *phi, T *acc, int ndim, int nx, in
 
 cudaError_t launch_finalize(Ctrl *ctrl, const Partial *part, int nparts, int mode, cudaStream_t s) {
   finalize_kernel<<<1, kFinalizeThreads, 0, s>>>(ctrl, part, nparts, mode);
+  return cudaGetLastError();
+}
+
+// go on with a run that stopped with kStatusPending
+__global__ void resume_kernel(Ctrl *c) {
+  c->status = 0;
+  c->done = 0;
+}
+
+cudaError_t launch_resume(Ctrl *ctrl, cudaStream_t s) {
+  resume_kernel<<<1, 1, 0, s>>>(ctrl);
   return cudaGetLastError();
 }
 
