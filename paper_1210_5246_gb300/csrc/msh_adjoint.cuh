@@ -251,7 +251,7 @@ __device__ __forceinline__ void mc_weights(float l, float r, float &fl, float &f
   fr = !on ? 0.0f : side ? (left ? 0.0f : 2.0f) : 0.5f;
 }
 __device__ __forceinline__ void mc_weights(double l, double r, double &fl, double &fr) {
-  // on the bit patterns, as mc_limit2
+  // on the bit patterns, as mc_half
   constexpr long long kAbs = 0x7fffffffffffffffll, kInf = 0x7ff0000000000000ll;
   const long long bl = __double_as_longlong(l), br = __double_as_longlong(r), al = bl & kAbs, ar = br & kAbs;
   const long long c = __double_as_longlong(l + r) & kAbs;
@@ -291,9 +291,9 @@ __device__ __forceinline__ void reconstruct_vjp(const T (&wm)[NV], const T (&w0)
   }
   E.project(dL, cl);
   E.project(dR, cr);
-  mc_limit2_v(cl, cr, m);
+  mc_half_v(cl, cr, m);
 #pragma unroll
-  for (int k = 0; k < NV; k++) m[k] *= T(0.5);
+  for (int k = 0; k < NV; k++) m[k] *= T(2);
   lm[0] = -E.cf * m[0]; lm[1] = -E.cs * m[1]; lm[2] = -E.cs * m[2];
   lm[3] = T(0); lm[4] = T(0); lm[5] = T(0); lm[6] = T(0);
   lm[7] = E.cs * m[7]; lm[8] = E.cs * m[8]; lm[9] = E.cf * m[9];

@@ -59,12 +59,12 @@ constexpr int kStagedSteps = 64;  // steps of one staged launch at most
 constexpr size_t kStagedMaxBytes = size_t(2) << 30;
 // FP32 grids of up to this many cells (1D, 2D, 3D) may take the staged step (beyond, its face
 // states leave L2); in 2D and 3D where its estimated time is the shorter one.  Fits to timed
-// steps: staged 2D 13.7 us + 0.97e-4 us per cell (64^2 13.7, 256^2 20.1, 512^2 39), 3D 14.7 us +
-// 2e-4 us per cell (32^3 21, 64^3 67, 97x61x45 72); a streaming step adds 8 us of launches to its
-// kernel (256^2 27.7 us, 512^2 38, 64^3 74, 97x61x45 73.5).
+// steps: staged 2D 13.0 us + 0.97e-4 us per cell (64^2 13, 256^2 20, 512^2 38), 3D 14.7 us + 1.9e-4 us per
+// cell (32^3 21, 64^3 64, 97x61x45 69); a streaming step adds 3 us to its kernel (256^2 19.5 us,
+// 512^2 28.8, 64^3 69).
 constexpr size_t kStagedMaxCells32[3] = {size_t(1) << 24, 400000, 400000};
-constexpr double kStagedBase[3] = {0.0, 13.7, 14.7}, kStagedPerCell[3] = {0.0, 0.97e-4, 2.0e-4};
-constexpr double kStreamLaunches = 8.0;
+constexpr double kStagedBase[3] = {0.0, 13.0, 14.7}, kStagedPerCell[3] = {0.0, 0.97e-4, 1.9e-4};
+constexpr double kStreamLaunches = 3.0;
 
 }  // namespace
 

@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
       const int c = g * 32 + lane;
       if (c >= (int)N) continue;
 #pragma unroll
-      for (int k = 0; k < NV; k++) d[k] += (double)U[k * N + c];
+      for (int k = 0; k < NV; k++) d[k] += widen(U[k * N + c]);
     }
     int comp;
     const double x = warp_sum10(d, comp);

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) scan_kernel(const T *src, T 
     if (!realizable(W)) bad = min(bad, (long long)c);
     smax = max_nonneg(smax, speed_sum<T, NDIM, MAXF>(W, idx, idy, idz));
 #pragma unroll
-    for (int k = 0; k < NV; k++) diag[k] += (double)Uc[k];
+    for (int k = 0; k < NV; k++) diag[k] += widen(Uc[k]);
   }
   block_partial<kFinalizeThreads>(diag, (double)smax, bad, part + blockIdx.x);
   __shared__ int s_last;
@@ -370,9 +370,10 @@ static double balanced_cost(long long ncols, long long nz, long long units, doub
 //            a prologue costs as much as 6 planes.  256^3: 16 rows balanced 1.60 ms against
 //            2.14 ms with 8 rows; 160^3: two chunks of 80 planes per column 0.47 ms, balanced
 //            0.70 ms (its last windows are 8 planes long); 48^3 CTU: 8 rows in chunks of 6.
-//   2D FP32  a row of a strip takes 2.7 us while a scheduler has up to two warps, 3.2 us with
-//            three and 3.7 us with four; a chunk's prologue, partial and start cost as much as
-//            3.6 rows.  512^2: 4 rows 28 us, 8 rows 31 us, 16 rows 54 us; 1024^2: 16 rows 73 us.
+//   2D FP32  a row of a strip takes 2.05 us while a scheduler has up to two warps, 2.5 us with
+//            three and 2.9 us with four; a chunk's prologue, partial and start cost as much as
+//            5.2 rows.  512^2: 4 rows 26.8 us, 8 rows 28.0 us; 1024^2: 16 rows 61.6 us; 700^2: 10 rows
+//            43.8 us.
 //   FP64     the double-precision pipe is the bound: time goes with the warps per scheduler,
 //            a prologue costs about one row or plane.
 Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu) {
@@ -396,7 +397,7 @@ Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu) {
         if (f32) {
           const long long slots = sms * (16 / rows), waves = blocks / slots, rest = blocks - waves * slots;
           const double w = (double)((rest + sms - 1) / sms) * rows / 4.0;  // warps per scheduler, last wave
-          cost = (c + 3.6) * (3.7 * (double)waves + (rest == 0 ? 0.0 : w <= 2.0 ? 2.7 : w <= 3.0 ? 3.2 : 3.7));
+          cost = (c + 5.2) * (2.9 * (double)waves + (rest == 0 ? 0.0 : w <= 2.0 ? 2.05 : w <= 3.0 ? 2.5 : 2.9));
         } else {
           cost = (c + 1.0) * (double)((blocks + sms - 1) / sms) * rows / 4.0;
         }

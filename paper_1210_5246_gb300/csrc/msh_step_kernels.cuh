@@ -1010,10 +1010,13 @@ __global__ void __launch_bounds__(32 * BY, (BY <= 8 && !CTU && sizeof(T) == 4 ? 
     }
   }
   cp_async_wait<0>();
+  // a chunk is the unit's only stretch: its sums go to the partial directly
+  if (a.zchunk > 0) break;
   if constexpr (sizeof(T) == 4) flush_totals<T, 32 * BY>(diag, tot);  // its barrier also ends the stretch
   __syncthreads();  // the next stretch restages every buffer
   }
   write_partial<T, 32 * BY>(diag, smax, bad, a.part + u, tot);
+  __syncthreads();  // the next unit restages every buffer and restarts the totals
   }
   if (kTma && tma_on && tid == 0 && tma_dead) {
     // a wait ran out: let copies still in flight land (bounded) before the block exits

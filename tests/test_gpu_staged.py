@@ -138,3 +138,40 @@ def test_staged_reverse_equals_pencils(msh, n, bc, prec):
         g.close()
     tol = 1e-12 if prec == "FP64" else 2e-5
     assert np.abs(out[0] - out[1]).max() <= tol * np.abs(out[1]).max()
+
+
+@pytest.mark.parametrize("prec", ["FP64", "FP32"])
+@pytest.mark.parametrize("n,tiling", [((60, 41), (4, 5)), ((90, 70), (16, 9)), ((25, 18, 12), (8, 0)), ((64, 33, 20), (8, 5))])
+def test_run_that_tags_cells(msh, n, tiling, prec):
+    """A streaming run launches its steps without fallback passes until one tags cells; profiled
+    runs launch every pass.  Extreme states tag cells in the first steps and later: states,
+    times and the error of a run that stays non-realizable agree, also over short runs."""
+    nd = len(n)
+    W = _state((1,) * (3 - nd) + n[::-1], 7, extreme=True)
+    out = []
+    for profiled in (False, True):
+        g = msh.Grid(n, (0.0,) * nd, (1.0,) * nd, (BCS["mix"],) * nd, 0.5, getattr(msh, prec))
+        g.set_tiling(*tiling)
+        g.set_profiling(profiled)
+        g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+        seen = []
+        for steps in (3, 40, 1):
+            try:
+                seen.append(g.run(max_steps=steps))
+            except msh.MshError as e:
+                seen.append((e.status, str(e)))
+                break
+        out.append((seen, g.get_state(), g.time(), g.diagnostics()[1:]))
+        g.close()
+    assert out[0][0] == out[1][0] and out[0][2:] == out[1][2:]
+    np.testing.assert_array_equal(out[0][1], out[1][1])
+    # the first step tags cells
+    g = msh.Grid(n, (0.0,) * nd, (1.0,) * nd, (BCS["mix"],) * nd, 0.5, getattr(msh, prec))
+    g.set_tiling(*tiling)
+    g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+    _, dt, _ = g.reduce_layers(0, n[-1])
+    try:
+        assert g.step_dt(dt) > 0
+    except msh.MshError:
+        pass
+    g.close()
