@@ -322,9 +322,7 @@ template <typename T, int NDIM> static cudaError_t launch_reverse_nd(const Stage
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     occ.store(per_sm, std::memory_order_relaxed);
   }
-  const size_t N = (size_t)a.a.s.nx * a.a.s.ny * a.a.s.nz;
-  const long long groups = (long long)NDIM * (long long)((N + 31) / 32);
-  const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)device_sms() * per_sm, (groups + 3) / 4));
+  const int blocks = staged_blocks<NDIM>(a.a.s, per_sm);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(kStagedThreads);

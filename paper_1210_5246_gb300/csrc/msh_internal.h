@@ -80,7 +80,7 @@ template <typename T> struct StepArgs {
 
 // Grid barrier of the staged step (msh_staged.cuh), zero between launches.
 struct GridBar {
-  unsigned arrived, left, dead;
+  unsigned arrived, left;
 };
 
 // Arguments of a staged launch: the step's, and the staging buffers.

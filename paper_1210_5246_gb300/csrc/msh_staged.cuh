@@ -31,31 +31,32 @@ constexpr int kStagedWarps = kStagedThreads / 32;
 // ------------------------------------------------------------ grid barrier
 // Arrivals only grow within a launch; the last block to leave a launch clears them for the
 // next.  Waits are bounded: a block that waits longer than 2^33 clocks (about four seconds)
-// marks the barrier dead, every block leaves, and the launch reports MSH_E_TIMEOUT.
+// sets the counter's top bit, every block leaves, and the launch reports MSH_E_TIMEOUT.  One
+// release, one polled word: a separate fence, counter and flag cost three trips to L2 (4100
+// cycles with 152 blocks on a small grid).
+constexpr unsigned kBarDead = 0x80000000u;
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void red_release_add(unsigned *p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ bool grid_barrier(GridBar *b, unsigned nblk, unsigned &epoch, int *s_dead) {
   __syncthreads();
   if (nblk == 1) return true;
   epoch += nblk;
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&b->arrived, 1u);
-    if (ld_acquire_u32(&b->arrived) < epoch) {
+    red_release_add(&b->arrived, 1u);
+    unsigned v = ld_acquire_u32(&b->arrived);
+    if (v < epoch) {
       const long long t0 = clock64();
-      while (ld_acquire_u32(&b->arrived) < epoch) {
-        if (ld_acquire_u32(&b->dead) != 0u) break;
-        if (clock64() - t0 > (1ll << 33)) {
-          atomicExch(&b->dead, 1u);
-          break;
-        }
+      while ((v = ld_acquire_u32(&b->arrived)) < epoch) {  // (a dead counter is above every epoch)
+        if (clock64() - t0 > (1ll << 33)) atomicOr(&b->arrived, kBarDead);
       }
     }
-    *s_dead = (int)ld_acquire_u32(&b->dead);
-    __threadfence();
+    *s_dead = (v & kBarDead) != 0u;
   }
   __syncthreads();
   return *s_dead == 0;
@@ -66,7 +67,6 @@ __device__ __forceinline__ void grid_leave(GridBar *b, unsigned nblk) {
   if (atomicAdd(&b->left, 1u) == nblk - 1) {  // every block has passed its last barrier
     b->arrived = 0u;
     b->left = 0u;
-    b->dead = 0u;
   }
 }
 
@@ -243,46 +243,48 @@ __device__ __forceinline__ void load_fluxes(const StagedArgs<T> &a, size_t N, in
 // upper y), so that the sums round alike.
 template <typename T, int NDIM>
 __device__ __forceinline__ void divergence(const StagedArgs<T> &a, size_t N, int c, T idx, T idy, T idz, T (&acc)[NV]) {
-  T fl[NV], fu[NV], t[NV], u[NV];
+  // every face flux is requested before the first is used (one wait instead of one per
+  // direction: stage C of a 64^3 FP32 grid took longer than the reconstructions)
+  T xl[NV], xu[NV], yl[NV], yu[NV], zl[NV], zu[NV], t[NV];
+  load_fluxes<T, 0>(a, N, c, xl, xu);
+  if constexpr (NDIM > 1) load_fluxes<T, 1>(a, N, c, yl, yu);
+  if constexpr (NDIM > 2) load_fluxes<T, 2>(a, N, c, zl, zu);
   if constexpr (NDIM == 1) {
-    load_fluxes<T, 0>(a, N, c, fl, fu);
 #pragma unroll
-    for (int k = 0; k < NV; k++) acc[k] = (fl[k] - fu[k]) * idx;
+    for (int k = 0; k < NV; k++) acc[k] = (xl[k] - xu[k]) * idx;
   } else if constexpr (NDIM == 2) {
-    load_fluxes<T, 1>(a, N, c, fl, fu);
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-      t[Frame<1>::g(k)] = fl[k];
-      u[Frame<1>::g(k)] = fu[k];
-    }
+    for (int k = 0; k < NV; k++) t[Frame<1>::g(k)] = yl[k];
     v_mul(acc, t, idy);
-    load_fluxes<T, 0>(a, N, c, fl, fu);
-    v_sub(fl, fl, fu);
-    v_fma(acc, fl, idx, acc);
-    v_fma(acc, u, -idy, acc);
+    v_sub(xl, xl, xu);
+    v_fma(acc, xl, idx, acc);
+#pragma unroll
+    for (int k = 0; k < NV; k++) t[Frame<1>::g(k)] = yu[k];
+    v_fma(acc, t, -idy, acc);
   } else {
-    load_fluxes<T, 2>(a, N, c, fl, fu);
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-      t[Frame<2>::g(k)] = fl[k];
-      u[Frame<2>::g(k)] = fu[k];
-    }
+    for (int k = 0; k < NV; k++) t[Frame<2>::g(k)] = zl[k];
     v_mul(acc, t, idz);
-    load_fluxes<T, 0>(a, N, c, fl, fu);
-    v_sub(fl, fl, fu);
-    v_fma(acc, fl, idx, acc);
-    load_fluxes<T, 1>(a, N, c, fl, fu);
+    v_sub(xl, xl, xu);
+    v_fma(acc, xl, idx, acc);
 #pragma unroll
-    for (int k = 0; k < NV; k++) t[Frame<1>::g(k)] = fl[k];
+    for (int k = 0; k < NV; k++) t[Frame<1>::g(k)] = yl[k];
     v_fma(acc, t, idy, acc);
-    v_fma(acc, u, -idz, acc);
 #pragma unroll
-    for (int k = 0; k < NV; k++) acc[Frame<1>::g(k)] -= fu[k] * idy;
+    for (int k = 0; k < NV; k++) t[Frame<2>::g(k)] = zu[k];
+    v_fma(acc, t, -idz, acc);
+#pragma unroll
+    for (int k = 0; k < NV; k++) acc[Frame<1>::g(k)] -= yu[k] * idy;
   }
 }
 
-// The time control of a launch, the same in every block.
+// The time control of a launch, the same in every block (the run's constants are copied from
+// the control block once).
 struct StagedTime {
+  double cfl, t_end, dt_max;
+  int64_t max_step, tape_base, tape_len, hist_base, hist_cap;
+  double *tape_dt, *hist;
+  int32_t *tape_had;
   double t, t_next, dt, dt_last, dt_cfl;
   int64_t step;
   int64_t first_bad;
@@ -303,6 +305,7 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
   __shared__ double s_red[kStagedWarps][NV];
   __shared__ double s_max[kStagedWarps];
   __shared__ long long s_bad[kStagedWarps];
+  __shared__ int s_cnt[kStagedWarps];
   const StepArgs<T> &s = a.s;
   Ctrl *ctrl = s.ctrl;
   if (a.seg == nullptr && ctrl->done) return;  // the same in every block: nothing writes it before the first barrier
@@ -312,6 +315,17 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
   const int ngrp = (int)((N + 31) / 32);
   unsigned epoch = 0;
   if (tid == 0) {
+    st.cfl = ctrl->cfl;
+    st.t_end = ctrl->t_end;
+    st.dt_max = ctrl->dt_max;
+    st.max_step = ctrl->max_step;
+    st.tape_base = ctrl->tape_base;
+    st.tape_len = ctrl->tape_len;
+    st.tape_dt = ctrl->tape_dt;
+    st.tape_had = ctrl->tape_had;
+    st.hist = ctrl->hist;
+    st.hist_base = ctrl->hist_base;
+    st.hist_cap = ctrl->hist_cap;
     st.t = ctrl->t;
     st.t_next = ctrl->t_next;
     st.dt = ctrl->dt;
@@ -444,19 +458,40 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     smax = T(0);
     bad = LLONG_MAX;
   };
-  auto reduce_parts = [&](double &m, long long &b, int &nb) {  // warp 0
+  // every thread takes a partial, so that all are in flight at once; the result is known to
+  // warp 0 (one warp walking over 152 partials waited for L2 five times)
+  auto reduce_parts = [&](double &m, long long &b, int &nb) {
     m = 0.0;
     b = LLONG_MAX;
     nb = 0;
-    for (unsigned i = lane; i < nblk; i += 32) {
-      m = max_nonneg(m, __ldcg(&s.part[i].smax));
-      b = min(b, __ldcg(&s.part[i].bad));
+    for (unsigned i = tid; i < nblk; i += kStagedThreads) {
+      const double pm = __ldcg(&s.part[i].smax);
+      const long long pb = __ldcg(&s.part[i].bad);
       nb += __ldcg(&a.newly[i]);
+      m = max_nonneg(m, pm);
+      b = min(b, pb);
     }
     m = warp_max_nonneg(m);
     nb = __reduce_add_sync(FULL, nb);
+    if (__any_sync(FULL, b != LLONG_MAX)) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b = min(b, __shfl_xor_sync(FULL, b, o));
+      for (int o = 16; o > 0; o >>= 1) b = min(b, __shfl_xor_sync(FULL, b, o));
+    }
+    if (nblk > 32) {
+      if (lane == 0) {
+        s_max[warp] = m;
+        s_bad[warp] = b;
+        s_cnt[warp] = nb;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        for (int w = 1; w < kStagedWarps; w++) {
+          m = max_nonneg(m, s_max[w]);
+          b = min(b, s_bad[w]);
+          nb += s_cnt[w];
+        }
+      }
+    }
   };
 
   {  // P
@@ -510,17 +545,15 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     double m;
     long long b;
     int nb;
-    if (warp == 0) {
-      reduce_parts(m, b, nb);
-      if (lane == 0) {
-        st.newly = nb;
-        st.any_tagged = nb;
-      }
-    }
-    __syncthreads();
+    reduce_parts(m, b, nb);
     // a-posteriori fallback: passes with first-order faces at the tagged cells, while the
     // pass before tagged new ones
     if (!kKt) {
+      if (tid == 0) {
+        st.newly = nb;
+        st.any_tagged = nb;
+      }
+      __syncthreads();
       for (int level = 1; level <= kFallbackPasses && st.newly > 0; level++) {
         stages_ab(W0, tag, level);
         if (!alive) break;
@@ -528,65 +561,76 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
         write_part();
         alive = grid_barrier(a.bar, nblk, epoch, &s_dead);
         if (!alive) break;
-        if (warp == 0) {
-          reduce_parts(m, b, nb);
-          if (lane == 0) st.newly = nb;
-        }
+        reduce_parts(m, b, nb);
+        if (tid == 0) st.newly = nb;
         __syncthreads();
       }
       if (!alive) break;
     }
     taken++;
-    if (tid == 0) {  // plan the next step, as the finalize kernel does
+    if (warp == 0) {  // plan the next step, as the finalize kernel does (every lane alike)
+      const int any = kKt ? 0 : st.any_tagged;
+      double nd;
+      bool stop;
       if (a.seg != nullptr) {
-        st.stop = taken >= a.max_iter;
-        if (!st.stop) st.dt = a.dts[taken];
-        st.step = step + 1;
-        if (blk == 0 && a.had != nullptr) a.had[taken - 1] = st.any_tagged > 0;
-        if (blk == 0 && st.any_tagged > 0)
-          for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
-      } else {
-        st.last_tagged = st.any_tagged;
-        st.realizable = b == LLONG_MAX;
-        st.first_bad = b == LLONG_MAX ? -1 : b;
-        st.dt_cfl = ctrl->cfl / m;
-        if (blk == 0) {
-          const int64_t ti = step - ctrl->tape_base;
-          if (ctrl->tape_dt != nullptr && ti >= 0 && ti < ctrl->tape_len) {
-            ctrl->tape_dt[ti] = dt;
-            ctrl->tape_had[ti] = st.any_tagged > 0;
-          }
-          const int64_t hi_ = step - ctrl->hist_base;
-          if (ctrl->hist != nullptr && hi_ >= 0 && hi_ < ctrl->hist_cap) ctrl->hist[hi_] = dt;
-          if (st.any_tagged > 0)
+        stop = taken >= a.max_iter;
+        nd = stop ? dt : a.dts[taken];
+        if (lane == 0) {
+          st.dt = nd;
+          st.step = step + 1;
+          if (blk == 0 && a.had != nullptr) a.had[taken - 1] = any > 0;
+          if (blk == 0 && any > 0)
             for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
         }
-        st.dt_last = dt;
-        st.t = st.t_next;
-        st.step = step + 1;
-        if (!st.realizable) {
-          st.status = 4;  // MSH_E_REALIZABILITY
-          st.done = 1;
-        } else if (st.t >= ctrl->t_end || st.step >= ctrl->max_step) {
-          st.done = 1;
-        } else {
-          double nd = st.dt_cfl;
-          if (nd > ctrl->dt_max) nd = ctrl->dt_max;
-          double tn = st.t + nd;
-          if (tn >= ctrl->t_end) {
-            nd = ctrl->t_end - st.t;
-            tn = ctrl->t_end;
+      } else {
+        const double t = st.t_next, dt_cfl = st.cfl / m;
+        double tn = t + dt_cfl;
+        nd = dt_cfl;
+        if (nd > st.dt_max) {
+          nd = st.dt_max;
+          tn = t + nd;
+        }
+        if (tn >= st.t_end) {
+          nd = st.t_end - t;
+          tn = st.t_end;
+        }
+        const bool real = b == LLONG_MAX;
+        const bool done = !real || t >= st.t_end || step + 1 >= st.max_step;
+        if (done) {
+          nd = dt;
+          tn = t;
+        }
+        stop = done || taken >= a.max_iter;
+        __syncwarp();  // every lane has read the old state
+        if (lane == 0) {
+          st.last_tagged = any;
+          st.realizable = real;
+          st.first_bad = real ? -1 : b;
+          st.dt_cfl = dt_cfl;
+          if (blk == 0) {
+            const int64_t ti = step - st.tape_base, hi_ = step - st.hist_base;
+            if (st.tape_dt != nullptr && ti >= 0 && ti < st.tape_len) {
+              st.tape_dt[ti] = dt;
+              st.tape_had[ti] = any > 0;
+            }
+            if (st.hist != nullptr && hi_ >= 0 && hi_ < st.hist_cap) st.hist[hi_] = dt;
+            if (any > 0)
+              for (int p = 0; p <= kFallbackPasses; p++) ctrl->nbad[p] = 0;
           }
+          st.dt_last = dt;
+          st.t = t;
+          st.step = step + 1;
+          if (!real) st.status = 4;  // MSH_E_REALIZABILITY
+          st.done = done;
           st.dt = nd;
           st.t_next = tn;
         }
-        st.stop = st.done || taken >= a.max_iter;
       }
+      if (lane == 0) st.stop = stop;
+      if (lane < 3 && !stop) st.nu[lane] = 0.5 * nd / (lane == 0 ? s.dx[0] : lane == 1 ? s.dx[1] : s.dx[2]);
     }
     __syncthreads();
     if (st.stop) break;
-    if (tid < 3) st.nu[tid] = 0.5 * st.dt / (tid == 0 ? s.dx[0] : tid == 1 ? s.dx[1] : s.dx[2]);
-    __syncthreads();
   }
   if (!alive) {  // a barrier gave up: the result is void
     if (tid == 0) {
@@ -653,6 +697,19 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
 }
 
 // ----------------------------------------------------------------- launcher
+// As many blocks as the SMs hold, but no more than give every scheduler one group of 32 items of
+// stage A, the ghost cells' included (four groups per block): a second double-precision warp on
+// a scheduler doubles a short stage (256 FP64 cells in 1D: stage A 22000 cycles with two blocks).
+template <int NDIM, typename T> int staged_blocks(const StepArgs<T> &s, int per_sm) {
+  const long long N = (long long)s.nx * s.ny * s.nz;
+  long long groups = NDIM * ((N + 31) / 32);
+  for (int d = 0; d < NDIM; d++) {
+    const long long np = N / (d == 0 ? s.nx : d == 1 ? s.ny : s.nz);
+    if (s.bc[2 * d] != BC_PERIODIC) groups += (2 * np + 31) / 32;
+  }
+  return (int)std::max<long long>(1, std::min<long long>((long long)device_sms() * per_sm, (groups + 3) / 4));
+}
+
 template <typename T, int NDIM, int SCH> cudaError_t launch_staged_nd(const StagedArgs<T> &a, cudaStream_t s, int *nblk) {
   static std::atomic<int> occ{0};
   int per_sm = occ.load(std::memory_order_relaxed);
@@ -663,11 +720,7 @@ template <typename T, int NDIM, int SCH> cudaError_t launch_staged_nd(const Stag
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     occ.store(per_sm, std::memory_order_relaxed);
   }
-  // as many blocks as the SMs hold, but no more than give every scheduler a group of 32 items
-  // of stage A (four groups per block)
-  const size_t N = (size_t)a.s.nx * a.s.ny * a.s.nz;
-  const long long groups = (long long)NDIM * (long long)((N + 31) / 32);
-  const int blocks = (int)std::max<long long>(1, std::min<long long>((long long)device_sms() * per_sm, (groups + 3) / 4));
+  const int blocks = staged_blocks<NDIM>(a.s, per_sm);
   if (nblk != nullptr) *nblk = blocks;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
