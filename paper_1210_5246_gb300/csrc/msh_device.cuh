@@ -772,12 +772,13 @@ __device__ __forceinline__ double widen(float x) {
 // ---------------------------------------------------------- accumulators
 // Per-thread running sums of the conserved totals over the cells one thread updates.  FP64
 // states add in FP64.  FP32 states add in FP32 per thread (relative rounding error of a
-// k-term sum below k 2^-24, random in sign across threads) and in FP64 from the block
-// reduction on, so the totals need no FP64 arithmetic per cell (FP64 throughput is a small
+// k-term sum below k 2^-24, random in sign across threads), in pairs of floats over a warp
+// (warp_sum10) and in FP64 from there on, so the totals need no FP64 arithmetic per cell (FP64 throughput is a small
 // fraction of FP32 on this GPU).  The 3D step moves a thread's FP32 sum into FP64 block
 // totals every 64 planes of a stretch and at its end, so one FP32 sum spans at most 64
 // cells; 2D strips and 1D tiles stream one chunk.
 template <typename T> struct Acc {
+  using Sum = double;  // what a thread hands to the warp's sum
   double v[NV];
   __device__ __forceinline__ void zero() {
 #pragma unroll
@@ -793,6 +794,7 @@ template <typename T> struct Acc {
   }
 };
 template <> struct Acc<float> {
+  using Sum = float;
   float v[NV];
   __device__ __forceinline__ void zero() {
 #pragma unroll
@@ -806,9 +808,9 @@ template <> struct Acc<float> {
       v[k + 1] = r.y;
     }
   }
-  __device__ __forceinline__ void get(double (&o)[NV]) const {
+  __device__ __forceinline__ void get(float (&o)[NV]) const {
 #pragma unroll
-    for (int k = 0; k < NV; k++) o[k] = widen(v[k]);
+    for (int k = 0; k < NV; k++) o[k] = v[k];
   }
 };
 

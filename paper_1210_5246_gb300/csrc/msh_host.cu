@@ -84,7 +84,7 @@ template <typename T> StepArgs<T> make_args(msh_grid *g) {
   a.ny = (int)g->n[1];
   a.nz = (int)g->n[2];
   for (int i = 0; i < 6; i++) a.bc[i] = g->bc[i];
-  for (int i = 0; i < 3; i++) a.dx[i] = g->dx[i];
+  a.set_widths(g->dx);
   a.zchunk = g->zchunk;
   a.level = 0;
   a.ck = g->tape_valid ? (T *)g->tape : nullptr;

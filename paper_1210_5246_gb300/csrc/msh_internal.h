@@ -66,7 +66,14 @@ template <typename T> struct StepArgs {
   int level;            // 0: the step; p >= 1: fallback pass p
   int nx, ny, nz;
   int bc[6];
-  double dx[3];
+  double dx[3];  // cell widths, and their reciprocals in the state's precision (set_widths):
+  T rdx[3];      // kernels take them from the constant bank as they are
+  void set_widths(const double *w) {
+    for (int i = 0; i < 3; i++) {
+      dx[i] = w[i];
+      rdx[i] = (T)(1.0 / w[i]);
+    }
+  }
   int zchunk;
   // adjoint tape: the step kernel stores U^s in ck[(s - ck_base) / ck_K] when s - ck_base
   // is a multiple of ck_K in [0, ck_len); ck = nullptr: no tape

@@ -58,7 +58,7 @@ msh_status noalloc_step(int ndim, const int64_t n[3], const double dx[3], const 
   a.ny = (int)n[1];
   a.nz = (int)n[2];
   for (int i = 0; i < 6; i++) a.bc[i] = i < 2 * ndim ? bc[i] : MSH_BC_PERIODIC;
-  for (int i = 0; i < 3; i++) a.dx[i] = dx[i];
+  a.set_widths(dx);
   a.level = 0;
   a.ck = nullptr;  // no adjoint tape
   a.ck_base = 0;

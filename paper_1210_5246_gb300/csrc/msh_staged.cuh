@@ -342,10 +342,8 @@ __global__ void __launch_bounds__(kStagedThreads, sizeof(T) == 4 ? 2 : 1) staged
     if (a.seg != nullptr) st.dt = a.dts[0];
   }
   __syncthreads();
-  __shared__ double sc[6];
-  step_factors(s.dx, st.dt, sc);
-  const T idx = (T)sc[3], idy = (T)sc[4], idz = (T)sc[5];
-  if (tid < 3) st.nu[tid] = sc[tid];  // first read after a barrier
+  step_factors(s.dx, st.dt, st.nu);
+  const T idx = s.rdx[0], idy = s.rdx[1], idz = s.rdx[2];
   // groups of 32 items are dealt out warp by warp, blocks first, so that a short list
   // spreads over the SMs and over the schedulers of each
   const int w0 = warp * (int)nblk + (int)blk, wstep = kStagedWarps * (int)nblk;

@@ -83,13 +83,75 @@ __device__ __forceinline__ double warp_sum10(double (&v)[NV], int &comp) {
   return x;
 }
 
+// The same for ten FP32 values per lane, in pairs of floats (an error-free sum and its running
+// error: relative error below 2^-45 over a warp, where one thread's FP32 sum carries up to
+// 2^-19): 107 FP32 operations instead of 12 FP64 additions at 77 pipe cycles and ten conversions,
+// 1.8 us at the end of a block of 16 warps.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = a + b;
+  const float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+__device__ __forceinline__ void pair_add(float &h, float &l, float bh, float bl) {
+  float s, e;
+  two_sum(h, bh, s, e);
+  e += l + bl;
+  h = s + e;
+  l = e - (h - s);
+}
+__device__ __forceinline__ double warp_sum10(float (&v)[NV], int &comp) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+  float h[6], l[6];
+#pragma unroll
+  for (int k = 0; k < 5; k++) {
+    const float o = __shfl_xor_sync(FULL, b4 ? v[k] : v[k + 5], 16);
+    two_sum(b4 ? v[k + 5] : v[k], o, h[k], l[k]);
+  }
+  h[5] = l[5] = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const float oh = __shfl_xor_sync(FULL, b3 ? h[k] : h[k + 3], 8), ol = __shfl_xor_sync(FULL, b3 ? l[k] : l[k + 3], 8);
+    h[k] = b3 ? h[k + 3] : h[k];
+    l[k] = b3 ? l[k + 3] : l[k];
+    pair_add(h[k], l[k], oh, ol);
+  }
+  h[3] = l[3] = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    const float oh = __shfl_xor_sync(FULL, b2 ? h[k] : h[k + 2], 4), ol = __shfl_xor_sync(FULL, b2 ? l[k] : l[k + 2], 4);
+    h[k] = b2 ? h[k + 2] : h[k];
+    l[k] = b2 ? l[k + 2] : l[k];
+    pair_add(h[k], l[k], oh, ol);
+  }
+  const float oh = __shfl_xor_sync(FULL, b1 ? h[0] : h[1], 2), ol = __shfl_xor_sync(FULL, b1 ? l[0] : l[1], 2);
+  float xh = b1 ? h[1] : h[0], xl = b1 ? l[1] : l[0];
+  pair_add(xh, xl, oh, ol);
+  const float ph = __shfl_xor_sync(FULL, xh, 1), pl = __shfl_xor_sync(FULL, xl, 1);
+  pair_add(xh, xl, ph, pl);
+  const int in3 = (b2 ? 2 : 0) + (b1 ? 1 : 0), in5 = (b3 ? 3 : 0) + in3;
+  comp = (in3 < 3 && in5 < 5) ? (b4 ? 5 : 0) + in5 : -1;
+  return widen(xh) + widen(xl);
+}
+
+// Sum over the warps of a block of ten values each, red[warp][component]: warp 0 alone, three
+// lanes per component and two shuffles; lane c < 10 returns component c (one thread per
+// component took 17 dependent additions for 16 warps).
+template <int NW, int PITCH> __device__ __forceinline__ double cross_warp_sum(const double (&red)[NW][PITCH]) {
+  const int lane = threadIdx.x & 31, g = lane / NV, c = lane - g * NV;
+  double v = 0.0;
+  if (g < 3)
+    for (int w = g; w < NW; w += 3) v += red[w][c];
+  const double v1 = __shfl_down_sync(FULL, v, 10), v2 = __shfl_down_sync(FULL, v, 20);
+  return (v + v1) + v2;
+}
+
 // Partial of a block of NT threads: totals (plus `base`), signal speed, first bad cell.  The
-// FP64 additions are few on purpose: 12 per warp (warp_sum10), then ten threads sum one
-// component each over the warps; every one holds a scheduler's FP64 pipe for 64 cycles or
+// FP64 additions are few on purpose: every one holds a scheduler's FP64 pipe for 64 cycles or
 // more, also in FP32 kernels (one thread adding ten components of 16 warps took 6 us).
-template <int NT>
-__device__ __forceinline__ void block_partial(double (&diag)[NV], double smax, long long bad,
-                                              Partial *out, const double *base = nullptr) {
+template <int NT, typename S>
+__device__ __forceinline__ void block_partial(S (&diag)[NV], double smax, long long bad, Partial *out,
+                                              const double *base = nullptr) {
   __shared__ double red[NT / 32][NV + 1];
   __shared__ long long redb[NT / 32];
   const int lane = threadIdx.x & 31;
@@ -108,10 +170,9 @@ __device__ __forceinline__ void block_partial(double (&diag)[NV], double smax, l
     redb[warp] = bad;
   }
   __syncthreads();
-  if (tid < NV) {
-    double sum = base != nullptr ? base[tid] : 0.0;
-    for (int w = 0; w < NT / 32; w++) sum += red[w][tid];
-    out->diag[tid] = sum;
+  if (warp == 0) {
+    const double sum = cross_warp_sum(red);
+    if (tid < NV) out->diag[tid] = base != nullptr ? base[tid] + sum : sum;
   }
   if (tid == NT - 1) {
     double m = red[0][NV];
@@ -141,15 +202,11 @@ __device__ __forceinline__ T speed_sum(const T (&W)[NV], T idx, T idy, T idz) {
   return s;
 }
 
-// nu_d = dt / (2 dx_d) and 1 / dx_d, rounded from FP64: one lane per quotient and a broadcast
-// through shared memory.  (Every thread dividing for itself took six FP64 divisions, 580
-// pipe cycles each, per warp of every block.)
+// nu_d = dt / (2 dx_d), divided in FP64: one lane per quotient and a broadcast through shared
+// memory.  (Every thread dividing for itself took 580 pipe cycles per quotient and warp.)
 __device__ __forceinline__ void step_factors(const double (&dx)[3], double dt, double *sc) {
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  if (tid < 6) {
-    const int d = tid < 3 ? tid : tid - 3;
-    sc[tid] = (tid < 3 ? 0.5 * dt : 1.0) / (d == 0 ? dx[0] : d == 1 ? dx[1] : dx[2]);
-  }
+  if (tid < 3) sc[tid] = 0.5 * dt / (tid == 0 ? dx[0] : tid == 1 ? dx[1] : dx[2]);
   __syncthreads();
 }
 
@@ -251,7 +308,7 @@ done:
 
 template <typename T, int NT>
 __device__ __forceinline__ void write_partial(const Acc<T> &diag, T smax, long long bad, Partial *out) {
-  double d[NV];
+  typename Acc<T>::Sum d[NV];
   diag.get(d);
   block_partial<NT>(d, (double)smax, bad, out);
 }
@@ -259,7 +316,7 @@ __device__ __forceinline__ void write_partial(const Acc<T> &diag, T smax, long l
 template <typename T, int NT>
 __device__ __forceinline__ void write_partial(const Acc<T> &diag, T smax, long long bad, Partial *out,
                                               const double *base) {
-  double d[NV];
+  typename Acc<T>::Sum d[NV];
   diag.get(d);
   block_partial<NT>(d, (double)smax, bad, out, base);
 }
@@ -275,7 +332,7 @@ __device__ __forceinline__ double *block_totals() {
 // block calls it.
 template <typename T, int NT> __device__ __forceinline__ void flush_totals(Acc<T> &diag, double *tot) {
   __shared__ double red[NT / 32][NV];
-  double d[NV];
+  typename Acc<T>::Sum d[NV];
   diag.get(d);
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -283,10 +340,9 @@ template <typename T, int NT> __device__ __forceinline__ void flush_totals(Acc<T
   const double x = warp_sum10(d, comp);
   if (comp >= 0 && (lane & 1) == 0) red[tid >> 5][comp] = x;
   __syncthreads();
-  if (tid < NV) {
-    double sum = tot[tid];
-    for (int w = 0; w < NT / 32; w++) sum += red[w][tid];
-    tot[tid] = sum;
+  if (tid < 32) {
+    const double sum = cross_warp_sum(red);
+    if (tid < NV) tot[tid] += sum;
   }
   diag.zero();
 }
@@ -303,19 +359,19 @@ template <typename T, int SCH, bool RETRY>
 __global__ void __launch_bounds__(kTile1D) step1d_kernel(StepArgs<T> a) {
   constexpr int B = kTile1D, SXX = B + 2;
   const Ctrl *ctrl = a.ctrl;
+  const int64_t step = ctrl->step;  // read together with the flags: one wait for L2
+  const double dtd = ctrl->dt;
   if (ctrl->done) return;
   if (RETRY && ctrl->nbad[a.level - 1] == 0 && !((ctrl->force >> a.level) & 1)) return;
-  const int64_t step = ctrl->step;
   const int32_t tag = (int32_t)(step & 0x0fffffff) + 1;
   __shared__ unsigned char sFl[RETRY ? SXX : 1];
   // sweep source, destination and U^n (the second Runge-Kutta stage sweeps U1)
   const T *__restrict__ U0 = a.U[step & 1];
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
-  const double dtd = ctrl->dt;
-  __shared__ double sc[6];
+  __shared__ double sc[3];
   step_factors(a.dx, dtd, sc);
-  const T dt = (T)dtd, nu = (T)sc[0], idx = (T)sc[3];
+  const T dt = (T)dtd, nu = (T)sc[0], idx = a.rdx[0];
   __shared__ T sW[NV][SXX];
   __shared__ T sH[NV][B];
   const int t = threadIdx.x;
@@ -489,9 +545,10 @@ __global__ void __launch_bounds__(32 * BY, (BY <= 8 && !CTU && sizeof(T) == 4 ? 
   constexpr int RSTR = kTma ? (NV * RNQ * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T) : NV * RNQ;
   constexpr unsigned kTmaBytes = (unsigned)(kTmaBoxX * SY * NV * sizeof(T));
   const Ctrl *ctrl = a.ctrl;
+  const int64_t step = ctrl->step;  // read together with the flags: one wait for L2
+  const double dtd = ctrl->dt;
   if (ctrl->done) return;
   if (RETRY && ctrl->nbad[a.level - 1] == 0 && !((ctrl->force >> a.level) & 1)) return;
-  const int64_t step = ctrl->step;
   const int32_t tag = (int32_t)(step & 0x0fffffff) + 1;
   // fallback tags of the staged cells (fallback pass only)
   __shared__ unsigned char sFl[RETRY ? 3 : 1][RETRY ? NQ : 1];
@@ -499,13 +556,12 @@ __global__ void __launch_bounds__(32 * BY, (BY <= 8 && !CTU && sizeof(T) == 4 ? 
   const T *__restrict__ U0 = a.U[step & 1];
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
-  const double dtd = ctrl->dt;
-  __shared__ double sc[6];
+  __shared__ double sc[3];
   step_factors(a.dx, dtd, sc);
   const T dt = (T)dtd;
-  const T nux = (T)sc[0], idx = (T)sc[3];
-  const T nuy = (T)sc[1], idy = (T)sc[4];
-  const T nuz = (T)sc[2], idz = (T)sc[5];
+  const T nux = (T)sc[0], idx = a.rdx[0];
+  const T nuy = (T)sc[1], idy = a.rdx[1];
+  const T nuz = (T)sc[2], idz = a.rdx[2];
   T *const ck = (RETRY || SCH != 0) ? nullptr : tape_slot(a, step, (size_t)a.nx * a.ny * a.nz);
   // shared memory: RAW raw conserved planes filled one plane ahead (bulk tensor copies or
   // cp.async), three primitive planes (ring), the y-sweep face states and fluxes, per staged
@@ -1046,20 +1102,18 @@ __global__ void __launch_bounds__(32 * WARPS) step_strip2d_kernel(StepArgs<T> a)
   extern __shared__ __align__(16) unsigned char strip_raw[];
   __shared__ T sTy[CTU ? WARPS : 1][NV][32];  // CTU: T_y of the lane's cell in the row of the x sweep
   const Ctrl *ctrl = a.ctrl;
+  const int64_t step = ctrl->step;  // read together with the flags: one wait for L2
+  const double dtd = ctrl->dt;
   if (ctrl->done) return;
   if (RETRY && ctrl->nbad[a.level - 1] == 0 && !((ctrl->force >> a.level) & 1)) return;
-  const int64_t step = ctrl->step;
   const int32_t tag = (int32_t)(step & 0x0fffffff) + 1;
   // sweep source, destination and U^n (the second Runge-Kutta stage sweeps U1)
   const T *__restrict__ U0 = a.U[step & 1];
   const T *__restrict__ Us = SCH == 2 ? a.U1 : U0;
   T *__restrict__ Ud = SCH == 1 ? a.U1 : a.U[(step + 1) & 1];
-  const double dtd = ctrl->dt;
-  __shared__ double sc[6];
-  step_factors(a.dx, dtd, sc);
-  const T dt = (T)dtd;
-  const T nux = (T)sc[0], idx = (T)sc[3];
-  const T nuy = (T)sc[1], idy = (T)sc[4];
+  __shared__ double sc[3];
+  const T dt = (T)dtd, idx = a.rdx[0], idy = a.rdx[1];
+  T nux = T(0), nuy = T(0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nx = a.nx, ny = a.ny, ych = a.zchunk;
   const size_t N = (size_t)nx * ny;
@@ -1072,23 +1126,34 @@ __global__ void __launch_bounds__(32 * WARPS) step_strip2d_kernel(StepArgs<T> a)
     diag.zero();
     T smax = T(0);
     long long bad = LLONG_MAX;
-    const int tile = grp * WARPS + warp;
+    const int tile = grp * WARPS + warp, tc = min(tile, ntiles - 1);
+    const int x0 = (tc % stripsx) * kStripX, y0 = (tc / stripsx) * ych;
+    const int y1 = min(y0 + ych, ny);
+    const int gx = x0 - 2 + lane;
+    bool mx;
+    const int xx = map_index(gx, nx, a.bc[0], a.bc[1], mx);
+    // the lane's column of the ring: field k of slot q at ring[(q * NV + k) * 32]
+    T *const ring = reinterpret_cast<T *>(strip_raw) + (size_t)warp * kStripRing * NV * 32 + lane;
+    auto slot = [&](int y) { return ring + ((y - y0 + 2) % kStripRing) * NV * 32; };
+    auto stage = [&](int y) {  // one commit group per row
+      bool my;
+      const int yy = map_index(y, ny, a.bc[2], a.bc[3], my);
+      cp_async_cell<T, 32 * (int)sizeof(T)>(slot(y), Us + (size_t)yy * nx + xx, N);
+      cp_async_commit();
+    };
     if (tile < ntiles) {  // warp-uniform
-      const int x0 = (tile % stripsx) * kStripX, y0 = (tile / stripsx) * ych;
-      const int y1 = min(y0 + ych, ny);
-      const int gx = x0 - 2 + lane;
-      bool mx;
-      const int xx = map_index(gx, nx, a.bc[0], a.bc[1], mx);
+      stage(y0 - 2);
+      stage(y0 - 1);
+      stage(y0);
+      stage(y0 + 1);
+    }
+    if (grp == (int)blockIdx.x) {  // the first rows are on their way while the factors are divided
+      step_factors(a.dx, dtd, sc);
+      nux = (T)sc[0];
+      nuy = (T)sc[1];
+    }
+    if (tile < ntiles) {
       const bool upd = lane >= 2 && lane <= kStripX + 1 && gx < nx;
-      // the lane's column of the ring: field k of slot q at ring[(q * NV + k) * 32]
-      T *const ring = reinterpret_cast<T *>(strip_raw) + (size_t)warp * kStripRing * NV * 32 + lane;
-      auto slot = [&](int y) { return ring + ((y - y0 + 2) % kStripRing) * NV * 32; };
-      auto stage = [&](int y) {  // one commit group per row
-        bool my;
-        const int yy = map_index(y, ny, a.bc[2], a.bc[3], my);
-        cp_async_cell<T, 32 * (int)sizeof(T)>(slot(y), Us + (size_t)yy * nx + xx, N);
-        cp_async_commit();
-      };
       // raw conserved row (with the reflect images' sign flips) and its fallback tag
       auto fetch = [&](int y, T (&U)[NV], bool &fl) {
         bool my;
@@ -1141,10 +1206,6 @@ __global__ void __launch_bounds__(32 * WARPS) step_strip2d_kernel(StepArgs<T> a)
       {
         T U[NV], w[NV], wa[NV];
         bool fa;
-        stage(y0 - 2);
-        stage(y0 - 1);
-        stage(y0);
-        stage(y0 + 1);
         cp_async_wait<3>();
         fetch(y0 - 2, U, fa); cons_to_prim(U, w); ylocal(w, wa);
         stage(y0 + 2);  // each row replaces one whose conversion is done
