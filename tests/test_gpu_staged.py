@@ -175,3 +175,23 @@ def test_run_that_tags_cells(msh, n, tiling, prec):
     except msh.MshError:
         pass
     g.close()
+
+
+def test_noalloc_thin_box_fits_the_fixed_scratch(msh):
+    # a box two cells wide and deep whose default shape for a grid would be 18695 blocks, more
+    # partials than the allocation-free step's scratch holds: stepped all the same, to the same bits
+    import torch
+    n, bc = (2, 261730, 2), ((0, 0),) * 3
+    W = _state((n[2], n[1], n[0]), seed=61)
+    g = msh.Grid(n, (0.0,) * 3, (1.0, 1.5, 0.5), bc, 0.3, msh.FP32)
+    g.set_tiling(8, 0)
+    g.set_state(W.astype(np.float32), msh.PRIMITIVE)
+    U0 = g.get_state()
+    dt = g.step()
+    U1 = g.get_state()
+    g.close()
+    u0 = torch.tensor(U0, device="cuda")
+    u1 = torch.empty_like(u0)
+    e = msh.msh_step_noalloc(n, (0.0,) * 3, (1.0, 1.5, 0.5), bc, msh.FP32, 0.3, u0, u1)
+    assert abs(e - dt) <= 1e-12 * dt
+    assert np.array_equal(u1.cpu().numpy().reshape(U1.shape), U1)
