@@ -189,11 +189,16 @@ msh_status msh_get_dt_history(msh_grid *g, double *dts, int64_t capacity, int64_
  * planes each).  2D: `rows` = warps per block (4, 8 or 16, each a strip of 28 updated
  * columns) and `zchunk` = grid rows each warp streams in y.  1D ignores both.  `zchunk` >=
  * 1 (3D: >= 0), clipped to the streamed axis.  3D FP64 grids take rows 4 or 8 (rows 16
- * would need more shared memory than a thread block has).  Defaults: rows 8; zchunk 0
- * (3D) or 16 (2D).  msh_autotune times the candidates (3D: rows 4/8/16 with the balanced
- * tiling and with chunks cutting z into 1..8 near-equal windows; 2D: rows 4/8/16 with
- * zchunk 8..64) on this grid's current state (without changing it or the tape) and keeps
- * the fastest; the chosen values are returned in *rows / *zchunk (may be NULL).
+ * would need more shared memory than a thread block has).  The default shape follows from an
+ * estimate of the step's time on the grid's size, precision and CTU setting.  FP64 grids whose
+ * staging buffers (2 + 2 ndim states) stay below 2 GiB, and small FP32 grids, take their steps
+ * by the staged kernel instead (the same results bit for bit; the buffers are allocated at
+ * the first step, and where they do not fit the streaming kernels go on); msh_set_tiling
+ * selects the streaming kernels.  msh_autotune times the candidates (the current shape; 3D:
+ * rows 4/8/16 with the balanced tiling and with chunks cutting z into 1..8 near-equal windows;
+ * 2D: rows 4/8/16 with zchunk 8..64; the staged step where the grid's size allows it) on this
+ * grid's current state (without changing it or the tape) and keeps the fastest; the chosen
+ * shape (the best streaming one) is returned in *rows / *zchunk (may be NULL).
  */
 msh_status msh_set_tiling(msh_grid *g, int32_t rows, int32_t zchunk);
 msh_status msh_get_tiling(msh_grid *g, int32_t *rows, int32_t *zchunk);
@@ -399,12 +404,13 @@ msh_status msh_count_tags(msh_grid *g, int64_t start, int64_t count, int32_t lev
  *   t_end[ntubes]    final times (host doubles, > 0)
  *   precision        MSH_FP32 or MSH_FP64
  * The tubes are stored back to back, [10][sum len] (tube k starts at the prefix sum of
- * len).  msh_batch_run advances all tubes in one persistent launch captured in a CUDA
- * graph; thread blocks take tubes longest first from a device work queue.  Cells whose
+ * len).  msh_batch_run advances all tubes in one persistent launch per class of lengths (at
+ * most three, side by side), captured in a CUDA graph; thread blocks take tubes longest first
+ * from a device work queue per class.  Cells whose
  * second-order update is not realizable trigger the same a-posteriori first-order
  * fallback as msh_step (the step is recomputed from U^n with first-order faces there);
  * a tube still non-realizable after it stops with MSH_E_REALIZABILITY.  threads is
- * the block size (0 = autotuned: the fastest of the candidates on a warm-up run).
+ * the block size (0: chosen by the tubes' lengths).
  * max_steps caps the steps of each tube (MSH_E_TIMEOUT if a tube hits it before t_end).
  */
 msh_status msh_batch_init(msh_batch **out, int32_t ntubes, const int32_t *len, const double *WL,
@@ -440,7 +446,8 @@ msh_status msh_batch_destroy(msh_batch *b);
  *   dt_taken   host pointer receiving the step size (may be NULL)
  * The step is always the default one of a new grid: characteristic MUSCL-Hancock with the
  * HLL flux, no corner-transport-upwind terms, the a-posteriori fallback, the default tiling
- * (8 rows); a grid set to another scheme, to CTU or to another tiling steps differently.
+ * of a grid of this size; a grid set to another scheme, to CTU or to another tiling steps
+ * differently.
  * A non-realizable U_in (rho <= 0 or P not positive definite in some cell) is rejected with
  * MSH_E_REALIZABILITY before any step, U_out untouched; a step whose result stays
  * non-realizable after the fallback passes also returns MSH_E_REALIZABILITY (U_out then

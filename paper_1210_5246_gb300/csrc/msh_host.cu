@@ -1,10 +1,12 @@
 // msh_host.cu -- C ABI of libmsh: grid lifecycle, state transfer, step/run control.
 //
 // A grid owns two state buffers (ping-pong by step parity), a device control block
-// (time, dt, step counter, stop flags), per-block reduction partials and a cached CUDA
-// graph holding kGraphSteps consecutive (step, finalize) launch pairs.  msh_run launches
-// that graph until the device control block reports completion; kernels of a finished
-// run return immediately, so over-launching past t_end is harmless.
+// (time, dt, step counter, stop flags), per-block reduction partials and either the staging
+// buffers of the staged step (up to kStagedSteps steps per cooperative launch) or cached CUDA
+// graphs of kGraphSteps streaming steps: a lean one of (step, finalize) launch pairs, run
+// until a step tags cells, and one with the fallback passes.  msh_run launches batches until
+// the device control block reports completion; kernels of a finished run return immediately,
+// so over-launching past t_end is harmless.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -847,7 +849,7 @@ msh_status msh_run_ensemble(msh_grid *g, int64_t count, const void *const *in, v
   }
   for (int64_t k = 0; k < count; k++)
     if (hs[(size_t)k] == MSH_E_TIMEOUT)
-      return fail(MSH_E_TIMEOUT, "ensemble state %lld: a step kernel gave up waiting for a bulk copy", (long long)k);
+      return fail(MSH_E_TIMEOUT, "ensemble state %lld: a step kernel gave up waiting", (long long)k);
   if (first_bad >= 0)
     return fail(MSH_E_REALIZABILITY, "ensemble state %lld is not realizable (input or result)", (long long)first_bad);
   return MSH_OK;
@@ -1014,7 +1016,7 @@ msh_status msh_step(msh_grid *g, double dt_max, double *dt_taken) {
   if (st) return st;
   if (dt_taken) *dt_taken = g->hctrl->dt_last;
   if (g->hctrl->status == MSH_E_TIMEOUT)
-    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting for a bulk copy of its staged planes");
+    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting (a bulk copy of its staged planes, or a barrier between its stages)");
   if (g->hctrl->status == MSH_E_REALIZABILITY)
     return fail(MSH_E_REALIZABILITY, "step produced a non-realizable cell %lld", (long long)g->hctrl->first_bad);
   return MSH_OK;
@@ -1077,7 +1079,7 @@ msh_status msh_run(msh_grid *g, double t_end, int64_t max_steps, int64_t *steps,
   if (steps) *steps = g->hctrl->step - s0;
   if (t_out) *t_out = g->hctrl->t;
   if (g->hctrl->status == MSH_E_TIMEOUT)
-    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting for a bulk copy of its staged planes");
+    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting (a bulk copy of its staged planes, or a barrier between its stages)");
   if (g->hctrl->status == MSH_E_REALIZABILITY)
     return fail(MSH_E_REALIZABILITY, "non-realizable cell %lld at step %lld", (long long)g->hctrl->first_bad,
                 (long long)g->hctrl->step);
@@ -1232,7 +1234,7 @@ msh_status msh_step_dt(msh_grid *g, double dt, int32_t *tagged_cells) {
   g->dt_stale = false;  // the finalize planned from the new state
   if (tagged_cells) *tagged_cells = g->hctrl->last_tagged;
   if (g->hctrl->status == MSH_E_TIMEOUT)
-    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting for a bulk copy of its staged planes");
+    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting (a bulk copy of its staged planes, or a barrier between its stages)");
   if (g->hctrl->status == MSH_E_REALIZABILITY)
     return fail(MSH_E_REALIZABILITY, "step produced a non-realizable cell %lld", (long long)g->hctrl->first_bad);
   return MSH_OK;
@@ -1327,7 +1329,7 @@ msh_status msh_step_end(msh_grid *g, int32_t *tagged_cells) {
   g->dt_stale = false;
   if (tagged_cells) *tagged_cells = g->hctrl->last_tagged;
   if (g->hctrl->status == MSH_E_TIMEOUT)
-    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting for a bulk copy of its staged planes");
+    return fail(MSH_E_TIMEOUT, "a step kernel gave up waiting (a bulk copy of its staged planes, or a barrier between its stages)");
   if (g->hctrl->status == MSH_E_REALIZABILITY)
     return fail(MSH_E_REALIZABILITY, "step produced a non-realizable cell %lld", (long long)g->hctrl->first_bad);
   return MSH_OK;
@@ -1482,6 +1484,9 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   for (int r : rows_c)
     for (int z : zcs)
       if (!(r == 16 && g->ndim == 3 && g->prec == MSH_FP64)) cands.push_back({r, z});
+  // the shape the grid has (the default's chunk need not be among the ones above)
+  if (std::find(cands.begin(), cands.end(), std::make_pair(g->rows, g->zchunk)) == cands.end())
+    cands.push_back({g->rows, g->zchunk});
   // the staged step is a candidate of its own (0, 0) where the grid's size allows it
   g->tiling_set = false;
   if (use_staged(g)) cands.push_back({0, 0});
