@@ -211,3 +211,30 @@ def test_iterated_fallback_tube_fp64(msh, oracle):
     assert ns == so and tg == to
     assert_fp64(g.get_state(), Uo.reshape(10, 1, 1, n), what="grid tube 3519")
     g.close()
+
+
+@pytest.mark.parametrize("prec,lengths", [
+    ("FP64", [29, 30, 31, 59, 60, 61, 91, 240, 241, 256, 257, 512, 513]),
+    ("FP32", [29, 30, 31, 59, 60, 61, 91, 481, 512, 513, 961, 1024, 1025]),
+])
+def test_segment_and_class_edges(msh, oracle, prec, lengths):
+    # lengths around the 30-cell segments of a warp and the limits of the length classes, all
+    # classes in one batch: the same bits as with one block size for all, and the oracle's states
+    tubes = _random_tubes(lengths, seed=47)
+    b = msh.Batch(tubes.length, tubes.WL, tubes.WR, tubes.t_end, tubes.cfl, getattr(msh, prec))
+    b.run()
+    U = b.get_state().copy()
+    W = b.get_state(msh.PRIMITIVE).astype(np.float64)
+    b.reset()
+    b.run(threads=128)
+    assert np.array_equal(U, b.get_state())
+    steps, _, _ = b.info()
+    for k in range(len(lengths)):
+        Uo, so, _, rc = _oracle_tube(oracle, tubes, k, np.float64 if prec == "FP64" else np.float32)
+        assert rc == 0
+        if prec == "FP64":
+            assert steps[k] == so
+            assert_fp64(b.tube(U, k), Uo, what=f"tube {k} (len {lengths[k]})")
+        else:
+            assert_fp32(b.tube(W, k), oracle.cons_to_prim(Uo), what=f"tube {k} (len {lengths[k]})")
+    b.close()
