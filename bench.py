@@ -308,9 +308,9 @@ def run_gpu(args):
     avg_kernel_s = (kms / kn) * 1e-3
     achieved = BYTES_PER_CELL["f32"] * ncells / avg_kernel_s / 1e9
     traffic = measured_traffic(ncells) if args.workload == "box" else None
-    # per step: step kernel, 4 fallback passes (idle unless cells were tagged), finalize;
-    # the graphs hold 16 steps, plus the run-start kernel
-    graph_launches = math.ceil(args.steps / 16) * 16 * 6 + 1
+    # per step: step kernel and finalize (the fallback passes are launched only once a step
+    # tagged cells, which the box never does); the graphs hold 16 steps, plus the run-start kernel
+    graph_launches = (args.steps if args.steps < 16 else math.ceil(args.steps / 16) * 16) * 2 + 1
     out = {
         "metric": "cell-updates/s", "value": value, "unit": "cell-updates/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -511,7 +511,7 @@ def run_suite(args):
         orc, cores, _ = _oracle_rate(p, steps=r["steps"])
         orc1, _ = _oracle_rate_1core(p, steps=r["steps"])
         # the same problem as one tube of the batched kernel: every step in one persistent
-        # launch (the grid path pays six launches per step, which a 256-cell step cannot hide)
+        # launch (the grid path takes its steps by one cooperative launch of the whole chip)
         WL, WR = p.W[:, 0, 0, 0], p.W[:, 0, 0, -1]
         b = msh.Batch([p.n[0]], WL[None, :], WR[None, :], p.t_end, p.cfl, msh.FP64, stream=stream.cuda_stream)
         b.run()
@@ -636,7 +636,7 @@ def tubes_rates(msh, inputs, stream, per_tube=True):
     import torch
     tb = inputs.tubes()
     b = msh.Batch(tb.length, tb.WL, tb.WR, tb.t_end, tb.cfl, msh.FP32, stream=stream.cuda_stream)
-    b.run()  # autotunes the block size
+    b.run()  # warm-up
     b.reset()
     torch.cuda.synchronize()
     t0 = time.perf_counter()
