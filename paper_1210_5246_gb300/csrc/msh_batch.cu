@@ -128,10 +128,79 @@ __device__ __forceinline__ T tube_pass(const T *src, T *dst, unsigned char *sFl,
   return smax;
 }
 
+// The same sweep chunk by chunk of NT cells, the face states and fluxes exchanged through shared
+// memory, for FP64 batches of more tubes than SMs: no cell is reconstructed twice (a segment
+// repeats 2 of its 32 lanes, and a double-precision instruction costs the same at any lane
+// count), and its three barriers per chunk cost little beside that pipe.  The update of a cell
+// runs one chunk position behind its reconstruction, when both its faces are known.
+template <typename T, int NT, bool FALLBACK>
+__device__ __forceinline__ T tube_pass_chunks(const T *src, T *dst, unsigned char *sFl, int n, int cap, T nu, T dtdx,
+                                              T idx, T *sF, T *sH, T *sHc, int *s_nbad, int *s_any) {
+  const int t = threadIdx.x;
+  T smax = T(0);
+  for (int b = -1; b <= n; b += NT) {
+    const int c = b + t;
+    T lo[NV], hi[NV], wm[NV];  // wm: W^n of the cell this thread updates (c - 1)
+    if (c <= n) {
+      T w0[NV], wp[NV];
+      load_w(src, cap, c - 1, n, wm);
+      load_w(src, cap, c, n, w0);
+      load_w(src, cap, c + 1, n, wp);
+      reconstruct(wm, w0, wp, nu, lo, hi);
+      if (FALLBACK) {  // tags of earlier passes (value 2) are active in this pass
+        auto f = [&](int i) { return sFl[min(max(i, 0), n - 1)] == 2; };
+        first_order_faces(f(c - 1), f(c), f(c + 1), w0, lo, hi);
+      }
+#pragma unroll
+      for (int v = 0; v < NV; v++) sH[v * NT + t] = hi[v];
+    }
+    __syncthreads();
+    if (c >= 0 && c <= n) {
+      T hl[NV], F[NV];
+#pragma unroll
+      for (int v = 0; v < NV; v++) hl[v] = (t > 0) ? sH[v * NT + t - 1] : sHc[v];
+      hll(hl, lo, F);
+#pragma unroll
+      for (int v = 0; v < NV; v++) sF[v * (NT + 1) + t + 1] = F[v];
+    }
+    __syncthreads();
+    // the last thread hands its upper face state to the next chunk (read after the next barrier;
+    // every read of the current one happened before the barrier above)
+    if (t == NT - 1 && c <= n) {
+#pragma unroll
+      for (int v = 0; v < NV; v++) sHc[v] = hi[v];
+    }
+    const int cu = c - 1;
+    if (cu >= 0 && cu < n) {
+      T U[NV], W[NV];
+      prim_to_cons(wm, U);
+#pragma unroll
+      for (int v = 0; v < NV; v++) U[v] -= dtdx * (sF[v * (NT + 1) + t + 1] - sF[v * (NT + 1) + t]);
+      cons_to_prim(U, W);
+#pragma unroll
+      for (int v = 0; v < NV; v++) dst[v * cap + cu] = W[v];
+      if (!realizable(W)) {
+        *s_any = 1;
+        if (sFl[cu] != 2) {
+          sFl[cu] = 1;
+          *s_nbad = 1;
+        }
+      }
+      smax = fmax(smax, tube_speed(W, idx));
+    }
+    __syncthreads();
+    if (t == 0) {  // the last face of this chunk is the lower face of the next chunk's first update
+#pragma unroll
+      for (int v = 0; v < NV; v++) sF[v * (NT + 1)] = sF[v * (NT + 1) + NT];
+    }
+  }
+  return smax;
+}
+
 // What the block does next with its tube (thread 0 decides between the passes).
 enum { TUBE_DONE = 0, TUBE_STEP = 1, TUBE_RETRY = 2 };
 
-template <typename T, int NT>
+template <typename T, int NT, bool CHUNKS>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tubes_kernel(TubeArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cap = a.cap;
@@ -139,7 +208,10 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
   // (the fallback passes re-read the untouched W^n), then the two swap roles
   T *sU = reinterpret_cast<T *>(smem_raw);  // [NV][cap]
   T *sUo = sU + (size_t)NV * cap;           // [NV][cap]
-  unsigned char *sFl = reinterpret_cast<unsigned char *>(sUo + (size_t)NV * cap);  // [cap] fallback tags
+  // chunk form: [NV][NT+1] fluxes (0: the one carried over), [NV][NT] upper face states, [NV] the
+  // one carried over
+  T *sF = sUo + (size_t)NV * cap, *sH = sF + (CHUNKS ? NV * (NT + 1) : 0), *sHc = sH + (CHUNKS ? NV * NT : 0);
+  unsigned char *sFl = reinterpret_cast<unsigned char *>(sHc + (CHUNKS ? NV : 0));  // [cap] fallback tags
   constexpr int kWarps = NT / 32;
   __shared__ T red[kWarps];
   __shared__ T s_dt;
@@ -242,9 +314,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
         for (int c = t; c < n; c += NT)
           if (sFl[c] == 1) sFl[c] = 2;  // tags of earlier passes become active
         __syncthreads();
-        smax = tube_pass<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
+        if constexpr (CHUNKS)
+          smax = tube_pass_chunks<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
+        else smax = tube_pass<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
       } else {
-        smax = tube_pass<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
+        if constexpr (CHUNKS)
+          smax = tube_pass_chunks<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
+        else smax = tube_pass<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
       }
     }
     for (int c = t; c < n; c += NT) {
@@ -265,26 +341,33 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
   }
 }
 
-template <typename T> size_t tube_smem(int cap) { return sizeof(T) * 2 * (size_t)NV * cap + (size_t)cap; }
+template <typename T> size_t tube_smem(int cap, int nt, bool chunks) {
+  return sizeof(T) * NV * (2 * (size_t)cap + (chunks ? 2 * nt + 2 : 0)) + (size_t)cap;
+}
 
-template <typename T, int NT> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, cudaStream_t s) {
-  const size_t smem = tube_smem<T>(a.cap);
-  cudaError_t e = cudaFuncSetAttribute(tubes_kernel<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T, int NT, bool CHUNKS> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, cudaStream_t s) {
+  const size_t smem = tube_smem<T>(a.cap, NT, CHUNKS);
+  cudaError_t e = cudaFuncSetAttribute(tubes_kernel<T, NT, CHUNKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tubes_kernel<T, NT>, NT, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tubes_kernel<T, NT, CHUNKS>, NT, smem);
   if (e != cudaSuccess) return e;
   const int blocks = std::min(sms * std::max(1, per_sm), (int)(a.last - a.first));
-  tubes_kernel<T, NT><<<blocks, NT, smem, s>>>(a);
+  tubes_kernel<T, NT, CHUNKS><<<blocks, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_tubes(const TubeArgs<T> &a, int nt, cudaStream_t s) {
-  if (nt == 64) return launch_tubes_nt<T, 64>(a, s);
-  if (nt == 128) return launch_tubes_nt<T, 128>(a, s);
-  if (nt == 512) return launch_tubes_nt<T, 512>(a, s);
-  return launch_tubes_nt<T, 256>(a, s);
+template <typename T> cudaError_t launch_tubes(const TubeArgs<T> &a, int nt, bool chunks, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {  // 256 threads at most: 512 would not leave room for the longest tubes
+    if (chunks && nt == 64) return launch_tubes_nt<T, 64, true>(a, s);
+    if (chunks && nt == 128) return launch_tubes_nt<T, 128, true>(a, s);
+    if (chunks && nt == 256) return launch_tubes_nt<T, 256, true>(a, s);
+  }
+  if (nt == 64) return launch_tubes_nt<T, 64, false>(a, s);
+  if (nt == 128) return launch_tubes_nt<T, 128, false>(a, s);
+  if (nt == 512) return launch_tubes_nt<T, 512, false>(a, s);
+  return launch_tubes_nt<T, 256, false>(a, s);
 }
 
 }  // namespace msh
@@ -367,16 +450,19 @@ msh_status upload_initial(msh_batch *b) {
 // A class of tubes: order[first .. last) on blocks of nt threads.
 struct TubeClass {
   int first, last, nt;
+  bool chunks;  // tube_pass_chunks
 };
 
 // threads > 0: every tube on blocks of that size.  0: by length.  FP32: 16 warps per tube above
 // 1024 cells, 8 above 512, 4 below (each class fills an SM with 16 warps); FP64, whose buffers
 // are twice as large and whose pipe two warps per scheduler saturate: 8, 4 and 2 warps at half
-// the lengths.
+// the lengths.  Batches too small to fill the SMs so: a class takes twice the warps, longest
+// first, while all its tubes' warps still run at once and have segments to sweep (one FP64 tube of
+// 256 cells to t = 0.02: 210 us with 8 warps, ~330 with 2).
 std::vector<TubeClass> tube_classes(const msh_batch *b, int threads) {
   std::vector<TubeClass> cls;
   if (threads > 0) {
-    cls.push_back({0, b->ntubes, threads});
+    cls.push_back({0, b->ntubes, threads, false});
     return cls;
   }
   const bool f32 = b->prec == MSH_FP32;
@@ -385,16 +471,41 @@ std::vector<TubeClass> tube_classes(const msh_batch *b, int threads) {
   for (int i = 0; i < 3; i++) {
     int end = at;
     while (end < b->ntubes && b->len[b->order[end]] > above[i]) end++;
-    if (end > at) cls.push_back({at, end, nt[i]});
+    if (end > at) cls.push_back({at, end, nt[i], false});
     at = end;
   }
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return cls;
+  }
+  // FP64 with more tubes than SMs: the double-precision pipes are full, and a sweep that repeats no
+  // cell counts for more than one without barriers (1216 tubes of up to 256 cells: 3.99 ms against
+  // 4.54 by segments; 152 tubes, one per SM: segments 1.57 ms, chunks 1.80).  64-thread blocks only
+  // where the queue has more tubes than blocks to level them with (600 tubes at once: 3.18 ms, 2.76 with
+  // 128 threads).
+  if (!f32 && b->ntubes > sms) {
+    for (TubeClass &c : cls) {
+      c.chunks = true;
+      if (c.nt == 64 && c.last - c.first <= 4 * sms) c.nt = 128;
+    }
+    return cls;
+  }
+  long long room = (long long)sms * (f32 ? 16 : 8);  // warps that run at once
+  for (const TubeClass &c : cls) room -= (long long)(c.last - c.first) * (c.nt / 32);
+  for (TubeClass &c : cls)
+    while (c.nt < nt[0] && c.nt / 32 * kTubeSeg < b->len[b->order[c.first]] &&
+           (long long)(c.last - c.first) * (c.nt / 32) <= room) {
+      room -= (long long)(c.last - c.first) * (c.nt / 32);
+      c.nt *= 2;
+    }
   return cls;
 }
 
 template <typename T> cudaError_t launch_class(msh_batch *b, const TubeClass &c, int i, int64_t max_steps, cudaStream_t s) {
   TubeArgs<T> a{(T *)b->U, b->d_off, b->d_len, b->d_tend, b->d_order, b->d_queue + i, c.first, c.last, b->d_steps, b->d_t,
                 b->d_status, b->d_fallback, b->total, b->len[b->order[c.first]], b->cfl, max_steps};
-  return launch_tubes<T>(a, c.nt, s);
+  return launch_tubes<T>(a, c.nt, c.chunks, s);
 }
 
 msh_status run_once(msh_batch *b, int threads, int64_t max_steps) {
@@ -533,7 +644,7 @@ msh_status msh_batch_run(msh_batch *b, int32_t threads, int64_t max_steps) {
   if (threads != 0 && threads != 128 && threads != 256 && threads != 512)
     return bfail(MSH_E_INVALID_ARG, "threads must be 0, 128, 256 or 512");
   if (max_steps < 1) return bfail(MSH_E_INVALID_ARG, "max_steps must be >= 1");
-  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap) : tube_smem<double>(b->cap);
+  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, 0, false) : tube_smem<double>(b->cap, 0, false);
   if (smem > 227 * 1024) return bfail(MSH_E_INVALID_ARG, "tubes too long for shared memory (%zu B)", smem);
   // one persistent launch per class of lengths, captured in a CUDA graph with the queue reset
   cudaGraph_t graph = nullptr;

@@ -238,3 +238,20 @@ def test_segment_and_class_edges(msh, oracle, prec, lengths):
         else:
             assert_fp32(b.tube(W, k), oracle.cons_to_prim(Uo), what=f"tube {k} (len {lengths[k]})")
     b.close()
+
+
+def test_fp64_batch_larger_than_the_chip(msh, oracle):
+    # more FP64 tubes than SMs sweep chunk by chunk through shared memory: lengths around the chunks
+    # of each class's blocks (64, 128, 256 cells, and two ghost cells) against the oracle
+    edges = [4, 61, 62, 63, 64, 126, 127, 190, 253, 254, 255, 256, 257, 382, 510, 511, 512, 513, 766, 1024]
+    tubes = _random_tubes(edges + [5] * 1300, seed=48)
+    tubes.t_end = 0.02
+    b = msh.Batch(tubes.length, tubes.WL, tubes.WR, tubes.t_end, tubes.cfl, msh.FP64)
+    b.run()
+    U = b.get_state()
+    steps, _, _ = b.info()
+    for k in range(len(edges) + 3):
+        Uo, so, _, rc = _oracle_tube(oracle, tubes, k)
+        assert rc == 0 and steps[k] == so
+        assert_fp64(b.tube(U, k), Uo, what=f"tube {k} (len {tubes.length[k]})")
+    b.close()
