@@ -457,8 +457,8 @@ msh_status msh_batch_destroy(msh_batch *b);
  * until the process exits; grids of more than 1,048,576 cells (or needing more than 16384
  * thread blocks) are rejected with MSH_E_INVALID_ARG.  The first call on a device looks up
  * that array's device address, so make the first call before any stream capture.  Every
- * call shares the array: each call clears what must start at zero, and calls that overlap
- * on the GPU (from other streams or host threads) race on it.  No cudaMalloc, cudaFree or
+ * call shares the array, and calls that overlap on the GPU (from other streams or host
+ * threads) race on it; a call after them that overlaps no other is right again.  No cudaMalloc, cudaFree or
  * other allocating routine is called.
  */
 msh_status msh_step_noalloc(int32_t ndim, const int64_t n[3], const double lo[3], const double hi[3],

@@ -9,9 +9,12 @@
 // partials, fallback tags) lives in one file-scope device array of fixed size that every
 // GPU holds from the moment it loads the library until the process exits.
 //
-// That array is shared by every call: each call clears what must start at zero (the
-// control block and the tags of its cells) before using it, and two calls whose work
-// overlaps on the GPU (other streams, other host threads) race on it.
+// That array is shared by every call, and two calls whose work overlaps on the GPU (other
+// streams, other host threads) race on it.  Every call writes the control block and clears
+// the tags of its cells before using them.  The scan's block counter must be zero when a
+// call starts; a call leaves it at zero, also calls that overlapped: their scans can mix
+// their counts, but every call's finalize stores zero again, and the last of these runs
+// after every scan, so that a later call that overlaps no other is right.
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -83,11 +86,12 @@ msh_status noalloc_step(int ndim, const int64_t n[3], const double dx[3], const 
   // data), sets up the control block and plans the step with dt = min(CFL dt, dt_max); a
   // non-realizable input leaves done = 1 and nothing is stepped.  The step and its finalize
   // follow; the fallback passes only if the host reads that cells were tagged.
-  const ScanEnd end = {ctrl, reinterpret_cast<unsigned *>(base + kNoallocCtrlBytes - 16), 1, cfl, dt_max};
+  unsigned *const scan_count = reinterpret_cast<unsigned *>(base + kNoallocCtrlBytes - 16);
+  const ScanEnd end = {ctrl, scan_count, 1, cfl, dt_max};
   Ctrl out;
   cudaError_t e = launch_scan<T>(Uin, nullptr, false, flags, N, ndim, dx, part, end, s);
   if (e == cudaSuccess) e = launch_step<T>(a, ndim, rows, false, s, nullptr);
-  if (e == cudaSuccess) e = launch_finalize(ctrl, part, nb, 2, s);
+  if (e == cudaSuccess) e = launch_finalize(ctrl, part, nb, 2, s, scan_count);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&out, ctrl, sizeof out, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess && out.done == 0) {  // cells were tagged: the finalize waited

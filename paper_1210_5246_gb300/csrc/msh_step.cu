@@ -120,9 +120,11 @@ __device__ void finalize_block(Ctrl *ctrl, const Partial *part, int nparts, int 
 }
 
 // mode 2: mode 0 unless the step tagged cells (the host then runs the fallback passes and mode
-// 0); mode 3: the same in the middle of a run, which stops there with kStatusPending
+// 0); mode 3: the same in the middle of a run, which stops there with kStatusPending.
+// scan_count: a scan counter to clear in any case (nullptr: none)
 __global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(Ctrl *ctrl, const Partial *part, int nparts,
-                                                                    int mode) {
+                                                                    int mode, unsigned *scan_count) {
+  if (scan_count != nullptr && threadIdx.x == 0) *scan_count = 0u;
   if (mode != 1 && ctrl->done) return;
   if (mode >= 2 && ctrl->nbad[0] != 0 && !ctrl->stage_timeout) {
     if (mode == 3 && threadIdx.x == 0) {
@@ -477,8 +479,9 @@ cudaError_t launch_gravity_field(const double *phi, T *acc, int ndim, int nx, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(Ctrl *ctrl, const Partial *part, int nparts, int mode, cudaStream_t s) {
-  finalize_kernel<<<1, kFinalizeThreads, 0, s>>>(ctrl, part, nparts, mode);
+cudaError_t launch_finalize(Ctrl *ctrl, const Partial *part, int nparts, int mode, cudaStream_t s,
+                            unsigned *scan_count) {
+  finalize_kernel<<<1, kFinalizeThreads, 0, s>>>(ctrl, part, nparts, mode, scan_count);
   return cudaGetLastError();
 }
 

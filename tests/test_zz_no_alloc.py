@@ -113,3 +113,40 @@ def test_noalloc_rejects_non_realizable_input(msh):
     assert msh.msh_step_noalloc(n, lo, hi, bc, msh.FP64, 0.5, u0, u1) > 0
     assert bool(torch.isfinite(u1).all()) and not bool((u1 == 7.0).any())
 
+
+
+def test_noalloc_is_right_again_after_overlapping_calls(msh):
+    """Two host threads step buffers of their own at the same time: the calls race on the shared
+    scratch and their results are undefined.  A call after them that overlaps no other gives the
+    bits and the time step of the call before them."""
+    import threading
+    import torch
+    n, lo, hi, bc = (512, 384), (0.0, 0.0), (1.0, 1.0), ((0, 0), (1, 1))
+    W = _state((1, n[1], n[0]), seed=3)
+    g = msh.Grid(n, lo, hi, bc, 0.5, msh.FP32)
+    g.set_state(W.astype(np.float32), msh.PRIMITIVE)
+    u0 = torch.tensor(g.get_state(), device="cuda")
+    g.close()
+    want, got = torch.empty_like(u0), torch.empty_like(u0)
+    dt = msh.msh_step_noalloc(n, lo, hi, bc, msh.FP32, 0.5, u0, want)
+    torch.cuda.synchronize()
+
+    def loop(a, b, stream):
+        for _ in range(100):
+            try:
+                msh.msh_step_noalloc(n, lo, hi, bc, msh.FP32, 0.5, a, b, stream=stream.cuda_stream)
+            except msh.MshError:
+                pass
+
+    bufs = [(u0.clone(), torch.empty_like(u0), torch.cuda.Stream()) for _ in range(2)]
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=loop, args=b) for b in bufs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for _ in range(2):
+        got.zero_()
+        assert msh.msh_step_noalloc(n, lo, hi, bc, msh.FP32, 0.5, u0, got) == dt
+        assert bool((got == want).all())
