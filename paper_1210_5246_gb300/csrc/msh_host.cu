@@ -1128,6 +1128,7 @@ msh_status msh_set_tape(msh_grid *g, int32_t K, int64_t max_steps) {
   CUDA_TRY(cudaStreamSynchronize(g->stream));
   msh_status st = stop_tape(g);
   if (st) return st;
+  drop_graph(g);  // also one captured without a tape: the checkpoints are in the step arguments
   if (K == 0) {
     free_tape(g);
     return MSH_OK;

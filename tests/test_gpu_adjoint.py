@@ -228,3 +228,27 @@ def test_tape_errors(msh, oracle):
     assert ei.value.status == msh.MSH_E_STATE
     g.set_tape(0, 0)  # frees
     g.close()
+
+
+def test_tape_set_after_runs_without_one(msh):
+    """A streaming run of 16 steps or more captures its steps; a tape set after such runs is
+    recorded all the same: its adjoint equals the one from the state and the schedule, bit for
+    bit."""
+    n, steps = (60, 41), 20
+    rng = np.random.default_rng(17)
+    W = np.zeros((10, 1, n[1], n[0]))
+    W[0] = rng.uniform(0.8, 1.2, W.shape[1:])
+    W[1:4] = rng.uniform(-0.2, 0.2, (3,) + W.shape[1:])
+    W[4] = W[7] = W[9] = 1.0
+    g = msh.Grid(n, (0.0, 0.0), (1.0, 1.0), ((0, 0), (0, 0)), 0.4, msh.FP64)
+    g.set_tiling(8, 16)
+    g.set_state(W, msh.PRIMITIVE)
+    g.run(max_steps=steps)
+    U0 = g.get_state()
+    g.set_recording(steps)
+    g.set_tape(3, steps)
+    g.run(max_steps=steps)
+    dts = g.dt_history()
+    lam = rng.normal(size=U0.shape)
+    np.testing.assert_array_equal(g.adjoint_tape(lam), g.adjoint_run(U0, dts, lam, K=3))
+    g.close()
