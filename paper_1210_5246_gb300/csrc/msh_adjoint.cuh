@@ -243,10 +243,11 @@ __device__ __forceinline__ void eig_init_vjp(const Eig<T> &E, const EigBar<T> &E
 
 // Derivatives of the limited amplitude mc(l, r) with its forward selection frozen: 2 on the
 // smaller side, 1/2 on both where the central difference is taken, 0 for differences of
-// opposite sign (ties go to the left side, then to the centre).
+// opposite sign (ties go to the left side, then to the centre).  The signs are compared as the
+// forward limiter does, not by a product, which underflows where the limiter still gives a slope.
 __device__ __forceinline__ void mc_weights(float l, float r, float &fl, float &fr) {
   const float al = fabsf(l), ar = fabsf(r), c = fabsf(l + r);
-  const bool on = l * r > 0.0f, left = al <= ar, side = left ? 4.0f * al <= c : 4.0f * ar < c;
+  const bool on = (l > 0.0f && r > 0.0f) || (l < 0.0f && r < 0.0f), left = al <= ar, side = left ? 4.0f * al <= c : 4.0f * ar < c;
   fl = !on ? 0.0f : side ? (left ? 2.0f : 0.0f) : 0.5f;
   fr = !on ? 0.0f : side ? (left ? 0.0f : 2.0f) : 0.5f;
 }

@@ -252,3 +252,34 @@ def test_tape_set_after_runs_without_one(msh):
     lam = rng.normal(size=U0.shape)
     np.testing.assert_array_equal(g.adjoint_tape(lam), g.adjoint_run(U0, dts, lam, K=3))
     g.close()
+
+
+@pytest.mark.parametrize("prec,power", [("FP32", 60), ("FP64", 540)])
+@pytest.mark.parametrize("n,tiling", [((96,), None), ((96,), (8, 1)), ((33, 18), None), ((33, 18), (8, 4))])
+def test_adjoint_of_amplitudes_whose_products_underflow(msh, n, tiling, prec, power):
+    """A field at rest with uniform density and stresses and a small random transverse velocity:
+    the step is linear in that velocity (its square is below half an ulp of the stresses) and the
+    limiter's selection does not depend on a common factor, so the gradient with respect to the
+    transverse momentum and the shear stress is the same at any amplitude, to the last bit but
+    for underflow: here at 2^-30 and at 2^-(30 + power), where the product of two differences is
+    zero.  Bound: six steps of at most 200 roundings each, of the largest entry."""
+    nd, eps = len(n), 2.0 ** (-23 if prec == "FP32" else -52)
+    shape = (10,) + (1,) * (3 - nd) + n[::-1]
+    rng = np.random.default_rng(29)
+    r = rng.uniform(-1.0, 1.0, shape[1:])
+    lam = np.zeros(shape)
+    lam[3], lam[6] = rng.normal(size=(2,) + shape[1:])
+    got = []
+    for a in (2.0 ** -30, 2.0 ** -(30 + power)):
+        W = np.zeros(shape)
+        W[0] = W[4] = W[7] = W[9] = 1.0
+        W[3] = a * r  # z: transverse to every axis of a 1D or 2D grid
+        g = msh.Grid(n, (0.0,) * nd, (1.0,) * nd, ((0, 0),) * nd, 0.3, getattr(msh, prec))
+        if tiling:
+            g.set_tiling(*tiling)
+        g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+        dt = 0.3 / max(n) / 3.0 ** 0.5 / nd
+        got.append(g.adjoint_run(g.get_state(), [dt] * 6, lam.astype(g.dtype), K=3).astype(np.float64)[[3, 6]])
+        g.close()
+    assert np.abs(got[0] - got[1]).max() <= 1200 * eps * np.abs(got[0]).max()
+    assert np.abs(got[0][0] - lam[3]).max() > 0.01
