@@ -70,7 +70,7 @@ __device__ __forceinline__ double warp_max_speed(double v) {
 }
 
 template <typename T> __device__ __forceinline__ T tube_speed(const T (&W)[NV], T idx) {
-  return (fabs(W[1]) + T(1.7320508075688772) * sqrt_ratio(W[4], W[0])) * idx;
+  return signal_speed(W[1], W[4], W[0]) * idx;
 }
 
 // One sweep of a tube, segment by segment of kTubeSeg cells, the warps of the block taking

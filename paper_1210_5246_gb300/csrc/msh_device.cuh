@@ -37,16 +37,47 @@ template <> struct Frame<2> {
 
 // ---------------------------------------------------------- fast arithmetic
 // FP32: hardware approximate reciprocal and reciprocal square root (a few ulp, far
-// inside the FP32 tolerances).  FP64: IEEE division, and CUDA's rsqrt() (1 ulp) for the
-// square roots: a double-precision warp instruction holds its scheduler's pipe for 64 cycles
-// on GB300, and 1 / sqrt(x) took 930 of them where rsqrt(x) takes 377, sqrt(p / r) 1160 where
-// p rsqrt(p r) takes 505 (measured, independent chains).
+// inside the FP32 tolerances).  FP64: IEEE division, and CUDA's rsqrt() for the square roots:
+// a double-precision warp instruction holds its scheduler's pipe for 64 cycles on GB300, and
+// 1 / sqrt(x) took 930 of them where rsqrt(x) takes 377 (measured, independent chains; errors up
+// to 1.48 and 0.51 ulp over 2^20 values).
 template <typename T> __device__ __forceinline__ T frcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float frcp<float>(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double frsqrt(double x) { return rsqrt(x); }
-// sqrt(p / r) for p, r > 0
-template <typename T> __device__ __forceinline__ T sqrt_ratio(T p, T r) { return p * frsqrt(p * r); }
+// sqrt(p / r) for p, r > 0.  FP64: p rsqrt(p r), corrected by its residual p - s (s r) (s r with
+// its rounding error), where p and p r are far enough from the ends of the range that nothing
+// under- or overflows, and otherwise the square root of the quotient: 828 pipe cycles and errors
+// up to 0.50 ulp, where the quotient's root takes 1159 (0.85 ulp) and p rsqrt(p r) alone 522 (1.67
+// ulp, and infinite or zero once p r under- or overflows).
+__device__ __forceinline__ float sqrt_ratio(float p, float r) { return p * rsqrtf(p * r); }
+static __device__ __noinline__ double sqrt_quotient(double p, double r) { return sqrt(p / r); }
+__device__ __forceinline__ double sqrt_ratio(double p, double r) {
+  const double q = p * r;
+  const unsigned ep = (unsigned)__double2hiint(p) - 0x04000000u, eq = (unsigned)__double2hiint(q) - 0x04000000u;
+  if (__builtin_expect(max(ep, eq) >= 0x78000000u, 0)) return sqrt_quotient(p, r);  // (also p <= 0 and NaN)
+  const double y = rsqrt(q), s = p * y, h = s * r, l = fma(s, r, -h);
+  const double e = fma(-s, l, fma(-s, h, p));
+  return fma(e, __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y)), s);  // s + e y / 2
+}
+// u - c and u + c, and |u| + c, with c = sqrt(3 p / r).  FP64 states its multiply-adds: the branch
+// of sqrt_ratio leaves the compiler a choice, and every kernel has to round alike.
+__device__ __forceinline__ void acoustic(float u, float p, float r, float &lo, float &hi) {
+  const float c = 1.7320508075688772f * sqrt_ratio(p, r);
+  lo = u - c;
+  hi = u + c;
+}
+__device__ __forceinline__ void acoustic(double u, double p, double r, double &lo, double &hi) {
+  const double q = sqrt_ratio(p, r);
+  lo = fma(-1.7320508075688772, q, u);
+  hi = fma(1.7320508075688772, q, u);
+}
+__device__ __forceinline__ float signal_speed(float u, float p, float r) {
+  return fabsf(u) + 1.7320508075688772f * sqrt_ratio(p, r);
+}
+__device__ __forceinline__ double signal_speed(double u, double p, double r) {
+  return fma(1.7320508075688772, sqrt_ratio(p, r), fabs(u));
+}
 
 // x > 0, x >= 0 and min / max.  FP64: on the bit patterns (integer instructions; the
 // double-precision compare runs on the 64-cycle pipe).  A NaN is neither > 0 nor >= 0; the
@@ -511,10 +542,10 @@ template <typename T>
 __device__ __forceinline__ void cons_pi(const T (&w)[NV], T (&U)[NV], T (&P)[NV]);
 template <typename T>
 __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
-  const T cl = T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
-  const T cr = T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
-  const T SL = min_of(wl[1] - cl, wr[1] - cr);
-  const T SR = max_of(wl[1] + cl, wr[1] + cr);
+  T lo_l, hi_l, lo_r, hi_r;
+  acoustic(wl[1], wl[4], wl[0], lo_l, hi_l);
+  acoustic(wr[1], wr[4], wr[0], lo_r, hi_r);
+  const T SL = min_of(lo_l, lo_r), SR = max_of(hi_l, hi_r);
   // F = a Fl + b Fr + c (Ur - Ul): (1, 0, 0) for SL >= 0, (0, 1, 0) for SR <= 0, else
   // (SR, -SL, SL SR) / (SR - SL); the branch selects three scalars, not ten fluxes
   T a, b, c;
@@ -568,12 +599,11 @@ __device__ __forceinline__ void kt_reconstruct(const T (&wm)[NV], const T (&w0)[
 // |u_n| + sqrt(3 P_nn / rho), of the two (eqs spectralfreq, soundspeed with gamma = 3).
 template <typename T>
 __device__ __forceinline__ void kt_flux(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
-  T Ul[NV], Fl[NV], Ur[NV], Fr[NV];
+  const T al = signal_speed(wl[1], wl[4], wl[0]), ar = signal_speed(wr[1], wr[4], wr[0]);
+  const T h = T(0.5) * fmax(al, ar);
+  T Ul[NV], Fl[NV], Ur[NV], Fr[NV];  // after the speeds' branches, so that it rounds alike everywhere
   phys(wl, Ul, Fl);
   phys(wr, Ur, Fr);
-  const T al = fabs(wl[1]) + T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
-  const T ar = fabs(wr[1]) + T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
-  const T h = T(0.5) * fmax(al, ar);
   T dU[NV], Fs[NV];
   v_sub(dU, Ur, Ul);
   v_add(Fs, Fl, Fr);
@@ -670,10 +700,10 @@ template <typename T> __device__ __forceinline__ void cons_pi(const T (&w)[NV], 
 // not strictly inside (S_L, S_R) the flux is HLL's.
 template <typename T>
 __device__ __forceinline__ void hllc_flux(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
-  const T cl = T(1.7320508075688772) * sqrt_ratio(wl[4], wl[0]);
-  const T cr = T(1.7320508075688772) * sqrt_ratio(wr[4], wr[0]);
-  const T SL = min_of(wl[1] - cl, wr[1] - cr);
-  const T SR = max_of(wl[1] + cl, wr[1] + cr);
+  T lo_l, hi_l, lo_r, hi_r;
+  acoustic(wl[1], wl[4], wl[0], lo_l, hi_l);
+  acoustic(wr[1], wr[4], wr[0], lo_r, hi_r);
+  const T SL = min_of(lo_l, lo_r), SR = max_of(hi_l, hi_r);
   const T CL = wl[0] * (SL - wl[1]), CR = wr[0] * (SR - wr[1]);
   const T inv = frcp(CR - CL);
   T us[3], ps[3];

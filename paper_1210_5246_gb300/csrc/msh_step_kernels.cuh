@@ -190,14 +190,14 @@ __device__ __forceinline__ void block_partial(S (&diag)[NV], double smax, long l
 // MAXF (the corner-transport-upwind step): the maximum over the dims instead of the sum.
 template <typename T, int NDIM, bool MAXF = false>
 __device__ __forceinline__ T speed_sum(const T (&W)[NV], T idx, T idy, T idz) {
-  T s = (fabs(W[1]) + sqrt_ratio(W[4], W[0]) * T(1.7320508075688772)) * idx;
+  T s = signal_speed(W[1], W[4], W[0]) * idx;
   if (NDIM > 1) {
-    const T sy = (fabs(W[2]) + sqrt_ratio(W[7], W[0]) * T(1.7320508075688772)) * idy;
-    s = MAXF ? fmax(s, sy) : s + sy;
+    const T y = signal_speed(W[2], W[7], W[0]);
+    s = MAXF ? fmax(s, y * idy) : fma(y, idy, s);
   }
   if (NDIM > 2) {
-    const T sz = (fabs(W[3]) + sqrt_ratio(W[9], W[0]) * T(1.7320508075688772)) * idz;
-    s = MAXF ? fmax(s, sz) : s + sz;
+    const T z = signal_speed(W[3], W[9], W[0]);
+    s = MAXF ? fmax(s, z * idz) : fma(z, idz, s);
   }
   return s;
 }
