@@ -535,11 +535,9 @@ __device__ __forceinline__ void phys(const T (&w)[NV], T (&U)[NV], T (&F)[NV]) {
 
 // HLL flux between local-frame face states wl | wr with signal speeds
 // S_L = min(u_L - cf_L, u_R - cf_R), S_R = max(u_L + cf_L, u_R + cf_R).
-// FP32 adds the two sides' physical fluxes and conserved states in packed instructions; FP64,
-// which pays per operation, uses F_K = u_K U_K + Pi_K (pi_terms), 84 instead of 98 operations
-// after the signal speeds.
-template <typename T>
-__device__ __forceinline__ void cons_pi(const T (&w)[NV], T (&U)[NV], T (&P)[NV]);
+// The difference U_R - U_L is formed first, so that its term vanishes between equal states; with
+// U_L and U_R weighted separately FP64 saves 14 of 98 operations (3 % of a step), but the mass flux
+// through a wall or in a gas at rest is then a rounding error of c rho instead of zero.
 template <typename T>
 __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
   T lo_l, hi_l, lo_r, hi_r;
@@ -558,16 +556,6 @@ __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)
     a = SR * inv;
     b = -SL * inv;
     c = SL * SR * inv;
-  }
-  if constexpr (sizeof(T) == 8) {
-    T Ul[NV], Pl[NV], Ur[NV], Pr[NV];
-    cons_pi(wl, Ul, Pl);
-    cons_pi(wr, Ur, Pr);
-    const T al = fma(a, wl[1], -c), br = fma(b, wr[1], c);
-    F[0] = fma(al, Ul[0], br * Ur[0]);
-#pragma unroll
-    for (int k = 1; k < NV; k++) F[k] = fma(al, Ul[k], fma(br, Ur[k], fma(a, Pl[k], b * Pr[k])));
-    return;
   }
   T Ul[NV], Fl[NV], Ur[NV], Fr[NV], t[NV];
   phys(wl, Ul, Fl);
@@ -679,12 +667,6 @@ __device__ __forceinline__ void pi_terms(T u, T v, T w, T pxx, T pxy, T pxz, T (
   P[7] = T(2) * pxy * v;
   P[8] = pxy * w + pxz * v;
   P[9] = T(2) * pxz * w;
-}
-
-// Conserved state and Pi of a local-frame primitive state.
-template <typename T> __device__ __forceinline__ void cons_pi(const T (&w)[NV], T (&U)[NV], T (&P)[NV]) {
-  prim_to_cons(w, U);
-  pi_terms(w[1], w[2], w[3], w[4], w[5], w[6], P);
 }
 
 // Three-wave HLLC flux for the ten-moment system (local frame).  Outer waves S_L, S_R as in
