@@ -30,3 +30,27 @@ def test_fp64_cfl_step_over_the_range(msh, rho, P):
     g.close()
     want = np.longdouble(cfl) / n / np.sqrt(np.longdouble(3) * np.longdouble(P) / np.longdouble(rho))
     assert ok and abs(np.longdouble(dt) - want) <= 3 * 2.0 ** -52 * want
+
+
+@pytest.mark.parametrize("n,tiling", [((96, 70), (4, 8)), ((96, 70), (16, 16)), ((40, 30, 20), (8, 0)), ((40, 30, 20), (16, 5)),
+                                      ((500,), (8, 1))])
+def test_fp32_totals_beyond_the_fp32_range(msh, n, tiling):
+    """Totals of a uniform FP32 state with a field (zz stress, in 3D the density) that is
+    representable in every cell and summed over a thread's, but not over a warp's: the totals are
+    FP64 sums (a thread's FP32 sum of at most 20 equal cells rounds by 20 2^-24 at most)."""
+    nd = len(n)
+    big = 1e38 if nd == 1 else 1e37
+    W = np.zeros((10,) + (1,) * (3 - nd) + n[::-1])
+    W[0] = W[4] = W[7] = 1.0
+    W[9] = 1.0
+    W[9 if nd < 3 else 0] = big
+    g = msh.Grid(n, (0.0,) * nd, (1.0,) * nd, ((0, 0),) * nd, 0.3, msh.FP32)
+    g.set_tiling(*tiling)
+    g.set_state(W.astype(np.float32), msh.PRIMITIVE)
+    g.run(max_steps=2)
+    tot, ok, _ = g.diagnostics()
+    U = g.get_state().astype(np.float64)
+    g.close()
+    want = U.reshape(10, -1).sum(axis=1)
+    assert ok and np.isfinite(tot).all()
+    assert (np.abs(tot - want) <= 20 * 2.0 ** -24 * np.abs(U).reshape(10, -1).sum(axis=1)).all()
