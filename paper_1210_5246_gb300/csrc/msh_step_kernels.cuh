@@ -198,16 +198,19 @@ __device__ __forceinline__ void block_partial(S (&diag)[NV], double smax, long l
 
 // Sum over active dims of (|u_d| + sqrt(3 P_dd / rho)) / dx_d: the CFL signal-speed sum.
 // MAXF (the corner-transport-upwind step): the maximum over the dims instead of the sum.
+// FP64 states its multiply-add (see acoustic).
+__device__ __forceinline__ float add_product(float s, float a, float b) { return s + a * b; }
+__device__ __forceinline__ double add_product(double s, double a, double b) { return fma(a, b, s); }
 template <typename T, int NDIM, bool MAXF = false>
 __device__ __forceinline__ T speed_sum(const T (&W)[NV], T idx, T idy, T idz) {
   T s = signal_speed(W[1], W[4], W[0]) * idx;
   if (NDIM > 1) {
     const T y = signal_speed(W[2], W[7], W[0]);
-    s = MAXF ? fmax(s, y * idy) : fma(y, idy, s);
+    s = MAXF ? fmax(s, y * idy) : add_product(s, y, idy);
   }
   if (NDIM > 2) {
     const T z = signal_speed(W[3], W[9], W[0]);
-    s = MAXF ? fmax(s, z * idz) : fma(z, idz, s);
+    s = MAXF ? fmax(s, z * idz) : add_product(s, z, idz);
   }
   return s;
 }
