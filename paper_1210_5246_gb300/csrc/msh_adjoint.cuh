@@ -11,7 +11,7 @@ namespace msh {
 // W = W(U): rho, u = m/rho, P = E - m m^T / rho.  Accumulates Ub += (dW/dU)^T Wb.
 template <typename T>
 __device__ __forceinline__ void cons_to_prim_vjp(const T (&U)[NV], const T (&Wb)[NV], T (&Ub)[NV]) {
-  const T ir = frcp(U[0]);
+  const T ir = T(1) / U[0];
   const T u0 = U[1] * ir, u1 = U[2] * ir, u2 = U[3] * ir;
   Ub[0] += Wb[0] - (Wb[1] * u0 + Wb[2] * u1 + Wb[3] * u2) * ir + Wb[4] * u0 * u0 + Wb[5] * u0 * u1 +
            Wb[6] * u0 * u2 + Wb[7] * u1 * u1 + Wb[8] * u1 * u2 + Wb[9] * u2 * u2;
@@ -90,11 +90,10 @@ __device__ __forceinline__ void hll_vjp(const T (&wl)[NV], const T (&wr)[NV], co
   T Ul[NV], Fl[NV], Ur[NV], Fr[NV];
   phys(wl, Ul, Fl);
   phys(wr, Ur, Fr);
-  // c = sqrt(3 P / rho) = sqrt(3) P s, s = 1 / sqrt(P rho)
-  const T sl = frsqrt(wl[4] * wl[0]), sr = frsqrt(wr[4] * wr[0]);
-  const T cl = T(1.7320508075688772) * (wl[4] * sl);
-  const T cr = T(1.7320508075688772) * (wr[4] * sr);
-  const T aL = wl[1] - cl, aR = wr[1] - cr, bL = wl[1] + cl, bR = wr[1] + cr;
+  const T ql = sqrt_ratio(wl[4], wl[0]), qr = sqrt_ratio(wr[4], wr[0]);
+  T aL, bL, aR, bR;
+  acoustic(wl[1], ql, aL, bL);
+  acoustic(wr[1], qr, aR, bR);
   const T SL = min_of(aL, aR), SR = max_of(bL, bR);
   T zero[NV];
 #pragma unroll
@@ -107,33 +106,34 @@ __device__ __forceinline__ void hll_vjp(const T (&wl)[NV], const T (&wr)[NV], co
     phys_vjp(wr, zero, Fb, wrb);
     return;
   }
-  // F = (SR Fl - SL Fr + SL SR dU) inv: the speeds' adjoints need three sums over the fields
-  const T inv = frcp(SR - SL);
+  // F = (SR Fl - SL Fr + SL SR dU) inv, dU = Ur - Ul, dF = Fr - Fl:
+  //   dF/dSR = SL (dF - SL dU) inv^2,  dF/dSL = -SR (dF - SR dU) inv^2,
+  // so the speeds' adjoints need two sums of differences over the fields (half the rounding error of
+  // sums with F itself; sums of Fl, Fr and dU cancel against each other)
+  const T inv = T(1) / (SR - SL);
   const T ca = SR * inv, cb = -SL * inv, cc = SL * SR * inv;
   T Flb[NV], Frb[NV], Urb[NV], Ulb[NV];
-  T X = T(0), Y = T(0), Z = T(0);
+  T X = T(0), Z = T(0);
 #pragma unroll
   for (int k = 0; k < NV; k++) {
-    X = fma(Fb[k], Fl[k], X);
-    Y = fma(Fb[k], Fr[k], Y);
+    X = fma(Fb[k], Fr[k] - Fl[k], X);
     Z = fma(Fb[k], Ur[k] - Ul[k], Z);
     Flb[k] = ca * Fb[k];
     Frb[k] = cb * Fb[k];
     Urb[k] = cc * Fb[k];
     Ulb[k] = -Urb[k];
   }
-  const T G = ca * X + cb * Y + cc * Z;  // sum of Fb F
-  const T SRb = inv * (X + SL * Z - G), SLb = inv * (SR * Z - Y + G);
+  const T inv2 = inv * inv;
+  const T SRb = SL * inv2 * (X - SL * Z), SLb = -SR * inv2 * (X - SR * Z);
   T clb = T(0), crb = T(0);
   if (!gt0(aL - aR)) { wlb[1] += SLb; clb -= SLb; } else { wrb[1] += SLb; crb -= SLb; }
   if (!gt0(bR - bL)) { wlb[1] += SRb; clb += SRb; } else { wrb[1] += SRb; crb += SRb; }
-  // dc/dP = c / (2 P) = (sqrt(3)/2) s,  dc/drho = -c / (2 rho) = -(sqrt(3)/2) s P / rho, where
-  // P / rho = (P s)^2
-  const T hl = T(0.8660254037844386) * sl, hr = T(0.8660254037844386) * sr, ql = wl[4] * sl, qr = wr[4] * sr;
-  wlb[4] += clb * hl;
-  wlb[0] -= clb * hl * (ql * ql);
-  wrb[4] += crb * hr;
-  wrb[0] -= crb * hr * (qr * qr);
+  // c = sqrt(3 P / rho) = sqrt(3) q: dc/dP = c / (2 P), dc/drho = -c / (2 rho)
+  const T hl = clb * (T(0.8660254037844386) * ql), hr = crb * (T(0.8660254037844386) * qr);
+  wlb[4] += hl / wl[4];
+  wlb[0] -= hl / wl[0];
+  wrb[4] += hr / wr[4];
+  wrb[0] -= hr / wr[0];
   phys_vjp(wl, Ulb, Flb, wlb);
   phys_vjp(wr, Urb, Frb, wrb);
 }
@@ -221,14 +221,13 @@ __device__ __forceinline__ void back_vjp(const Eig<T> &E, const T (&c)[NV], cons
 // Reverse of Eig::init: adds the adjoints of the eigen-quantities into w0b (local frame).
 template <typename T>
 __device__ __forceinline__ void eig_init_vjp(const Eig<T> &E, const EigBar<T> &Eb, T (&w0b)[NV]) {
-  const T q = E.cs * E.cs;        // P_xx / rho
-  const T rs = T(2) * E.ics2;     // 1 / cs
-  const T ir = q * E.ip;          // 1 / rho
+  // with q = P_xx / rho, cs = sqrt(q): csb on cs and rsb on 1 / cs give q the adjoint
+  // (csb - rsb / q) / (2 cs) = t / cs, and P_xx and rho its multiples by 1 / rho and -q / rho
   const T csb = Eb.cs + T(1.7320508075688772) * Eb.cf;
-  const T rsb = T(0.28867513459481287) * Eb.icf2 + T(0.5) * Eb.ics2 + csb * q;
-  const T qb = csb * rs - T(0.5) * rsb * rs * (rs * rs);
-  T Pxxb = Eb.Pxx + qb * ir;
-  const T rhob = Eb.rho - qb * q * ir;
+  const T rsb = T(0.28867513459481287) * Eb.icf2 + T(0.5) * Eb.ics2;
+  const T t = T(0.5) * (csb - rsb * (E.rho * E.ip));
+  T Pxxb = Eb.Pxx + t * (E.cs * E.ip);
+  const T rhob = Eb.rho - t * E.cs / E.rho;
   const T ipb = Eb.ip + Eb.a * E.Pxy + Eb.b * E.Pxz;
   Pxxb -= ipb * E.ip * E.ip;
   w0b[0] += rhob;

@@ -60,15 +60,14 @@ __device__ __forceinline__ double sqrt_ratio(double p, double r) {
   const double e = fma(-s, l, fma(-s, h, p));
   return fma(e, __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y)), s);  // s + e y / 2
 }
-// u - c and u + c, and |u| + c, with c = sqrt(3 p / r).  FP64 states its multiply-adds: the branch
+// u - c and u + c, and |u| + c, with c = sqrt(3 p / r), q = sqrt(p / r).  FP64 states its multiply-adds: the branch
 // of sqrt_ratio leaves the compiler a choice, and every kernel has to round alike.
-__device__ __forceinline__ void acoustic(float u, float p, float r, float &lo, float &hi) {
-  const float c = 1.7320508075688772f * sqrt_ratio(p, r);
+__device__ __forceinline__ void acoustic(float u, float q, float &lo, float &hi) {
+  const float c = 1.7320508075688772f * q;
   lo = u - c;
   hi = u + c;
 }
-__device__ __forceinline__ void acoustic(double u, double p, double r, double &lo, double &hi) {
-  const double q = sqrt_ratio(p, r);
+__device__ __forceinline__ void acoustic(double u, double q, double &lo, double &hi) {
   lo = fma(-1.7320508075688772, q, u);
   hi = fma(1.7320508075688772, q, u);
 }
@@ -541,8 +540,8 @@ __device__ __forceinline__ void phys(const T (&w)[NV], T (&U)[NV], T (&F)[NV]) {
 template <typename T>
 __device__ __forceinline__ void hll(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
   T lo_l, hi_l, lo_r, hi_r;
-  acoustic(wl[1], wl[4], wl[0], lo_l, hi_l);
-  acoustic(wr[1], wr[4], wr[0], lo_r, hi_r);
+  acoustic(wl[1], sqrt_ratio(wl[4], wl[0]), lo_l, hi_l);
+  acoustic(wr[1], sqrt_ratio(wr[4], wr[0]), lo_r, hi_r);
   const T SL = min_of(lo_l, lo_r), SR = max_of(hi_l, hi_r);
   // F = a Fl + b Fr + c (Ur - Ul): (1, 0, 0) for SL >= 0, (0, 1, 0) for SR <= 0, else
   // (SR, -SL, SL SR) / (SR - SL); the branch selects three scalars, not ten fluxes
@@ -683,8 +682,8 @@ __device__ __forceinline__ void pi_terms(T u, T v, T w, T pxx, T pxy, T pxz, T (
 template <typename T>
 __device__ __forceinline__ void hllc_flux(const T (&wl)[NV], const T (&wr)[NV], T (&F)[NV]) {
   T lo_l, hi_l, lo_r, hi_r;
-  acoustic(wl[1], wl[4], wl[0], lo_l, hi_l);
-  acoustic(wr[1], wr[4], wr[0], lo_r, hi_r);
+  acoustic(wl[1], sqrt_ratio(wl[4], wl[0]), lo_l, hi_l);
+  acoustic(wr[1], sqrt_ratio(wr[4], wr[0]), lo_r, hi_r);
   const T SL = min_of(lo_l, lo_r), SR = max_of(hi_l, hi_r);
   const T CL = wl[0] * (SL - wl[1]), CR = wr[0] * (SR - wr[1]);
   const T inv = frcp(CR - CL);
