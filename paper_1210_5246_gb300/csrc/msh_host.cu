@@ -16,6 +16,9 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "../../include/msh.h"
 #include "msh_internal.h"
 
@@ -525,15 +528,37 @@ msh_status prime(msh_grid *g, int which) {
   return read_ctrl(g);
 }
 
-// Whether p points to memory of the current device that its kernels may read.
-bool device_readable(const void *p) {
+PFN_cuMemGetAddressRange_v3020 address_range() {
+  static const PFN_cuMemGetAddressRange_v3020 fn = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &p, 3020, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      return (PFN_cuMemGetAddressRange_v3020) nullptr;
+    }
+    return reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(p);
+  }();
+  return fn;
+}
+
+// Whether the kernels of the current device may read `bytes` bytes at p in elements of esize: its
+// own memory, aligned to the elements, and all of it in one allocation.  What they may not is copied,
+// which takes any address and reports a range that is not allocated as an error.
+bool device_readable(const void *p, size_t bytes, size_t esize) {
+  if (reinterpret_cast<uintptr_t>(p) % esize != 0) return false;
   cudaPointerAttributes at;
   int dev = -1;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     (void)cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == dev;
+  if (at.type != cudaMemoryTypeDevice || at.device != dev || address_range() == nullptr) return false;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr a = reinterpret_cast<CUdeviceptr>(p);
+  if (address_range()(&base, &size, a) != CUDA_SUCCESS) return false;
+  return a >= base && bytes <= size && a - base <= size - bytes;
 }
 
 int cur_buf(msh_grid *g) { return (int)(g->hctrl->step & 1); }
@@ -737,7 +762,7 @@ msh_status msh_set_state(msh_grid *g, const void *U, int32_t where, int32_t kind
   // it, checks it, clears the fallback tags (they are step numbers; a new state must not see
   // those of an earlier trajectory) and writes it to the spare buffer; if it is realizable the
   // device copies it on into the current one.
-  const bool direct = where == MSH_DEVICE && device_readable(U);
+  const bool direct = where == MSH_DEVICE && device_readable(U, bytes, g->esize);
   msh_status st = ensure_partials(g, kScanBlocks);
   if (st) return st;
   if (!direct)

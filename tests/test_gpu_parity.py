@@ -362,3 +362,30 @@ def test_fallback_inside_graphs(msh, oracle, shape, n, bc, cfl):
         g.close()
     assert_fp64(out[0], Uo, what=f"graph fallback {shape}")
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("prec,offset", [("FP64", 4), ("FP64", 1), ("FP32", 2), ("FP32", 4), ("FP64", 8)])
+def test_device_state_at_any_address(msh, prec, offset):
+    """A device buffer need not be aligned to its elements (C callers): the state set from it is
+    the one set from an aligned buffer, bit for bit."""
+    import ctypes
+    import torch
+    n = (37, 21)
+    g = msh.Grid(n, (0.0, 0.0), (1.0, 1.0), ((0, 0), (1, 1)), 0.4, getattr(msh, prec))
+    rng = np.random.default_rng(2)
+    W = np.zeros(g.shape)
+    W[0] = rng.uniform(0.8, 1.2, W.shape[1:])
+    W[1:4] = rng.uniform(-0.2, 0.2, (3,) + W.shape[1:])
+    W[4] = W[7] = W[9] = 1.0
+    W = W.astype(g.dtype)
+    g.set_state(W, msh.PRIMITIVE)
+    want = g.get_state()
+    raw = torch.from_numpy(np.frombuffer(W.tobytes(), dtype=np.uint8).copy())
+    buf = torch.zeros(raw.numel() + 64, dtype=torch.uint8, device="cuda")
+    buf[offset:offset + raw.numel()] = raw.cuda()
+    torch.cuda.synchronize()
+    g.set_state(np.ones_like(W) * W[:, :, :1, :1], msh.PRIMITIVE)
+    st = msh.load().msh_set_state(g.h, ctypes.c_void_p(buf.data_ptr() + offset), msh.DEVICE, msh.PRIMITIVE)
+    assert st == msh.MSH_OK, msh.msh_last_error()
+    np.testing.assert_array_equal(g.get_state(), want)
+    g.close()
