@@ -129,10 +129,16 @@ __device__ __forceinline__ T tube_pass(const T *src, T *dst, unsigned char *sFl,
 }
 
 // The same sweep chunk by chunk of NT cells, the face states and fluxes exchanged through shared
-// memory, for FP64 batches of more tubes than SMs: no cell is reconstructed twice (a segment
-// repeats 2 of its 32 lanes, and a double-precision instruction costs the same at any lane
-// count), and its three barriers per chunk cost little beside that pipe.  The update of a cell
+// memory (FP64): no cell is reconstructed twice, at three barriers per chunk.  The update of a cell
 // runs one chunk position behind its reconstruction, when both its faces are known.
+//
+// Which of the two sweeps is the faster one follows from the most loaded scheduler: a
+// double-precision instruction costs the same at any lane count, and of n cells segments of 30 leave
+// it ceil(ceil(n / 30) / 4) groups of 32 lanes, chunks of n + 2 positions ceil((n + 2) / 128).  FP64
+// tubes take chunks where that is fewer (n = 121 .. 126, 241 .. 254, 481 .. 510 ...) and segments, which
+// need no barriers, otherwise (blocks of 8 warps, one per SM: 64 tubes of 240 to 250 cells take 27 %
+// less time by chunks, 152 tubes of 205 to 256 cells, the slowest of them of 256, 5 % more).
+__device__ __forceinline__ bool takes_chunks(int n) { return (n + 129) / 128 < (n + 119) / 120; }
 template <typename T, int NT, bool FALLBACK>
 __device__ __forceinline__ T tube_pass_chunks(const T *src, T *dst, unsigned char *sFl, int n, int cap, T nu, T dtdx,
                                               T idx, T *sF, T *sH, T *sHc, int *s_nbad, int *s_any) {
@@ -200,8 +206,9 @@ __device__ __forceinline__ T tube_pass_chunks(const T *src, T *dst, unsigned cha
 // What the block does next with its tube (thread 0 decides between the passes).
 enum { TUBE_DONE = 0, TUBE_STEP = 1, TUBE_RETRY = 2 };
 
-template <typename T, int NT, bool CHUNKS>
+template <typename T, int NT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tubes_kernel(TubeArgs<T> a) {
+  constexpr bool CHUNKS = sizeof(T) == 8;  // the chunk form too
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cap = a.cap;
   // two tube buffers (primitive): a step reads W^n from one and writes W^{n+1} to the other
@@ -226,6 +233,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
     const int k = a.order[q];
     const int n = a.len[k];
     const int64_t off = a.off[k];
+    const bool chunks = CHUNKS && takes_chunks(n);
     T *cur = sU, *nxt = sUo;  // W^n and W^{n+1} of the current step
     const T idx = (T)n, half_idx = T(0.5) * idx;
     T smax = T(0);  // signal speed of the initial state
@@ -314,11 +322,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
         for (int c = t; c < n; c += NT)
           if (sFl[c] == 1) sFl[c] = 2;  // tags of earlier passes become active
         __syncthreads();
-        if constexpr (CHUNKS)
+        if (CHUNKS && chunks)
           smax = tube_pass_chunks<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
         else smax = tube_pass<T, NT, true>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
       } else {
-        if constexpr (CHUNKS)
+        if (CHUNKS && chunks)
           smax = tube_pass_chunks<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, sF, sH, sHc, &s_nbad, &s_any);
         else smax = tube_pass<T, NT, false>(cur, nxt, sFl, n, cap, nu, dtdx, idx, &s_nbad, &s_any);
       }
@@ -341,33 +349,29 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 512 / NT : 256 / NT) tube
   }
 }
 
-template <typename T> size_t tube_smem(int cap, int nt, bool chunks) {
-  return sizeof(T) * NV * (2 * (size_t)cap + (chunks ? 2 * nt + 2 : 0)) + (size_t)cap;
+// FP64 blocks hold the chunk form's buffers too.
+template <typename T> size_t tube_smem(int cap, int nt) {
+  return sizeof(T) * NV * (2 * (size_t)cap + (sizeof(T) == 8 ? 2 * nt + 2 : 0)) + (size_t)cap;
 }
 
-template <typename T, int NT, bool CHUNKS> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, cudaStream_t s) {
-  const size_t smem = tube_smem<T>(a.cap, NT, CHUNKS);
-  cudaError_t e = cudaFuncSetAttribute(tubes_kernel<T, NT, CHUNKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T, int NT> static cudaError_t launch_tubes_nt(const TubeArgs<T> &a, cudaStream_t s) {
+  const size_t smem = tube_smem<T>(a.cap, NT);
+  cudaError_t e = cudaFuncSetAttribute(tubes_kernel<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tubes_kernel<T, NT, CHUNKS>, NT, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tubes_kernel<T, NT>, NT, smem);
   if (e != cudaSuccess) return e;
   const int blocks = std::min(sms * std::max(1, per_sm), (int)(a.last - a.first));
-  tubes_kernel<T, NT, CHUNKS><<<blocks, NT, smem, s>>>(a);
+  tubes_kernel<T, NT><<<blocks, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_tubes(const TubeArgs<T> &a, int nt, bool chunks, cudaStream_t s) {
-  if constexpr (sizeof(T) == 8) {  // 256 threads at most: 512 would not leave room for the longest tubes
-    if (chunks && nt == 64) return launch_tubes_nt<T, 64, true>(a, s);
-    if (chunks && nt == 128) return launch_tubes_nt<T, 128, true>(a, s);
-    if (chunks && nt == 256) return launch_tubes_nt<T, 256, true>(a, s);
-  }
-  if (nt == 64) return launch_tubes_nt<T, 64, false>(a, s);
-  if (nt == 128) return launch_tubes_nt<T, 128, false>(a, s);
-  if (nt == 512) return launch_tubes_nt<T, 512, false>(a, s);
-  return launch_tubes_nt<T, 256, false>(a, s);
+template <typename T> cudaError_t launch_tubes(const TubeArgs<T> &a, int nt, cudaStream_t s) {
+  if (nt == 64) return launch_tubes_nt<T, 64>(a, s);
+  if (nt == 128) return launch_tubes_nt<T, 128>(a, s);
+  if (nt == 512) return launch_tubes_nt<T, 512>(a, s);
+  return launch_tubes_nt<T, 256>(a, s);
 }
 
 }  // namespace msh
@@ -450,48 +454,46 @@ msh_status upload_initial(msh_batch *b) {
 // A class of tubes: order[first .. last) on blocks of nt threads.
 struct TubeClass {
   int first, last, nt;
-  bool chunks;  // tube_pass_chunks
 };
 
-// threads > 0: every tube on blocks of that size.  0: by length.  FP32: 16 warps per tube above
-// 1024 cells, 8 above 512, 4 below (each class fills an SM with 16 warps); FP64, whose buffers
-// are twice as large and whose pipe two warps per scheduler saturate: 8, 4 and 2 warps at half
-// the lengths.  Batches too small to fill the SMs so: a class takes twice the warps, longest
-// first, while all its tubes' warps still run at once and have segments to sweep (one FP64 tube of
-// 256 cells to t = 0.02: 210 us with 8 warps, ~330 with 2).
+// threads > 0: every tube on blocks of that size.  0: by length.
+// FP32: 16 warps per tube above 1024 cells, 8 above 512, 4 below (each class fills an SM with 16
+// warps).  Batches too small to fill the SMs so: a class takes twice the warps, longest first, while
+// all its tubes' warps still run at once and have segments to sweep.
+// FP64, whose buffers are twice as large and whose pipe two warps per scheduler saturate: 8 warps
+// per tube, one tube per SM; many short tubes take blocks of 4 warps (up to 126 cells, whose sweep
+// leaves one group of lanes to every scheduler) or 2, two or four per SM.  Times to t = 0.02 with
+// 2 / 4 / 8 warps: 220 tubes of 113 to 126 cells 0.64 / 0.46 / 0.44 ms, 600 of them 0.84 / 0.70 / 0.79;
+// 300 of 31 to 62 cells 0.28 / 0.19 / 0.21; 600 of 16 to 32 cells 0.146 / 0.144 / 0.20, 2000 of them
+// 0.20 / 0.29 / 0.50; 2000 of 31 to 62 cells 0.43 / 0.47 / 0.79.
 std::vector<TubeClass> tube_classes(const msh_batch *b, int threads) {
   std::vector<TubeClass> cls;
   if (threads > 0) {
-    cls.push_back({0, b->ntubes, threads, false});
+    cls.push_back({0, b->ntubes, threads});
     return cls;
-  }
-  const bool f32 = b->prec == MSH_FP32;
-  const int above[3] = {f32 ? 1024 : 512, f32 ? 512 : 256, 0}, nt[3] = {f32 ? 512 : 256, f32 ? 256 : 128, f32 ? 128 : 64};
-  int at = 0;
-  for (int i = 0; i < 3; i++) {
-    int end = at;
-    while (end < b->ntubes && b->len[b->order[end]] > above[i]) end++;
-    if (end > at) cls.push_back({at, end, nt[i], false});
-    at = end;
   }
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     (void)cudaGetLastError();
-    return cls;
+    sms = 1;
   }
-  // FP64 with more tubes than SMs: the double-precision pipes are full, and a sweep that repeats no
-  // cell counts for more than one without barriers (1216 tubes of up to 256 cells: 3.99 ms against
-  // 4.54 by segments; 152 tubes, one per SM: segments 1.57 ms, chunks 1.80).  64-thread blocks only
-  // where the queue has more tubes than blocks to level them with (600 tubes at once: 3.18 ms, 2.76 with
-  // 128 threads).
-  if (!f32 && b->ntubes > sms) {
-    for (TubeClass &c : cls) {
-      c.chunks = true;
-      if (c.nt == 64 && c.last - c.first <= 4 * sms) c.nt = 128;
-    }
-    return cls;
+  auto longer = [&](int n) {  // tubes of more than n cells
+    int i = 0;
+    while (i < b->ntubes && b->len[b->order[i]] > n) i++;
+    return i;
+  };
+  const bool f32 = b->prec == MSH_FP32;
+  const int tiny = b->ntubes - longer(62) > 12 * sms ? 62 : 30;
+  int cut[2] = {longer(f32 ? 1024 : 126), longer(f32 ? 512 : tiny)}, nt[3] = {f32 ? 512 : 256, f32 ? 256 : 128, f32 ? 128 : 64};
+  if (!f32) {  // classes of few tubes join the next longer one
+    if (b->ntubes - cut[1] <= 2 * sms) cut[1] = b->ntubes;
+    if (cut[1] > cut[0] && cut[1] - cut[0] <= (b->len[b->order[cut[0]]] <= 62 ? sms : 2 * sms)) cut[0] = cut[1];
   }
-  long long room = (long long)sms * (f32 ? 16 : 8);  // warps that run at once
+  const int end[4] = {0, cut[0], cut[1], b->ntubes};
+  for (int i = 0; i < 3; i++)
+    if (end[i + 1] > end[i]) cls.push_back({end[i], end[i + 1], nt[i]});
+  if (!f32) return cls;
+  long long room = (long long)sms * 16;  // warps that run at once
   for (const TubeClass &c : cls) room -= (long long)(c.last - c.first) * (c.nt / 32);
   for (TubeClass &c : cls)
     while (c.nt < nt[0] && c.nt / 32 * kTubeSeg < b->len[b->order[c.first]] &&
@@ -505,7 +507,7 @@ std::vector<TubeClass> tube_classes(const msh_batch *b, int threads) {
 template <typename T> cudaError_t launch_class(msh_batch *b, const TubeClass &c, int i, int64_t max_steps, cudaStream_t s) {
   TubeArgs<T> a{(T *)b->U, b->d_off, b->d_len, b->d_tend, b->d_order, b->d_queue + i, c.first, c.last, b->d_steps, b->d_t,
                 b->d_status, b->d_fallback, b->total, b->len[b->order[c.first]], b->cfl, max_steps};
-  return launch_tubes<T>(a, c.nt, c.chunks, s);
+  return launch_tubes<T>(a, c.nt, s);
 }
 
 msh_status run_once(msh_batch *b, int threads, int64_t max_steps) {
@@ -644,8 +646,9 @@ msh_status msh_batch_run(msh_batch *b, int32_t threads, int64_t max_steps) {
   if (threads != 0 && threads != 128 && threads != 256 && threads != 512)
     return bfail(MSH_E_INVALID_ARG, "threads must be 0, 128, 256 or 512");
   if (max_steps < 1) return bfail(MSH_E_INVALID_ARG, "max_steps must be >= 1");
-  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, 0, false) : tube_smem<double>(b->cap, 0, false);
-  if (smem > 227 * 1024) return bfail(MSH_E_INVALID_ARG, "tubes too long for shared memory (%zu B)", smem);
+  const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, threads) : tube_smem<double>(b->cap, threads);
+  if (threads > 0 && smem > 227 * 1024)
+    return bfail(MSH_E_INVALID_ARG, "tubes too long for %d threads (%zu B shared)", threads, smem);
   // one persistent launch per class of lengths, captured in a CUDA graph with the queue reset
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;

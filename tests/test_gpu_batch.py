@@ -255,3 +255,33 @@ def test_fp64_batch_larger_than_the_chip(msh, oracle):
         assert rc == 0 and steps[k] == so
         assert_fp64(b.tube(U, k), Uo, what=f"tube {k} (len {tubes.length[k]})")
     b.close()
+
+
+def test_fp64_sweep_form_edges(msh, oracle):
+    # lengths at which an FP64 tube changes between segments and chunks, in a batch whose medium
+    # tubes fill a class of their own: against the oracle, and the same bits at every block size
+    edges = [119, 120, 121, 126, 127, 239, 240, 241, 254, 255, 361, 382, 383, 480, 481, 510, 511, 842, 894, 895]
+    tubes = _random_tubes(edges + [100] * 310 + [20] * 310, seed=49)
+    tubes.t_end = 0.02
+    b = msh.Batch(tubes.length, tubes.WL, tubes.WR, tubes.t_end, tubes.cfl, msh.FP64)
+    b.run()
+    U = b.get_state()
+    steps, _, _ = b.info()
+    for k in list(range(len(edges))) + [len(edges), len(tubes.length) - 1]:
+        Uo, so, _, rc = _oracle_tube(oracle, tubes, k)
+        assert rc == 0 and steps[k] == so
+        assert_fp64(b.tube(U, k), Uo, what=f"tube {k} (len {tubes.length[k]})")
+    for threads in (128, 256, 512):
+        b.reset()
+        b.run(threads=threads)
+        assert np.array_equal(U, b.get_state())
+    b.close()
+
+
+def test_fp64_tubes_too_long_for_512_threads_are_refused(msh):
+    tubes = _random_tubes([1000], seed=50)
+    b = msh.Batch(tubes.length, tubes.WL, tubes.WR, tubes.t_end, tubes.cfl, msh.FP64)
+    with pytest.raises(msh.MshError) as ei:
+        b.run(threads=512)
+    assert ei.value.status == msh.MSH_E_INVALID_ARG and "512 threads" in str(ei.value)
+    b.close()
