@@ -106,7 +106,10 @@ template <typename T> struct StagedArgs {
   int64_t seg_step = 0;         // step number of seg[0] (fallback tags)
   int32_t *had = nullptr;       // had[i]: whether step i tagged cells (may be null)
 };
-constexpr int kStagedMaxBlocks = 2048;  // blocks of a staged launch at most (partials, counts)
+constexpr int kScanBlocks = 608;  // 4 x 152 SMs
+// Blocks of a staged launch at most (the launcher keeps to it): its partials and counts per block have
+// room for them, and every grid holds at least kScanBlocks partials.
+constexpr int kStagedMaxBlocks = kScanBlocks;
 
 constexpr int kTile1D = 128;   // threads per block of the 1D step kernel
 constexpr int kTileX = 30;     // interior cells per warp row of the 3D kernel
@@ -177,7 +180,6 @@ template <typename T> cudaError_t launch_convert(T *U, size_t N, int to_primitiv
 template <typename T> cudaError_t launch_gravity_field(const double *phi, T *acc, int ndim, int nx, int ny, int nz,
                                                        const double *dx, cudaStream_t s);
 
-constexpr int kScanBlocks = 608;  // 4 x 152 SMs
 // States in flight in an ensemble run: one uploading, one computing, one downloading and
 // one spare, so that no stage waits for a slot while the other two are busy.
 constexpr int kEnsembleSlots = 4;

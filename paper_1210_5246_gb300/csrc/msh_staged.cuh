@@ -705,7 +705,8 @@ template <int NDIM, typename T> int staged_blocks(const StepArgs<T> &s, int per_
     const long long np = N / (d == 0 ? s.nx : d == 1 ? s.ny : s.nz);
     if (s.bc[2 * d] != BC_PERIODIC) groups += (2 * np + 31) / 32;
   }
-  return (int)std::max<long long>(1, std::min<long long>((long long)device_sms() * per_sm, (groups + 3) / 4));
+  const long long most = std::min<long long>((long long)device_sms() * per_sm, kStagedMaxBlocks);
+  return (int)std::max<long long>(1, std::min<long long>(most, (groups + 3) / 4));
 }
 
 template <typename T, int NDIM, int SCH> cudaError_t launch_staged_nd(const StagedArgs<T> &a, cudaStream_t s, int *nblk) {
