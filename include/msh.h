@@ -193,8 +193,9 @@ msh_status msh_get_dt_history(msh_grid *g, double *dts, int64_t capacity, int64_
  * estimate of the step's time on the grid's size, precision and CTU setting.  FP64 grids whose
  * staging buffers (2 + 2 ndim states) stay below 2 GiB, and small FP32 grids, take their steps
  * by the staged kernel instead (the same results bit for bit; the buffers are allocated at
- * the first step, and where they do not fit the streaming kernels go on); msh_set_tiling
- * selects the streaming kernels.  msh_autotune times the candidates (the current shape; 3D:
+ * the first step, and where they do not fit the streaming kernels go on; a call on the grid
+ * that runs out of device memory is tried once more without them); msh_set_tiling selects
+ * the streaming kernels.  msh_autotune times the candidates (the current shape; 3D:
  * rows 4/8/16 with the balanced tiling and with chunks cutting z into 1..8 near-equal windows;
  * 2D: rows 4/8/16 with zchunk 8..64; the staged step where the grid's size allows it) on this
  * grid's current state (without changing it or the tape) and keeps the fastest; the chosen

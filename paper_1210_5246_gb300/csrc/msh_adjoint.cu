@@ -779,9 +779,10 @@ extern "C" msh_status msh_adjoint_run(msh_grid *g, const void *U0, int64_t nstep
   if (g->ctu && g->ndim > 1)
     return afail(MSH_E_STATE, "the adjoint covers the step without transverse (CTU) terms only");
   if (g->sg_G > 0.0) return afail(MSH_E_STATE, "the adjoint covers external potentials only");
-  if (g->prec == MSH_FP32)
-    return adjoint_impl<float>(g, U0, nsteps, dt_sched, K, dL_dUN, dL_dU0, where, kind);
-  return adjoint_impl<double>(g, U0, nsteps, dt_sched, K, dL_dUN, dL_dU0, where, kind);
+  return with_room(g, [&] {
+    return g->prec == MSH_FP32 ? adjoint_impl<float>(g, U0, nsteps, dt_sched, K, dL_dUN, dL_dU0, where, kind)
+                               : adjoint_impl<double>(g, U0, nsteps, dt_sched, K, dL_dUN, dL_dU0, where, kind);
+  });
 }
 
 extern "C" msh_status msh_adjoint_tape(msh_grid *g, const void *dL_dUN, void *dL_dU0, int32_t where, int32_t kind) {
@@ -795,6 +796,8 @@ extern "C" msh_status msh_adjoint_tape(msh_grid *g, const void *dL_dUN, void *dL
   if (nsteps < 0 || nsteps > g->tape_len)
     return afail(MSH_E_STATE, "the run took %lld steps since msh_set_tape, the tape holds %lld", (long long)nsteps,
                  (long long)g->tape_len);
-  if (g->prec == MSH_FP32) return adjoint_tape_impl<float>(g, dL_dUN, dL_dU0, where, kind);
-  return adjoint_tape_impl<double>(g, dL_dUN, dL_dU0, where, kind);
+  return with_room(g, [&] {
+    return g->prec == MSH_FP32 ? adjoint_tape_impl<float>(g, dL_dUN, dL_dU0, where, kind)
+                               : adjoint_tape_impl<double>(g, dL_dUN, dL_dU0, where, kind);
+  });
 }

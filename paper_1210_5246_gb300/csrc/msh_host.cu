@@ -231,6 +231,15 @@ bool msh::use_staged(msh_grid *g) {
   return true;
 }
 
+bool msh::release_staged(msh_grid *g) {
+  if (!g->stg_mem || g->phase_level >= 0) return false;
+  cudaStreamSynchronize(g->stream);
+  drop_graph(g);  // its steps may be staged ones
+  cudaFree(g->stg_mem);
+  g->stg_mem = nullptr;
+  return true;
+}
+
 namespace {
 
 template <typename T> StagedArgs<T> make_staged(msh_grid *g, const StepArgs<T> &s, int max_iter) {
@@ -820,7 +829,7 @@ msh_status msh_run_ensemble(msh_grid *g, int64_t count, const void *const *in, v
   if (count == 0) return MSH_OK;
   msh_status st = stop_tape(g);
   if (st) return st;
-  st = ensure_ensemble(g, count);
+  st = with_room(g, [&] { return ensure_ensemble(g, count); });
   if (st) return st;
   st = ensure_partials(g, std::max(kScanBlocks, blocks_for(g, g->rows, g->zchunk)));
   if (st) return st;
@@ -923,8 +932,12 @@ msh_status msh_set_potential(msh_grid *g, const double *phi, int32_t where) {
   if (where != MSH_HOST && where != MSH_DEVICE) return fail(MSH_E_INVALID_ARG, "bad where");
   size_t cnt = 1;
   for (int d = 0; d < 3; d++) cnt *= (size_t)(g->n[d] + (d < g->ndim ? 2 : 0));
-  if (!g->phi) CUDA_TRY(cudaMalloc(&g->phi, cnt * sizeof(double)));
-  if (!g->acc) CUDA_TRY(cudaMalloc(&g->acc, 3 * g->N * g->esize));
+  const msh_status st = with_room(g, [&]() -> msh_status {
+    if (!g->phi) CUDA_TRY(cudaMalloc(&g->phi, cnt * sizeof(double)));
+    if (!g->acc) CUDA_TRY(cudaMalloc(&g->acc, 3 * g->N * g->esize));
+    return MSH_OK;
+  });
+  if (st) return st;
   CUDA_TRY(cudaMemcpyAsync(g->phi, phi, cnt * sizeof(double),
                            where == MSH_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, g->stream));
   cudaError_t e = g->prec == MSH_FP32
@@ -948,7 +961,11 @@ msh_status msh_set_scheme(msh_grid *g, int32_t scheme) {
   if (scheme == MSH_SCHEME_KT && g->ctu)
     return fail(MSH_E_STATE, "the transverse (CTU) terms belong to the characteristic schemes: switch CTU off first");
   CUDA_TRY(cudaStreamSynchronize(g->stream));
-  if (scheme == MSH_SCHEME_KT && !g->U1) CUDA_TRY(cudaMalloc(&g->U1, g->N * 10 * g->esize));
+  const msh_status st = with_room(g, [&]() -> msh_status {
+    if (scheme == MSH_SCHEME_KT && !g->U1) CUDA_TRY(cudaMalloc(&g->U1, g->N * 10 * g->esize));
+    return MSH_OK;
+  });
+  if (st) return st;
   if (scheme != g->scheme) drop_graph(g);
   g->scheme = scheme;
   return MSH_OK;
@@ -993,7 +1010,7 @@ msh_status msh_set_self_gravity(msh_grid *g, double G) {
     free_self_gravity(g);
     return MSH_OK;
   }
-  msh_status st = setup_self_gravity(g, G);
+  msh_status st = with_room(g, [&] { return setup_self_gravity(g, G); });
   if (st) return st;
   g->hctrl->sg_hist = 0;
   CUDA_TRY(cudaMemsetAsync(&g->ctrl->sg_hist, 0, sizeof(int32_t), g->stream));
@@ -1129,7 +1146,11 @@ msh_status msh_set_recording(msh_grid *g, int64_t capacity) {
   g->hist = nullptr;
   g->hist_cap = 0;
   if (capacity > 0) {
-    CUDA_TRY(cudaMalloc(&g->hist, sizeof(double) * (size_t)capacity));
+    const msh_status st = with_room(g, [&]() -> msh_status {
+      CUDA_TRY(cudaMalloc(&g->hist, sizeof(double) * (size_t)capacity));
+      return MSH_OK;
+    });
+    if (st) return st;
     g->hist_cap = capacity;
   }
   g->hctrl->hist = g->hist;
@@ -1161,10 +1182,14 @@ msh_status msh_set_tape(msh_grid *g, int32_t K, int64_t max_steps) {
   const int64_t nck = (max_steps + K - 1) / K;
   const int64_t have_ck = g->tape_K > 0 ? (g->tape_len + g->tape_K - 1) / g->tape_K : 0;
   if (nck > have_ck || max_steps > g->tape_len) {
-    free_tape(g);
-    CUDA_TRY(cudaMalloc(&g->tape, (size_t)nck * g->N * 10 * g->esize));
-    CUDA_TRY(cudaMalloc(&g->tape_dt, sizeof(double) * (size_t)max_steps));
-    CUDA_TRY(cudaMalloc(&g->tape_had, sizeof(int32_t) * (size_t)max_steps));
+    st = with_room(g, [&]() -> msh_status {
+      free_tape(g);
+      CUDA_TRY(cudaMalloc(&g->tape, (size_t)nck * g->N * 10 * g->esize));
+      CUDA_TRY(cudaMalloc(&g->tape_dt, sizeof(double) * (size_t)max_steps));
+      CUDA_TRY(cudaMalloc(&g->tape_had, sizeof(int32_t) * (size_t)max_steps));
+      return MSH_OK;
+    });
+    if (st) return st;
   }
   g->tape_K = K;
   g->tape_len = max_steps;
@@ -1470,7 +1495,11 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   const size_t bytes = g->N * 10 * g->esize;
   const int cur = cur_buf(g);
   void *save = nullptr;
-  CUDA_TRY(cudaMalloc(&save, bytes));
+  msh_status st = with_room(g, [&]() -> msh_status {
+    CUDA_TRY(cudaMalloc(&save, bytes));
+    return MSH_OK;
+  });
+  if (st) return st;
   Ctrl saved_ctrl = *g->hctrl;
   // the trial steps must not write the adjoint tape
   Ctrl trial_ctrl = saved_ctrl;
@@ -1480,7 +1509,6 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   const bool tape_was_valid = g->tape_valid;
   g->tape_valid = false;
   *g->hctrl = trial_ctrl;
-  msh_status st = MSH_OK;
   // the trial steps overwrite the stored self-gravity acceleration: keep a copy
   void *sg_save = nullptr;
   if (g->sg_G > 0.0 && cudaMalloc(&sg_save, 3 * g->N * g->esize) == cudaSuccess)

@@ -250,7 +250,7 @@ struct msh_grid {
   int rows = 8, zchunk = 32;
   bool tiling_set = false;  // msh_set_tiling chose the streaming kernels' shape: they step the grid
   // the staged step (msh_staged.cuh): its buffers in one allocation, made at the first step
-  // that uses it; stg_off: the allocation failed, the streaming kernels step the grid
+  // that uses it; stg_off: there is no room for it, the streaming kernels step the grid
   void *stg_mem = nullptr;
   bool stg_off = false;
   double tile_us = 0.0;  // estimated step time of the streaming kernels' default shape
@@ -275,6 +275,24 @@ struct msh_grid {
 namespace msh {
 // Whether the staged step takes this grid's steps (allocates its buffers at the first use).
 bool use_staged(msh_grid *g);
+// Frees the staging buffers; false if there are none or a phased step still needs them.
+bool release_staged(msh_grid *g);
+// call(), and if it runs out of device memory once more without the grid's staging buffers: they are a
+// cache of speed, and a call that fits beside the streaming step succeeds.  The grid streams from then
+// on; if the call fails all the same, the next staged step allocates its buffers again.
+template <typename F> msh_status with_room(msh_grid *g, F &&call) {
+  msh_status st = call();
+  if (st != MSH_E_NOMEM) return st;
+  (void)cudaGetLastError();
+  if (!release_staged(g)) return st;
+  g->stg_off = true;
+  st = call();
+  if (st == MSH_OK) clear_error();
+  if (st != MSH_E_NOMEM) return st;
+  (void)cudaGetLastError();
+  g->stg_off = false;
+  return st;
+}
 // The `steps` states after seg[0], written to seg[1 .. steps] ([NV][N] each, device), with the
 // given time steps (device) by one staged launch; tags carry the step numbers from step0 on.
 template <typename T>
