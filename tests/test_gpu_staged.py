@@ -195,3 +195,40 @@ def test_noalloc_thin_box_fits_the_fixed_scratch(msh):
     e = msh.msh_step_noalloc(n, (0.0,) * 3, (1.0, 1.5, 0.5), bc, msh.FP32, 0.3, u0, u1)
     assert abs(e - dt) <= 1e-12 * dt
     assert np.array_equal(u1.cpu().numpy().reshape(U1.shape), U1)
+
+
+def _after_step_ms(g, reps=6):
+    """Time that a profiled step takes after its step kernel: fallback passes and finalize of a
+    streaming step (five launches), nothing but two events of a staged one."""
+    ms = []
+    for _ in range(reps):
+        g.set_profiling(True)
+        g.run(max_steps=1)
+        ms.append(g.profile()[1])
+        g.set_profiling(False)
+    return min(ms)
+
+
+@pytest.mark.parametrize("prec,n,staged", [("FP32", 3000, True), ("FP32", 600000, True), ("FP32", 1500000, False),
+                                           ("FP64", 1500000, True)])
+def test_large_1d_grids(msh, n, prec, staged):
+    """1D grids around the size at which the staged step's buffers leave L2: the default takes the
+    staged step below it only (FP32), and gives the bits of the streaming step."""
+    rng = np.random.default_rng(6)
+    W = np.zeros((10, 1, 1, n))
+    W[0] = rng.uniform(0.8, 1.2, n)
+    W[1:4] = rng.uniform(-0.2, 0.2, (3, 1, 1, n))
+    W[4] = W[7] = W[9] = rng.uniform(0.9, 1.1, n)
+    out, after = [], []
+    for tiling in (False, True):
+        g = msh.Grid((n,), (0.0,), (1.0,), ((1, 1),), 0.4, getattr(msh, prec))
+        if tiling:
+            g.set_tiling(8, 1)
+        g.set_state(W.astype(g.dtype), msh.PRIMITIVE)
+        g.run(max_steps=3)
+        out.append((g.time(), g.get_state()))
+        after.append(_after_step_ms(g))
+        g.close()
+    assert (after[0] < 0.5 * after[1]) == staged
+    assert out[0][0] == out[1][0]
+    np.testing.assert_array_equal(out[0][1], out[1][1])
