@@ -199,13 +199,17 @@ struct StagedLayout {
   }
 };
 
+// Whether the staged step can take this grid's steps: its size, precision and scheme allow it.
+bool staged_fits(const msh_grid *g) {
+  if (g->ctu || g->stg_off || StagedLayout(g).bytes > kStagedMaxBytes) return false;
+  return g->prec == MSH_FP64 || g->N <= kStagedMaxCells32[g->ndim - 1];
+}
+
+// Whether it does: as chosen (msh_set_tiling, msh_autotune), else where it is the faster form.
 bool staged_wanted(const msh_grid *g) {
-  if (g->ctu || g->tiling_set || g->stg_off) return false;
-  if (StagedLayout(g).bytes > kStagedMaxBytes) return false;
-  if (g->prec == MSH_FP64) return true;
+  if (g->form == msh_grid::kStream || !staged_fits(g)) return false;
   const int d = g->ndim - 1;
-  if (g->N > kStagedMaxCells32[d]) return false;
-  return d == 0 || kStagedBase[d] + kStagedPerCell[d] * (double)g->N < kStreamLaunches + g->tile_us;
+  return g->form == msh_grid::kStaged || g->prec == MSH_FP64 || d == 0 || kStagedBase[d] + kStagedPerCell[d] * (double)g->N < kStreamLaunches + g->tile_us;
 }
 
 }  // namespace
@@ -1466,10 +1470,11 @@ msh_status msh_set_tiling(msh_grid *g, int32_t rows, int32_t zchunk) {
   if (zchunk > stream_len) zchunk = (int)stream_len;
   msh_status st = ensure_partials(g, blocks_for(g, rows, zchunk));
   if (st) return st;
-  if (rows != g->rows || zchunk != g->zchunk || !g->tiling_set) drop_graph(g);
+  if (rows != g->rows || zchunk != g->zchunk || g->form != msh_grid::kStream) drop_graph(g);
   g->rows = rows;
   g->zchunk = zchunk;
   g->tiling_set = true;
+  g->form = msh_grid::kStream;
   return MSH_OK;
 }
 
@@ -1481,8 +1486,10 @@ msh_status msh_get_tiling(msh_grid *g, int32_t *rows, int32_t *zchunk) {
   return MSH_OK;
 }
 
-// Time each tile shape on copies of the current state (the state, time and step
-// counter are restored afterwards) and keep the fastest.
+// Time each tile shape, and the staged step, on copies of the current state (the state, time and
+// step counter are restored afterwards) and keep the fastest.  Both forms take the same number of
+// steps as a run launches them: streaming steps without their fallback passes, unless one tags cells
+// (then every shape is timed again with them), staged steps in one launch.
 msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   msh::NvtxRange nvtx_range("msh_autotune");
   begin();
@@ -1543,12 +1550,21 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   if (std::find(cands.begin(), cands.end(), std::make_pair(g->rows, g->zchunk)) == cands.end())
     cands.push_back({g->rows, g->zchunk});
   // the staged step is a candidate of its own (0, 0) where the grid's size allows it
-  g->tiling_set = false;
+  const int rows0 = g->rows, zchunk0 = g->zchunk;
+  const bool tiling_set0 = g->tiling_set;
+  const msh_grid::Form form0 = g->form;
+  g->form = msh_grid::kStaged;
   if (use_staged(g)) cands.push_back({0, 0});
   float best = 1e30f, best_tile = 1e30f;
   std::pair<int, int> best_c = {g->rows, g->zchunk};
-  bool best_staged = false;
-  const int reps = 3;
+  bool best_staged = false, lean = !g->tags_seen;
+  const int reps = g->N <= size_t(1) << 20 ? kGraphSteps : 3;
+  auto take = [&](int n) -> msh_status {
+    if (!lean || !lean_steps(g)) return launch_steps(g, n);
+    msh_status s = MSH_OK;
+    for (int i = 0; i < n && s == MSH_OK; i++) s = launch_lean_step(g);
+    return s;
+  };
   if (st == MSH_OK && (cudaMemcpyAsync(save, g->U[cur], bytes, cudaMemcpyDeviceToDevice, g->stream) != cudaSuccess ||
                        cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) {
     st = fail(MSH_E_CUDA, "autotune setup: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1557,23 +1573,25 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   g->profiling = false;
   for (size_t i = 0; st == MSH_OK && i < cands.size(); i++) {
     const bool staged = cands[i].first == 0;
-    if (staged) g->tiling_set = false;
+    if (staged) g->form = msh_grid::kStaged;
     else st = msh_set_tiling(g, cands[i].first, cands[i].second);
     if (st) break;
     cudaError_t e = launch_run_start(g->ctrl, INFINITY, 1 << 30, INFINITY, g->stream);
-    st = launch_steps(g, 1);
+    st = take(1);
     if (st == MSH_OK) e = cudaEventRecord(e0, g->stream);
-    if (st == MSH_OK) st = launch_steps(g, reps);
+    if (st == MSH_OK) st = take(reps);
     if (st == MSH_OK) e = cudaEventRecord(e1, g->stream);
     if (st == MSH_OK && e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (st == MSH_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (st == MSH_OK && e != cudaSuccess) st = fail(MSH_E_CUDA, "autotune timing: %s", cudaGetErrorString(e));
-    if (st == MSH_OK && ms < best) {
+    if (st == MSH_OK) st = read_ctrl(g);
+    const bool tagged = st == MSH_OK && g->hctrl->status == kStatusPending;
+    if (st == MSH_OK && !tagged && ms < best) {
       best = ms;
       best_staged = staged;
     }
-    if (st == MSH_OK && !staged && ms < best_tile) {
+    if (st == MSH_OK && !tagged && !staged && ms < best_tile) {
       best_tile = ms;
       best_c = cands[i];
     }
@@ -1583,6 +1601,11 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
       e = cudaMemcpyAsync(g->ctrl, g->hctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, g->stream);
       if (e == cudaSuccess) e = cudaMemcpyAsync(g->U[cur], save, bytes, cudaMemcpyDeviceToDevice, g->stream);
       if (e != cudaSuccess) st = fail(MSH_E_CUDA, "autotune restore: %s", cudaGetErrorString(e));
+    }
+    if (st == MSH_OK && tagged) {  // start over with the fallback passes
+      lean = false;
+      best = best_tile = 1e30f;
+      i = (size_t)-1;
     }
   }
   g->profiling = prof;
@@ -1600,10 +1623,15 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
   if (e1) cudaEventDestroy(e1);
   cudaStreamSynchronize(g->stream);
   cudaFree(save);
-  if (st) return st;
-  st = msh_set_tiling(g, best_c.first, best_c.second);
-  if (st) return st;
-  if (best_staged) g->tiling_set = false;  // the staged step goes on; the streaming shape is the best of its kind
+  if (st == MSH_OK) st = msh_set_tiling(g, best_c.first, best_c.second);
+  if (st) {
+    g->rows = rows0;
+    g->zchunk = zchunk0;
+    g->tiling_set = tiling_set0;
+    g->form = form0;
+    return st;
+  }
+  if (best_staged) g->form = msh_grid::kStaged;  // the streaming shape is the best of its kind
   if (rows_out) *rows_out = g->rows;
   if (zchunk_out) *zchunk_out = g->zchunk;
   return MSH_OK;

@@ -248,7 +248,10 @@ struct msh_grid {
   int32_t test_fault = 0;  // msh_set_test_fault: applied to the next eager step launch
   unsigned long long *tag_count = nullptr;  // device counter of msh_count_tags
   int rows = 8, zchunk = 32;
-  bool tiling_set = false;  // msh_set_tiling chose the streaming kernels' shape: they step the grid
+  bool tiling_set = false;  // msh_set_tiling or msh_autotune chose the streaming kernels' shape
+  // the form of the step: by the size (kAuto), or the one that msh_set_tiling (kStream) or a
+  // measurement (msh_autotune) chose
+  enum Form { kAuto, kStream, kStaged } form = kAuto;
   // the staged step (msh_staged.cuh): its buffers in one allocation, made at the first step
   // that uses it; stg_off: there is no room for it, the streaming kernels step the grid
   void *stg_mem = nullptr;
