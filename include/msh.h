@@ -411,7 +411,8 @@ msh_status msh_count_tags(msh_grid *g, int64_t start, int64_t count, int32_t lev
  * second-order update is not realizable trigger the same a-posteriori first-order
  * fallback as msh_step (the step is recomputed from U^n with first-order faces there);
  * a tube still non-realizable after it stops with MSH_E_REALIZABILITY.  threads is
- * the block size (0: chosen by the tubes' lengths).
+ * the block size (0: chosen by the tubes' number and lengths; the first run of a batch with
+ * threads = 0 starts from the initial state, whatever ran before it).
  * max_steps caps the steps of each tube (MSH_E_TIMEOUT if a tube hits it before t_end).
  */
 msh_status msh_batch_init(msh_batch **out, int32_t ntubes, const int32_t *len, const double *WL,

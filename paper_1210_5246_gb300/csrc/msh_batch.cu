@@ -414,6 +414,8 @@ struct msh_batch {
   std::vector<int64_t> off;
   std::vector<double> t_end;
   std::vector<unsigned char> init;  // initial conserved state, host copy for reset
+  bool advanced = false;            // the state is no longer the initial one
+  bool sized = false;               // a run chose its block sizes itself (threads = 0)
   void *U = nullptr;
   int64_t *d_off = nullptr;
   int32_t *d_len = nullptr, *d_order = nullptr, *d_queue = nullptr, *d_status = nullptr;
@@ -636,6 +638,7 @@ msh_status msh_batch_init(msh_batch **out, int32_t ntubes, const int32_t *len, c
 msh_status msh_batch_reset(msh_batch *b) {
   clear_error();
   if (!b) return bfail(MSH_E_INVALID_ARG, "null batch");
+  b->advanced = false;
   return upload_initial(b);
 }
 
@@ -649,6 +652,13 @@ msh_status msh_batch_run(msh_batch *b, int32_t threads, int64_t max_steps) {
   const size_t smem = b->prec == MSH_FP32 ? tube_smem<float>(b->cap, threads) : tube_smem<double>(b->cap, threads);
   if (threads > 0 && smem > 227 * 1024)
     return bfail(MSH_E_INVALID_ARG, "tubes too long for %d threads (%zu B shared)", threads, smem);
+  // the first run with threads = 0 starts from the initial state, whatever ran before it
+  if (threads == 0 && !b->sized && b->advanced) {
+    const msh_status st0 = upload_initial(b);
+    if (st0) return st0;
+  }
+  b->sized = b->sized || threads == 0;
+  b->advanced = true;
   // one persistent launch per class of lengths, captured in a CUDA graph with the queue reset
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -676,6 +686,7 @@ msh_status msh_batch_run_per_tube(msh_batch *b, const int32_t *tubes, int32_t co
   if (!b) return bfail(MSH_E_INVALID_ARG, "null batch");
   if (tubes && count < 0) return bfail(MSH_E_INVALID_ARG, "bad count");
   const int m = tubes ? count : b->ntubes;
+  b->advanced = true;
   if ((int)b->grids.size() < b->ntubes) b->grids.resize(b->ntubes, nullptr);
   for (int i = 0; i < m; i++) {
     const int k = tubes ? tubes[i] : i;

@@ -285,3 +285,17 @@ def test_fp64_tubes_too_long_for_512_threads_are_refused(msh):
         b.run(threads=512)
     assert ei.value.status == msh.MSH_E_INVALID_ARG and "512 threads" in str(ei.value)
     b.close()
+
+
+def test_first_run_with_chosen_block_sizes_starts_over(msh):
+    """The first run with threads = 0 starts from the initial state, also after runs with an
+    explicit block size; later runs go on from where the tubes are."""
+    tubes = _random_tubes([60, 200, 333], seed=51)
+    b = msh.Batch(tubes.length, tubes.WL, tubes.WR, tubes.t_end, tubes.cfl, msh.FP64)
+    b.run(threads=256)
+    U = b.get_state()
+    b.run()
+    np.testing.assert_array_equal(b.get_state(), U)
+    b.run()
+    assert not np.array_equal(b.get_state(), U)
+    b.close()
