@@ -1632,6 +1632,7 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows_out, int32_t *zchunk_out) {
     return st;
   }
   if (best_staged) g->form = msh_grid::kStaged;  // the streaming shape is the best of its kind
+  else (void)release_staged(g);
   if (rows_out) *rows_out = g->rows;
   if (zchunk_out) *zchunk_out = g->zchunk;
   return MSH_OK;
