@@ -86,8 +86,8 @@ __device__ __forceinline__ double warp_sum10(double (&v)[NV], int &comp) {
 // The same for ten FP32 values per lane, in pairs of floats (an error-free sum and its running
 // error: relative error below 2^-45 over a warp, where one thread's FP32 sum carries up to
 // 2^-19): 107 FP32 operations instead of 12 FP64 additions at 77 pipe cycles and ten conversions,
-// 1.8 us at the end of a block of 16 warps.  A sum that overflows FP32 within the warp is formed
-// again in FP64.
+// 1.8 us at the end of a block of 16 warps.  Values so large that their sum could overflow FP32 within
+// the warp are added in FP64.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
   s = a + b;
   const float bb = s - a;
@@ -111,6 +111,11 @@ __device__ __forceinline__ double warp_sum10(float (&v)[NV], int &comp) {
   const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
   const int in3 = (b2 ? 2 : 0) + (b1 ? 1 : 0), in5 = (b3 ? 3 : 0) + in3;
   comp = (in3 < 3 && in5 < 5) ? (b4 ? 5 : 0) + in5 : -1;
+  float m = fabsf(v[0]);
+#pragma unroll
+  for (int k = 1; k < NV; k++) m = fmaxf(m, fabsf(v[k]));
+  if (__builtin_expect(__any_sync(FULL, m >= 0x1p122f), 0))
+    return warp_sum10_wide(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9]);
   float h[6], l[6];
 #pragma unroll
   for (int k = 0; k < 5; k++) {
@@ -138,9 +143,6 @@ __device__ __forceinline__ double warp_sum10(float (&v)[NV], int &comp) {
   pair_add(xh, xl, oh, ol);
   const float ph = __shfl_xor_sync(FULL, xh, 1), pl = __shfl_xor_sync(FULL, xl, 1);
   pair_add(xh, xl, ph, pl);
-  if (__builtin_expect(__any_sync(FULL, !(fabsf(xh) < INFINITY)), 0)) {  // inf, or NaN from its error term
-    return warp_sum10_wide(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9]);
-  }
   return widen(xh) + widen(xl);
 }
 
