@@ -210,7 +210,9 @@ msh_status msh_autotune(msh_grid *g, int32_t *rows, int32_t *zchunk);
  * graph and brackets every step-kernel launch with CUDA events on the grid's stream,
  * accumulating their elapsed times.  msh_get_profile returns the summed step-kernel time,
  * the summed time from each step kernel's end to its finalize kernel's end (both in
- * ms) and the number of timed launches since profiling was switched on.
+ * ms) and the number of timed launches since profiling was switched on.  On a grid that takes
+ * the staged step the timed launches are whole staged steps, one per launch (msh_run without
+ * profiling takes up to 64 per launch), and nothing follows them.
  */
 msh_status msh_set_profiling(msh_grid *g, int32_t on);
 msh_status msh_get_profile(msh_grid *g, double *step_kernel_ms, double *finalize_ms, int64_t *launches);

@@ -10,13 +10,14 @@
 // the second tube buffer, and the buffers swap roles, so W^n stays intact for the fallback
 // passes without a copy.  A step costs two block barriers; between them one thread plans the
 // time step.  Tubes go to the kernel in up to three classes by length, launched side by side:
-// long tubes need a whole SM's shared memory for their two buffers (16 warps, one block per
+// long FP32 tubes need a whole SM's shared memory for their two buffers (16 warps, one block per
 // SM), shorter ones two or four blocks per SM with 8 or 4 warps each, which hide each other's
-// time control and fill the SMs that the long tubes leave.
+// time control and fill the SMs that the long tubes leave.  FP64 tubes: see tube_classes, and
+// takes_chunks for their second form of the sweep.
 // Bound: instruction issue.  4096 tubes of 128 to 2048 cells to t = 0.1 (7.4e8 cell updates):
 // 27.9 ms with one tube per block of 256 threads, three barriers per chunk and every thread
 // planning the time step; 19.6 ms now (14.7 + 3.8 + 1.1 for the three classes one after another),
-// 0.58 instructions per scheduler and cycle.
+// 0.61 to 0.65 instructions per scheduler and cycle.
 // The step is the same as the grid kernels': MUSCL-Hancock on the characteristic
 // variables (Sec. 3.3), HLL flux, outflow boundaries by index clamping, CFL time step
 // dt = C dx / max(|u| + sqrt(3 P_xx/rho)) with the last step clipped to t_end.

@@ -377,7 +377,9 @@ static double balanced_cost(long long ncols, long long nz, long long units, doub
 //            5.2 rows.  512^2: 4 rows 26.8 us, 8 rows 28.0 us; 1024^2: 16 rows 61.6 us; 700^2: 10 rows
 //            43.8 us.
 //   FP64     the double-precision pipe is the bound: time goes with the warps per scheduler,
-//            a prologue costs about one row or plane.
+//            a prologue costs about one row or plane.  2D blocks of 16 warps are held to 128
+//            registers and spill (780 B), which that pipe hides: 4096^2 29.2 ms in chunks of 50 rows,
+//            8 warps in chunks of 16 (the fixed shape before) 29.4, 2500^2 11.0 and 11.4.
 Tiling default_tiling(int ndim, const int64_t n[3], int prec, bool ctu) {
   if (ndim == 1) return {8, 1, 0.0};
   const bool f32 = prec == MSH_FP32;
