@@ -63,11 +63,13 @@ constexpr int kStagedSteps = 64;  // steps of one staged launch at most
 // the staged step's buffers (2 + 2 ndim states) stay below this; larger grids stream
 constexpr size_t kStagedMaxBytes = size_t(2) << 30;
 // FP32 grids of up to this many cells (1D, 2D, 3D) may take the staged step (beyond, its buffers
-// leave L2).  1D: below the line it is the faster one at every size (10^3 cells 8.9 us per step, streaming
-// 10.5; 10^5 15.0 and 16.7; 7 10^5 54.3 and 55.9), beyond it the slower one (10^6 88 and 75.5; 1.2 10^7 1059
-// and 840).  2D and 3D: where its estimated time is the shorter one.  Fits to timed steps: staged 2D 13.0 us + 0.97e-4 us per cell (64^2 13, 256^2 20, 512^2 38), 3D 14.7 us + 1.9e-4 us per
-// cell (32^3 21, 64^3 64, 97x61x45 69); a streaming step adds 3 us to its kernel (256^2 19.5 us,
-// 512^2 28.8, 64^3 69).
+// leave L2).  1D: below the line it is the faster one at every size (10^3 cells 8.9 us per step,
+// streaming 10.5; 10^5 15.0 and 16.7; 7 10^5 54.3 and 55.9), beyond it the slower one (10^6 88 and
+// 75.5; 1.2 10^7 1059 and 840).  2D and 3D: where its estimated time is the shorter one.  Fits to
+// timed steps: staged 2D 13.0 us + 0.97e-4 us per cell (64^2 13, 256^2 20, 512^2 38), 3D 14.7 us +
+// 1.9e-4 us per cell (32^3 21, 64^3 64, 97x61x45 69); a streaming step adds 3 us to its kernel (256^2
+// 19.5 us, 512^2 28.8, 64^3 69; 512^2 25.7 and 64^3 62 since block ends are shorter, which the
+// estimates do not know: at 64^3, 65.7 us staged, autotune finds the streaming one).
 constexpr size_t kStagedMaxCells32[3] = {700000, 400000, 400000};
 constexpr double kStagedBase[3] = {0.0, 13.0, 14.7}, kStagedPerCell[3] = {0.0, 0.97e-4, 1.9e-4};
 constexpr double kStreamLaunches = 3.0;
